@@ -1102,4 +1102,273 @@ ACOPF_HD inline bool line_solve_predicted(const LineQP<double>& P, double x[4], 
   return true;
 }
 
+// ------------------------------------- exact FP64 line QP from a kept active set
+// On a fixed active set the KKT point is an affine function of the linear
+// term c, the only part of the subproblem that changes from one ADMM iteration
+// to the next: x = p0 - P c, mu = m0 - M c.  A thread that keeps its branch
+// through the sweep keeps this operator (P symmetric 4x4 with zero rows for
+// the bounds held, M and m0 for up to two active rows) and evaluates it, with
+// one step of iterative refinement, and the KKT check of
+// line_solve_predicted; the set is corrected and the operator built again
+// only when the check fails.  Most iterations change no set, and each then
+// takes about 120 FP64 instructions in short chains instead of the FP32
+// prediction, an FP64 Cholesky factorisation and triangular solves.
+//
+// Set: bits 0-3 bounds held, 4-7 at the upper bound, 8-11 rows active; bit 12
+// marks a set that holds an operator.  Operator: value e at op[e * stride]:
+//   0-9 P (packed)  10-13 p0  14-17 M of the first active row  18-21 of the
+//   second  22, 23 m0  24 max |q|  25-28 1 + |b_r| of the four rows
+constexpr int kLineOp = 29;
+constexpr unsigned kSetValid = 1u << 12;
+
+ACOPF_HD inline unsigned hi_of(double x) { return (unsigned)(bits_of(x) >> 32); }
+ACOPF_HD inline unsigned abs_hi(double x) { return hi_of(x) & 0x7fffffffu; }
+// v <= t for t >= 0, on the leading 32 bits of the patterns (both tolerances
+// here are free to 2^-20 of themselves; no FP64 comparison); v not a NaN
+ACOPF_HD inline bool le_tol(double v, unsigned t_hi) { return (int)hi_of(v) <= (int)t_hi; }
+
+// the two lowest active rows (-1: none)
+ACOPF_HD inline void set_rows(unsigned act, int& r0, int& r1) {
+  r0 = r1 = -1;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if ((act >> r) & 1u) {
+      if (r0 < 0) r0 = r;
+      else if (r1 < 0) r1 = r;
+    }
+}
+
+// normal and right-hand side of row r (n . x <= b): the line limits, then
+// x1 - x3 <= ahi and x3 - x1 <= -alo
+ACOPF_HD inline void row_normal(const LineQP<double>& P, int r, double n[4], double& b) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) n[i] = r == 0 ? P.R[0][i] : (r == 1 ? P.R[1][i] : 0.0);
+  b = r == 0 ? P.rb[0] : P.rb[1];
+  if (r == 2) { n[1] = 1.0; n[3] = -1.0; b = P.ahi; }
+  if (r == 3) { n[1] = -1.0; n[3] = 1.0; b = -P.alo; }
+}
+
+// The operator of a set; false when it has more than two active rows or its
+// system is singular.
+ACOPF_HD inline bool line_operator(const LineQP<double>& P, unsigned set, double* op, int stride) {
+  const unsigned fx = set & 15u, hs = (set >> 4) & 15u, act = (set >> 8) & 15u;
+  int r0, r1;
+  set_rows(act, r0, r1);
+  if ((act & (act - 1u)) & ((act & (act - 1u)) - 1u)) return false;  // three or four rows
+  Chol4<double> fac;
+  if (!chol4_factor(P.q, ~fx & 15u, fac)) return false;
+  // columns of Q_FF^-1 (zero on the bounds held)
+  double H[4][4], x0[4], rhs[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    double e[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) e[i] = (i == j && !((fx >> j) & 1u)) ? 1.0 : 0.0;
+    chol4_solve(fac, e, H[j]);
+  }
+  // the point for c = 0 with no rows: bounds held, -Q_FF^-1 Q_FB x_B
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    double v = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if ((fx >> j) & 1u) v -= P.q[pk(i, j)] * (((hs >> j) & 1u) ? P.hi[j] : P.lo[j]);
+    rhs[i] = ((fx >> i) & 1u) ? 0.0 : v;
+  }
+  chol4_solve(fac, rhs, x0);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if ((fx >> i) & 1u) x0[i] = ((hs >> i) & 1u) ? P.hi[i] : P.lo[i];
+  double M0[4] = {0.0, 0.0, 0.0, 0.0}, M1[4] = {0.0, 0.0, 0.0, 0.0}, c0 = 0.0, c1 = 0.0;
+  if (r0 >= 0) {
+    // W = Q_FF^-1 N', S = N W, M = S^-1 W', m0 = S^-1 (N x0 - b), P = Q_FF^-1 - W M, p0 = x0 - W m0
+    double n0[4], n1[4], W0[4], W1[4] = {0.0, 0.0, 0.0, 0.0}, b0, b1 = 0.0;
+    row_normal(P, r0, n0, b0);
+    row_normal(P, r1, n1, b1);
+    double t0 = -b0, t1 = -b1, s00 = 0.0, s01 = 0.0, s11 = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      W0[i] = H[0][i] * n0[0] + H[1][i] * n0[1] + H[2][i] * n0[2] + H[3][i] * n0[3];
+      t0 += n0[i] * x0[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s00 += n0[i] * W0[i];
+    if (!(s00 > 0.0)) return false;
+    if (r1 >= 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        W1[i] = H[0][i] * n1[0] + H[1][i] * n1[1] + H[2][i] * n1[2] + H[3][i] * n1[3];
+        t1 += n1[i] * x0[i];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        s01 += n0[i] * W1[i];
+        s11 += n1[i] * W1[i];
+      }
+      const double det = s00 * s11 - s01 * s01;
+      if (!(det > 0.0)) return false;
+      const double id = 1.0 / det;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        M0[i] = (s11 * W0[i] - s01 * W1[i]) * id;
+        M1[i] = (s00 * W1[i] - s01 * W0[i]) * id;
+      }
+      c0 = (s11 * t0 - s01 * t1) * id;
+      c1 = (s00 * t1 - s01 * t0) * id;
+    } else {
+      const double is = 1.0 / s00;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) M0[i] = W0[i] * is;
+      c0 = t0 * is;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (!((fx >> i) & 1u)) x0[i] -= W0[i] * c0 + W1[i] * c1;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) H[i][j] -= W0[i] * M0[j] + W1[i] * M1[j];
+    }
+  }
+  double qm = 0.0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int j = i; j < 4; ++j) {
+      op[pk(i, j) * stride] = 0.5 * (H[i][j] + H[j][i]);
+      qm = fmax(qm, fabs(P.q[pk(i, j)]));
+    }
+    op[(10 + i) * stride] = x0[i];
+    op[(14 + i) * stride] = M0[i];
+    op[(18 + i) * stride] = M1[i];
+  }
+  op[22 * stride] = c0;
+  op[23 * stride] = c1;
+  op[24 * stride] = qm;
+  op[25 * stride] = 1.0 + fabs(P.rb[0]);
+  op[26 * stride] = 1.0 + fabs(P.rb[1]);
+  op[27 * stride] = 1.0 + fabs(P.ahi);
+  op[28 * stride] = 1.0 + fabs(P.alo);
+  return true;
+}
+
+// Evaluates the operator of `set` at P.c.  Returns true when the point is the
+// KKT point (checks of line_solve_predicted, to 1e-11 of the scales): x inside
+// the box, u the row multipliers.  Otherwise `next` is the corrected set (equal
+// to `set` when there is nothing to correct: non-finite values).
+ACOPF_HD inline bool line_eval(const LineQP<double>& P, unsigned set, const double* op, int stride, double x[4],
+                               double u[4], unsigned& next) {
+  const unsigned fx = set & 15u, hs = (set >> 4) & 15u, act = (set >> 8) & 15u;
+  double H[10];
+#pragma unroll
+  for (int k = 0; k < 10; ++k) H[k] = op[k * stride];
+  double g[4], mu[4] = {0.0, 0.0, 0.0, 0.0};
+  symv4(H, P.c, g);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = op[(10 + i) * stride] - g[i];
+  // g = Q x + c + N' mu, then x -= P g (and mu -= M g): one refinement step
+  symv4(P.q, x, g);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) g[i] += P.c[i];
+  if (act) {
+    int r0, r1;
+    set_rows(act, r0, r1);
+    double a = op[22 * stride], b = op[23 * stride], Ma[4], Mb[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      Ma[i] = op[(14 + i) * stride];
+      Mb[i] = op[(18 + i) * stride];
+      a -= Ma[i] * P.c[i];
+      b -= Mb[i] * P.c[i];
+    }
+    double dg[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) mu[r] = r == r0 ? a : (r == r1 ? b : 0.0);
+    const double ma = mu[2] - mu[3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dg[i] = mu[0] * P.R[0][i] + mu[1] * P.R[1][i];
+    dg[1] += ma;
+    dg[3] -= ma;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      g[i] += dg[i];
+      a -= Ma[i] * g[i];
+      b -= Mb[i] * g[i];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) mu[r] = r == r0 ? a : (r == r1 ? b : 0.0);
+  }
+  {
+    double dx[4];
+    symv4(H, g, dx);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] -= dx[i];
+  }
+  // scales and tolerances from the leading halves of the patterns
+  unsigned xh = 0u, ch = 0u, gh = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const unsigned a = abs_hi(x[i]), b = abs_hi(P.c[i]), d = abs_hi(g[i]);
+    xh = a > xh ? a : xh;
+    ch = b > ch ? b : ch;
+    gh = d > gh ? d : gh;
+  }
+  bool ok = xh < 0x7ff00000u && ch < 0x7ff00000u && gh < 0x7ff00000u;
+  next = set;
+  if (!ok) return false;
+  const double xm = double_of((unsigned long long)xh << 32), cm = double_of((unsigned long long)ch << 32);
+  const double tx = 1e-11 * (xm + 1.0);
+  const double tol = 1e-11 * (cm + 1.0) + 1e-11 * op[24 * stride] * xm;
+  const unsigned th = hi_of(tol), txh = hi_of(tx);
+  // rows: v = n . x - b
+  const double dth = x[1] - x[3];
+  double v[4];
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+    v[r] = P.R[r][0] * x[0] + P.R[r][1] * x[1] + P.R[r][2] * x[2] + P.R[r][3] * x[3] - P.rb[r];
+  v[2] = dth - P.ahi;
+  v[3] = P.alo - dth;
+  unsigned nfx = fx, nhs = hs, nact = act;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const bool on = r < 2 ? P.on[r] : P.ang;
+    const bool feas = !on || le_tol(v[r], hi_of(tx * op[(25 + r) * stride]));
+    if (!feas) ok = false;
+    if ((act >> r) & 1u) {
+      if (!le_tol(-mu[r], th)) { ok = false; nact &= ~(1u << r); }
+    } else if (!feas) {
+      nact |= 1u << r;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double below = P.lo[i] - x[i], above = x[i] - P.hi[i];
+    if (!((fx >> i) & 1u)) {
+      if (abs_hi(g[i]) > th) ok = false;  // stationary in the free variables before the refinement
+      if (!le_tol(below, txh)) { ok = false; nfx |= 1u << i; nhs &= ~(1u << i); }
+      else if (!le_tol(above, txh)) { ok = false; nfx |= 1u << i; nhs |= 1u << i; }
+      if ((long long)bits_of(below) > 0) x[i] = P.lo[i];
+      if ((long long)bits_of(above) > 0) x[i] = P.hi[i];
+    } else if (bits_of(P.lo[i]) != bits_of(P.hi[i]) && ((bits_of(P.lo[i]) | bits_of(P.hi[i])) << 1)) {
+      if (!le_tol(((hs >> i) & 1u) ? g[i] : -g[i], th)) { ok = false; nfx &= ~(1u << i); nhs &= ~(1u << i); }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) u[r] = ((act >> r) & 1u) && pos_w(mu[r]) ? mu[r] : 0.0;
+  next = nfx | (nhs << 4) | (nact << 8);
+  return ok;
+}
+
+// the set that a solution shows: bounds that x equals, rows with a multiplier
+ACOPF_HD inline unsigned line_set_of(const LineQP<double>& P, const double x[4], const double u[4]) {
+  unsigned set = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (x[i] <= P.lo[i] || !(P.lo[i] < P.hi[i])) set |= 1u << i;
+    else if (x[i] >= P.hi[i]) set |= 0x11u << i;
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if (u[r] > 0.0 && row_on(P, r)) set |= 0x100u << r;
+  return set;
+}
+
 }  // namespace acopf

@@ -185,6 +185,19 @@ __device__ __forceinline__ void gen_compute(const Dev& d, int g, const V4<T>& a,
   ((V2<T>*)d.XG)[g] = gen_value(a, b, ((const V2<T>*)d.ZG)[g], ((const V2<T>*)d.LG)[g]);
 }
 
+// FP64 resident forms: the two divisors are constant during a sweep, so the
+// thread keeps their reciprocals (an FP64 division is some ten FP64
+// instructions, in the same warp as the first branches)
+__device__ __forceinline__ void gen_compute_kept(const Dev& d, int g, const V4<double>& a, const V4<double>& b,
+                                                 double inv_p, double inv_q) {
+  const double rho = b.z;
+  const V2<double> z = ((const V2<double>*)d.ZG)[g], lam = ((const V2<double>*)d.LG)[g];
+  V2<double> x;
+  x.x = clampv((rho * z.x - lam.x - a.x) * inv_p, a.z, a.w);
+  x.y = clampv((rho * z.y - lam.y) * inv_q, b.x, b.y);
+  ((V2<double>*)d.XG)[g] = x;
+}
+
 template <typename T>
 __device__ __forceinline__ void gen_phase(const SweepP<T>& p, int g, float sc) {
   const Dev& d = p.d;
@@ -266,6 +279,54 @@ __device__ __noinline__ T rb_rescale(const Dev& d, int l, float sc, V4<T>* rs, i
   return rn;
 }
 
+// The line subproblem of a branch from its record and the bus side's z, lambda
+template <typename T, typename Rec>
+__device__ __forceinline__ void line_problem(const Rec& rec, const V4<T>& z0, const V4<T>& z1, const V4<T>& l0,
+                                             const V4<T>& l1, T rho, LineQP<T>& P) {
+  // couplings: flows p_ij q_ij p_ji q_ji (F rows 0..3), voltages dbar 0..3
+  const T zf[4] = {z0.x, z0.y, z1.x, z1.y}, lf[4] = {l0.x, l0.y, l1.x, l1.y};
+  const T zv[4] = {z0.z, z0.w, z1.z, z1.w}, lv[4] = {l0.z, l0.w, l1.z, l1.w};
+#pragma unroll
+  for (int k = 0; k < 10; ++k) P.q[k] = rec(k);
+  // c = c0 + F'(lambda_F - rho z_F) + lambda_V - rho z_V
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    T s = rec(30 + i) + lv[i] - rho * zv[i];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) s += rec(10 + 4 * f + i) * (lf[f] - rho * zf[f]);
+    P.c[i] = s;
+    P.lo[i] = rec(34 + i);
+    P.hi[i] = rec(38 + i);
+  }
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) P.R[e][i] = rec(42 + 4 * e + i);
+    P.rb[e] = rec(50 + e);
+    P.on[e] = rec(54 + e) > T(0);
+  }
+  P.alo = rec(52);
+  P.ahi = rec(53);
+  P.ang = P.ahi < T(1e29);
+}
+
+// its outputs: flows and voltages of both ends, the row multipliers
+template <typename T, typename Rec>
+__device__ __forceinline__ void line_outputs(const Rec& rec, const T* x, const T* u, V4<T>& o0, V4<T>& o1, V4<T>& ou) {
+  // flows at the solution (F and f0 read again)
+  T xf[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    T s = rec.again(26 + f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s += rec.again(10 + 4 * f + i) * x[i];
+    xf[f] = s;
+  }
+  o0.x = xf[0]; o0.y = xf[1]; o0.z = x[0]; o0.w = x[1];
+  o1.x = xf[2]; o1.y = xf[3]; o1.z = x[2]; o1.w = x[3];
+  ou.x = u[0]; ou.y = u[1]; ou.z = u[2]; ou.w = u[3];
+}
+
 // One branch's line subproblem.  rec reads the branch's record (global
 // memory, a shared-memory tile or registers); values are read where they are
 // used rather than copied to registers, to keep the kernel's register count
@@ -296,33 +357,9 @@ __device__ __forceinline__ void line_compute(const SweepP<T>& p, int l, const Re
 template <typename T, typename Rec, typename Out>
 __device__ __forceinline__ void line_compute_to(const SweepP<T>& p, int l, const Rec& rec, V4<T> z0, V4<T> z1,
                                                 V4<T> l0, V4<T> l1, V4<T> uu, T rho, Out out, unsigned* wset) {
-  const Dev& d = p.d;
-  // couplings: flows p_ij q_ij p_ji q_ji (F rows 0..3), voltages dbar 0..3
-  const T zf[4] = {z0.x, z0.y, z1.x, z1.y}, lf[4] = {l0.x, l0.y, l1.x, l1.y};
-  const T zv[4] = {z0.z, z0.w, z1.z, z1.w}, lv[4] = {l0.z, l0.w, l1.z, l1.w};
+  const T zv[4] = {z0.z, z0.w, z1.z, z1.w};
   LineQP<T> P;
-#pragma unroll
-  for (int k = 0; k < 10; ++k) P.q[k] = rec(k);
-  // c = c0 + F'(lambda_F - rho z_F) + lambda_V - rho z_V
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    T s = rec(30 + i) + lv[i] - rho * zv[i];
-#pragma unroll
-    for (int f = 0; f < 4; ++f) s += rec(10 + 4 * f + i) * (lf[f] - rho * zf[f]);
-    P.c[i] = s;
-    P.lo[i] = rec(34 + i);
-    P.hi[i] = rec(38 + i);
-  }
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) P.R[e][i] = rec(42 + 4 * e + i);
-    P.rb[e] = rec(50 + e);
-    P.on[e] = rec(54 + e) > T(0);
-  }
-  P.alo = rec(52);
-  P.ahi = rec(53);
-  P.ang = P.ahi < T(1e29);
+  line_problem(rec, z0, z1, l0, l1, rho, P);
   T x[4], u[4] = {uu.x, uu.y, uu.z, uu.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = clampv(zv[i], P.lo[i], P.hi[i]);
@@ -352,20 +389,90 @@ __device__ __forceinline__ void line_compute_to(const SweepP<T>& p, int l, const
     const T beta = p.beta_scale * fmax(fmax(P.q[0], P.q[4]), fmax(P.q[7], P.q[9]));
     line_solve(P, x, u, beta, p.alm_tol, p.alm_outer, p.newton_max, nullptr, wset);
   }
-  // flows at the solution (F and f0 read again)
-  T xf[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    T s = rec.again(26 + f);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) s += rec.again(10 + 4 * f + i) * x[i];
-    xf[f] = s;
-  }
   V4<T> o0, o1, ou;
-  o0.x = xf[0]; o0.y = xf[1]; o0.z = x[0]; o0.w = x[1];
-  o1.x = xf[2]; o1.y = xf[3]; o1.z = x[2]; o1.w = x[3];
-  ou.x = u[0]; ou.y = u[1]; ou.z = u[2]; ou.w = u[3];
+  line_outputs(rec, x, u, o0, o1, ou);
   out(o0, o1, ou);
+}
+
+// FP64 resident forms: the line update with the branch's active set and the
+// set's operator kept from one iteration to the next (line_eval; op in shared
+// memory, one column per thread).  The set is corrected up to three times; a
+// subproblem that this does not settle, and line_solver = 1, take the general
+// solves above.  Bound by the count of FP64 instructions on the slowest warp
+// (see line_qp.cuh); full FP64 solves: 2,000 buses 244 -> 157 ms (30.5 -> 19.7
+// us per iteration), 30 buses 638 -> 402 ms (22 -> 14).
+__device__ __noinline__ bool line_operator_call(const LineQP<double>& P, unsigned set, double* op, int stride) {
+  return line_operator(P, set, op, stride);
+}
+__device__ __noinline__ void line_general_call(const LineQP<double>& P, const double* z, double* x, double* u,
+                                               int exact, double beta_scale, double tol, int outer, int newton) {
+  const double u_in[4] = {u[0], u[1], u[2], u[3]};
+  for (int i = 0; i < 4; ++i) x[i] = clampv(z[i], P.lo[i], P.hi[i]);
+  if (exact) {
+    if (line_pred_call(P, x, u)) return;
+    for (int i = 0; i < 4; ++i) u[i] = u_in[i];
+    if (line_exact_call(P, x, u) >= 0) return;
+    for (int i = 0; i < 4; ++i) {
+      x[i] = clampv(z[i], P.lo[i], P.hi[i]);
+      u[i] = u_in[i];
+    }
+  }
+  const double beta = beta_scale * fmax(fmax(P.q[0], P.q[4]), fmax(P.q[7], P.q[9]));
+  line_alm_call(P, x, u, beta, tol, outer, newton);
+}
+
+template <typename Rec>
+__device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, int l, const Rec& rec, V4<double> z0,
+                                                  V4<double> z1, V4<double> l0, V4<double> l1, V4<double> uu,
+                                                  double rho, unsigned& set, double* op, int stride) {
+  LineQP<double> P;
+  line_problem(rec, z0, z1, l0, l1, rho, P);
+  double x[4], u[4];
+  bool ok = false;
+  if (p.line_exact) {
+    for (int attempt = 0; attempt < 4; ++attempt) {
+      if (!(set & kSetValid)) {
+        const LineQP<double> Q = P;  // a copy for the call: P itself stays in registers
+        if (!line_operator_call(Q, set, op, stride)) break;
+        set |= kSetValid;
+      }
+      unsigned next;
+      ok = line_eval(P, set, op, stride, x, u, next);
+      if (ok || next == (set & ~kSetValid)) break;
+      set = next;
+    }
+  }
+  if (!ok) {
+    const LineQP<double> Q = P;
+    const double zv[4] = {z0.z, z0.w, z1.z, z1.w};
+    double xs[4], us[4] = {uu.x, uu.y, uu.z, uu.w};
+    line_general_call(Q, zv, xs, us, p.line_exact, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
+    set = line_set_of(Q, xs, us);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x[i] = xs[i];
+      u[i] = us[i];
+    }
+  }
+  V4<double> o0, o1, ou;
+  line_outputs(rec, x, u, o0, o1, ou);
+  V4<double>* X = (V4<double>*)p.d.X;
+  X[2 * l] = o0;
+  X[2 * l + 1] = o1;
+  ((V4<double>*)p.d.U)[l] = ou;
+}
+
+// the set shown by the branch's last point (from global memory), where a
+// launch starts
+template <typename Rec>
+__device__ __forceinline__ unsigned line_set_start(const Dev& d, int l, const Rec& rec) {
+  LineQP<double> P;
+  const V4<double> zero = {0.0, 0.0, 0.0, 0.0};
+  line_problem(rec, zero, zero, zero, zero, 0.0, P);
+  const V4<double> x0 = ((const V4<double>*)d.X)[2 * l], x1 = ((const V4<double>*)d.X)[2 * l + 1];
+  const V4<double> uu = ((const V4<double>*)d.U)[l];
+  const double x[4] = {x0.z, x0.w, x1.z, x1.w}, u[4] = {uu.x, uu.y, uu.z, uu.w};
+  return line_set_of(P, x, u);
 }
 
 // line update of branch l reading its record from global memory (rs, stride L)
@@ -939,20 +1046,23 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
   int my_k = -1;
   V4<T> rr[kRecChunks];
   T my_rho = T(0);
-  unsigned my_wset = 0u;  // the box bounds held at the end of the branch's last solve
+  unsigned my_wset = 0u;  // the box bounds held at the end of the branch's last solve; FP64: its active set
+  double* s_op = (double*)(((uintptr_t)(s_scale + K) + 15) & ~(uintptr_t)15);  // RES FP64: kLineOp values per thread
   TaskStatic<T> ta, tb;
   if (RES) {
     if (tid < d.G) {
       my_k = d.gen_inst[tid];
       rr[0] = ((const V4<T>*)d.grec)[tid];
       rr[1] = ((const V4<T>*)d.grec)[d.G + tid];
+      if (sizeof(T) == 8) rr[2] = {T(1) / (rr[0].y + rr[1].z), T(1) / rr[1].z, T(0), T(0)};
     } else if (tid < d.G + d.L) {
       const int l = tid - d.G;
       my_k = d.br_inst[l];
 #pragma unroll
       for (int c = 0; c < kRecChunks; ++c) rr[c] = ((const V4<T>*)d.lrec)[(size_t)c * d.L + l];
       my_rho = ((const T*)d.trho_l)[l];
-      my_wset = d.wset[l];
+      if constexpr (sizeof(T) == 8) my_wset = line_set_start(d, l, RRec<T>{rr});
+      else my_wset = d.wset[l];
     }
     ta = task_static<T>(d, wid < d.NT ? load_slot(d, wid, lane) : none);
     tb = task_static<T>(d, wid + nw < d.NT ? load_slot(d, wid + nw, lane) : none);
@@ -969,13 +1079,18 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     if (RES) {
       if (my_k >= 0 && !s_done[my_k]) {
         if (tid < d.G) {
-          gen_compute(d, tid, rr[0], rr[1]);
+          if constexpr (sizeof(T) == 8) gen_compute_kept(d, tid, rr[0], rr[1], rr[2].x, rr[2].y);
+          else gen_compute(d, tid, rr[0], rr[1]);
         } else {
           const int l = tid - d.G;
           const V4<T>* Z = (const V4<T>*)d.Z;
           const V4<T>* LM = (const V4<T>*)d.LAM;
-          line_compute(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1], ((const V4<T>*)d.U)[l],
-                       my_rho, &my_wset);
+          if constexpr (sizeof(T) == 8)
+            line_compute_kept(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1],
+                              ((const V4<T>*)d.U)[l], my_rho, my_wset, s_op + threadIdx.x, blockDim.x);
+          else
+            line_compute(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1], ((const V4<T>*)d.U)[l],
+                         my_rho, &my_wset);
         }
       }
     } else if (!kTiled) {
@@ -1198,18 +1313,22 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
   // RES: this thread's generator or branch record, this warp's two tasks
   V4<T> rr[kRecChunks];
   T my_rho = T(0);
-  unsigned my_wset = 0u;  // the box bounds held at the end of the branch's last solve
+  unsigned my_wset = 0u;  // the box bounds held at the end of the branch's last solve; FP64: its active set
+  extern __shared__ __align__(16) unsigned char s_dyn_c[];
+  double* s_op = (double*)s_dyn_c;  // RES FP64: kLineOp values per thread
   TaskStatic<T> ta, tb;
   if (RES) {
     if (ct < nG) {
       rr[0] = ((const V4<T>*)d.grec)[g0 + ct];
       rr[1] = ((const V4<T>*)d.grec)[d.G + g0 + ct];
+      if (sizeof(T) == 8) rr[2] = {T(1) / (rr[0].y + rr[1].z), T(1) / rr[1].z, T(0), T(0)};
     } else if (l0 + ct - nG < l1) {
       const int l = l0 + ct - nG;
 #pragma unroll
       for (int c = 0; c < kRecChunks; ++c) rr[c] = ((const V4<T>*)d.lrec)[(size_t)c * d.L + l];
       my_rho = ((const T*)d.trho_l)[l];
-      my_wset = d.wset[l];
+      if constexpr (sizeof(T) == 8) my_wset = line_set_start(d, l, RRec<T>{rr});
+      else my_wset = d.wset[l];
     }
     ta = task_static<T>(d, t0 + cw < t1 ? load_slot(d, t0 + cw, lane) : none);
     tb = task_static<T>(d, t0 + cw + nwc < t1 ? load_slot(d, t0 + cw + nwc, lane) : none);
@@ -1225,13 +1344,18 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
     // phase A: the instance's generators, then its branches
     if (RES) {
       if (ct < nG) {
-        gen_compute(d, g0 + ct, rr[0], rr[1]);
+        if constexpr (sizeof(T) == 8) gen_compute_kept(d, g0 + ct, rr[0], rr[1], rr[2].x, rr[2].y);
+        else gen_compute(d, g0 + ct, rr[0], rr[1]);
       } else if (l0 + ct - nG < l1) {
         const int l = l0 + ct - nG;
         const V4<T>* Z = (const V4<T>*)d.Z;
         const V4<T>* LM = (const V4<T>*)d.LAM;
-        line_compute(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1], ((const V4<T>*)d.U)[l],
-                     my_rho, &my_wset);
+        if constexpr (sizeof(T) == 8)
+          line_compute_kept(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1],
+                            ((const V4<T>*)d.U)[l], my_rho, my_wset, s_op + threadIdx.x, blockDim.x);
+        else
+          line_compute(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1], ((const V4<T>*)d.U)[l],
+                       my_rho, &my_wset);
       }
     } else {
       int u = ct;
@@ -1634,6 +1758,12 @@ static size_t sweep_smem(int K, int threads, int stages) {
   return b;
 }
 
+// dynamic shared memory of the kept line operators (FP64 resident forms)
+template <typename T>
+static size_t op_smem(int threads) {
+  return sizeof(T) == 8 ? (size_t)kLineOp * sizeof(double) * threads : 0;
+}
+
 // Launch shape of k_sweep<T>.  The resident form (sweep_stages 3) is used when
 // residual balancing is off and a co-resident grid gives every generator and
 // branch a thread of its own and every warp at most two bus tasks; otherwise
@@ -1650,7 +1780,7 @@ static acopf_status sweep_shape(Ctx& c, const SweepP<T>& p, SweepShape& sh) {
   const Dev& d = c.d;
   const int threads = c.block_threads;
   if (c.sweep_stages == 3 && p.rb_period == 0) {
-    const size_t smem = sweep_smem<T>(d.K, threads, 0);
+    const size_t smem = sweep_smem<T>(d.K, threads, 0) + 16 + op_smem<T>(threads);
     cudaFuncSetAttribute(k_sweep<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, true>, threads, smem);
@@ -1711,6 +1841,8 @@ static int cluster_size(Ctx& c, int threads, cudaLaunchConfig_t& cfg, cudaLaunch
   if (cs > 16) cs = 16;
   void* fn = res ? (void*)k_sweep_cluster<T, true> : (void*)k_sweep_cluster<T, false>;
   cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cfg.dynamicSmemBytes = res ? op_smem<T>(threads) : 0;
+  if (cfg.dynamicSmemBytes) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
   const long cs_b1 = (tasks + wpb - 1) / wpb;
   if (sizeof(T) == 8 && res && cs_b1 > cs && cs_b1 <= 16) {
     cfg.gridDim = dim3((unsigned)cs_b1);
@@ -1726,6 +1858,7 @@ static int cluster_size(Ctx& c, int threads, cudaLaunchConfig_t& cfg, cudaLaunch
     if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) break;
     cudaGetLastError();
     res = false;  // a smaller cluster no longer covers every component
+    cfg.dynamicSmemBytes = 0;
     fn = (void*)k_sweep_cluster<T, false>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   }
@@ -1771,7 +1904,7 @@ static acopf_status run_sweep_cluster(Ctx& c, const SweepP<T>& p) {
   }
   const int cs = c.cluster_cs;
   attr[0].val.clusterDim.x = cs;
-  if (c.cluster_dsm) cfg.dynamicSmemBytes = dsm_smem;
+  cfg.dynamicSmemBytes = c.cluster_dsm ? dsm_smem : (c.cluster_res ? op_smem<T>(threads) : 0);
   if (!c.capturing) cudaMemsetAsync(c.d.err, 0, sizeof(int), c.stream);
   cfg.gridDim = dim3((unsigned)(c.d.K * cs));
   const bool prof = c.profiling && !c.capturing;

@@ -47,3 +47,28 @@ extern "C" void host_line_solves(int n, const double* in, int* ok, double* xp, d
     for (int i = 0; i < 4; ++i) { xe[4 * b + i] = x2[i]; ue[4 * b + i] = u2[i]; }
   }
 }
+
+// per problem: the kept-set solve -- the set of (x, u) given, its operator,
+// evaluation and up to three corrections -- its flag, x, u and the number of
+// operators built
+extern "C" void host_line_kept(int n, const double* in, const double* x0, const double* u0, int* ok, double* x,
+                               double* u, int* built) {
+  for (int b = 0; b < n; ++b) {
+    LineQP<double> P = make(in + 41 * b);
+    double op[2 * kLineOp];  // stride 2
+    unsigned set = line_set_of(P, x0 + 4 * b, u0 + 4 * b);
+    ok[b] = 0;
+    built[b] = 0;
+    for (int attempt = 0; attempt < 4; ++attempt) {
+      if (!(set & kSetValid)) {
+        ++built[b];
+        if (!line_operator(P, set, op, 2)) break;
+        set |= kSetValid;
+      }
+      unsigned next;
+      ok[b] = line_eval(P, set, op, 2, x + 4 * b, u + 4 * b, next);
+      if (ok[b] || next == (set & ~kSetValid)) break;
+      set = next;
+    }
+  }
+}

@@ -137,3 +137,64 @@ def test_predicted_line_solve_matches_the_dual_method(lib):
     su = np.maximum(1.0, np.abs(ue).max(1))
     assert (np.abs(xp - xe).max(1) / sx)[both].max() <= 1e-10
     assert (np.abs(up - ue).max(1) / su)[both].max() <= 1e-8
+
+
+@pytest.mark.parametrize("start", ["solution", "neighbour", "nothing"])
+def test_kept_set_line_solve_matches_the_dual_method(lib, start):
+    """The affine operator of an active set (line_operator, line_eval) from the
+    solution's own set, the set of a neighbouring subproblem (c changed by one
+    ADMM iteration's worth) and no set: where it is accepted it is the dual
+    method's KKT point, it is accepted at once on the right set, and never
+    where no point is feasible."""
+    rng = np.random.default_rng(17)
+    n = 3000
+    P = np.ascontiguousarray(_random_problems(rng, n))
+    N = P.copy()
+    if start == "neighbour":
+        N[:, 10:14] += 1e-3 * np.abs(P[:, 10:14]).max(1, keepdims=True) * rng.standard_normal((n, 4))
+
+    def solves(A):
+        ok, st = np.zeros(n, dtype=np.int32), np.zeros(n, dtype=np.int32)
+        xp, up, xe, ue = (np.zeros((n, 4)) for _ in range(4))
+        lib.host_line_solves(n, A.ctypes.data_as(DP), ok.ctypes.data_as(IP), xp.ctypes.data_as(DP),
+                             up.ctypes.data_as(DP), st.ctypes.data_as(IP), xe.ctypes.data_as(DP),
+                             ue.ctypes.data_as(DP))
+        return st, xe, ue, xp, up
+
+    st, xe, ue, _, _ = solves(P)
+    # the sweep's own solves: the predicted method's point, exactly at the bounds it holds
+    _, _, _, xs, us = solves(N)
+    if start == "nothing":
+        xs, us = np.zeros((n, 4)), np.zeros((n, 4))
+    ok, built = np.zeros(n, dtype=np.int32), np.zeros(n, dtype=np.int32)
+    x, u = np.zeros((n, 4)), np.zeros((n, 4))
+    lib.host_line_kept(n, P.ctypes.data_as(DP), np.ascontiguousarray(xs).ctypes.data_as(DP),
+                       np.ascontiguousarray(us).ctypes.data_as(DP), ok.ctypes.data_as(IP), x.ctypes.data_as(DP),
+                       u.ctypes.data_as(DP), built.ctypes.data_as(IP))
+    feas, good = st >= 0, ok.astype(bool)
+    assert not (good & ~feas).any()
+    if start == "solution":  # every subproblem with at most two active rows, with the first operator
+        two = feas & ((us > 0).sum(1) <= 2)
+        assert good[two].all() and (built[two] == 1).all()
+    else:
+        assert good.sum() > n // 4
+    both = good & feas
+    sx = np.maximum(1e-3, np.abs(xe).max(1))
+    su = np.maximum(1.0, np.abs(ue).max(1))
+    # the bounds of test_predicted_line_solve_matches_the_dual_method
+    assert (np.abs(x - xe).max(1) / sx)[both].max() <= 1e-10
+    assert (np.abs(u - ue).max(1) / su)[both].max() <= 1e-8
+    for k in range(4):
+        assert (x[both, k] >= P[both, 14 + k]).all() and (x[both, k] <= P[both, 18 + k]).all()
+
+
+def test_kept_set_line_solve_refuses_non_finite_values(lib):
+    rng = np.random.default_rng(3)
+    P = np.ascontiguousarray(_random_problems(rng, 12))
+    for k, v in enumerate((np.nan, np.inf, -np.inf)):
+        P[4 * k:4 * k + 4, 10 + np.arange(4)] = np.where(np.eye(4) > 0, v, P[4 * k:4 * k + 4, 10:14])
+    ok, built = np.zeros(12, dtype=np.int32), np.zeros(12, dtype=np.int32)
+    x, u, z = np.zeros((12, 4)), np.zeros((12, 4)), np.zeros((12, 4))
+    lib.host_line_kept(12, P.ctypes.data_as(DP), z.ctypes.data_as(DP), z.ctypes.data_as(DP), ok.ctypes.data_as(IP),
+                       x.ctypes.data_as(DP), u.ctypes.data_as(DP), built.ctypes.data_as(IP))
+    assert not ok.any()
