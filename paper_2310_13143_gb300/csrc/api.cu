@@ -375,7 +375,7 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   // bus update work list and its warp tasks (consecutive whole buses, at most
   // 32 entries per task; a bus with more entries is a task of its own)
   const size_t E = (size_t)G + 2 * (size_t)L;
-  std::vector<int> ent(E), ebus(E), pent, pbus, pinst, big, task_off, big_off;
+  std::vector<int> ent(E), ebus(E), pent, pbus, pmeta, tinst, big, task_off, big_off;
   {
     size_t q = 0;
     for (int i = 0; i < B; ++i) {
@@ -386,12 +386,19 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
     size_t cnt = 0;  // its entries
     auto close = [&]() {
       if (cnt == 0) return;
-      for (size_t j = 0; j < 32; ++j) {
-        bool in = j < cnt;
+      // lanes of one bus are consecutive: first and last lane of each lane's bus
+      int first[32], lst[32], most = 0;
+      for (int j = 0; j < 32; ++j) first[j] = j > 0 && j < (int)cnt && ebus[q0 + j] == ebus[q0 + j - 1] ? first[j - 1] : j;
+      for (int j = 31; j >= 0; --j)
+        lst[j] = j + 1 < (int)cnt && ebus[q0 + j] == ebus[q0 + j + 1] ? lst[j + 1] : j;
+      for (int j = 0; j < (int)cnt; ++j) most = std::max(most, j - first[j]);
+      for (int j = 0; j < 32; ++j) {
+        const bool in = j < (int)cnt;
         pent.push_back(in ? ent[q0 + j] : 0);
         pbus.push_back(in ? ebus[q0 + j] : -1);
-        pinst.push_back(in ? bus_inst[ebus[q0 + j]] : -1);
+        pmeta.push_back(make_meta(j - first[j], lst[j], most, in && lst[j] == j, in && isref[ebus[q0 + j]]));
       }
+      tinst.push_back(bus_inst[ebus[q0]]);
       q0 += cnt;
       cnt = 0;
     };
@@ -434,7 +441,8 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   A(d.bus_inst, B); A(d.br_inst, L); A(d.gen_inst, G);
   A(d.pd, B); A(d.qd, B); A(d.gs, B); A(d.bs, B); A(d.wmin, B); A(d.wmax, B); A(d.isref, B);
   A(d.end_ptr, B + 1); A(d.end_idx, 2 * (size_t)L); A(d.gen_ptr, B + 1);
-  A(d.ent, E); A(d.ebus, E); A(d.pent, pent.size()); A(d.pbus, pbus.size()); A(d.pinst, pinst.size());
+  A(d.ent, E); A(d.ebus, E); A(d.pent, pent.size()); A(d.pbus, pbus.size()); A(d.pmeta, pmeta.size());
+  A(d.tinst, tinst.size());
   A(d.big, big.size()); A(d.task_off, K + 1); A(d.big_off, K + 1); A(d.wset, L);
   d.E = (int)E;
   d.NT = (int)(pbus.size() / 32);
@@ -453,7 +461,7 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   AR(d.X, T * 4 * 2 * (size_t)L); AR(d.Z, T * 4 * 2 * (size_t)L); AR(d.LAM, T * 4 * 2 * (size_t)L);
   AR(d.U, T * 4 * (size_t)L);
   AR(d.XG, T * 2 * (size_t)G); AR(d.ZG, T * 2 * (size_t)G); AR(d.LG, T * 2 * (size_t)G);
-  AR(d.ZB, T * 2 * (size_t)B); AR(d.NU, T * 2 * (size_t)B);
+  AR(d.ZB, T * 2 * (size_t)B); AR(d.NU, T * 2 * (size_t)B); AR(d.bk, T * 4 * (size_t)B);
   A(d.res_slots, 4 * (size_t)K); A(d.admm_done, K); A(d.admm_iters, K); A(d.admm_rs, 2 * (size_t)K);
   A(d.bar, 2); A(d.err, 1);
   A(d.flow_xd, 4 * (size_t)L); A(d.tbr, 8 * (size_t)L); A(d.tbus, 4 * (size_t)B); A(d.tgen, 8 * (size_t)G);
@@ -476,7 +484,8 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   U(d.bus_inst, bus_inst); U(d.br_inst, br_inst); U(d.gen_inst, gen_inst_s);
   U(d.pd, pd); U(d.qd, qd); U(d.gs, gs); U(d.bs, bs); U(d.wmin, wmin); U(d.wmax, wmax); U(d.isref, isref);
   U(d.end_ptr, end_ptr); U(d.end_idx, end_idx); U(d.gen_ptr, gen_ptr);
-  U(d.ent, ent); U(d.ebus, ebus); U(d.pent, pent); U(d.pbus, pbus); U(d.pinst, pinst); U(d.big, big);
+  U(d.ent, ent); U(d.ebus, ebus); U(d.pent, pent); U(d.pbus, pbus); U(d.pmeta, pmeta);
+  U(d.tinst, tinst); U(d.big, big);
   U(d.task_off, task_off); U(d.big_off, big_off);
   c->h_task_off = task_off;
   c->h_big_off = big_off;

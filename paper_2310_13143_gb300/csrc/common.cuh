@@ -75,6 +75,13 @@ __host__ __device__ inline bool live(const InstCtl& c, int pass) {
   return c.result == ACOPF_RUNNING && (pass == 0 || c.soc_active);
 }
 
+// A bus-task lane's place in its bus's segment: entries of the bus on lower
+// lanes (bits 0-4), the bus's last lane (5-9), the task's largest such count
+// (10-14), whether this is the last lane (15), reference bus (16)
+inline int make_meta(int up, int src, int most, bool last, bool ref) {
+  return up | (src << 5) | (most << 10) | ((int)last << 15) | ((int)ref << 16);
+}
+
 // raw device pointers shared by all kernels
 struct Dev {
   int K, B, L, G;
@@ -88,10 +95,11 @@ struct Dev {
   // branch ends) is ent[q] = -(g + 1) for generator g or the end id 2 l + side,
   // ebus[q] its bus.  Warp tasks of consecutive whole buses with at most 32
   // entries are stored padded: slot 32 t + j holds lane j's entry (pent), bus
-  // (pbus, -1: empty) and instance (pinst).  A bus with more than 32 entries
-  // is a big task: entries [big[2 b], big[2 b + 1]) of ent/ebus.
+  // (pbus, -1: empty) and place in its bus's segment of lanes (pmeta, see
+  // make_meta); tinst[t] is the task's instance.  A bus with more than 32
+  // entries is a big task: entries [big[2 b], big[2 b + 1]) of ent/ebus.
   int *ent, *ebus;
-  int *pent, *pbus, *pinst;
+  int *pent, *pbus, *pmeta, *tinst;
   int* big;
   int E, NT, NBIG;
   // per branch: the box bounds held at the end of its last FP32 line solve in
@@ -133,6 +141,7 @@ struct Dev {
   void* U;            // V4 [L]
   void *XG, *ZG, *LG; // V2 [G]
   void *ZB, *NU;      // V2 [B]
+  void* bk;           // V4 [B] what the penalties give of each bus's system (formed by the streaming sweep)
   // sweep control
   unsigned long long* res_slots; // [2 slots][2 (r,s)][K]
   int* admm_done;     // [K]

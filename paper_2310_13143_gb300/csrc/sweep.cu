@@ -576,54 +576,39 @@ __device__ __forceinline__ T nan_big(T v) {
   else return v == v ? v : T(1e30);
 }
 
-// Warp-level max of the residuals over runs of lanes that hold the same
-// instance (buses are sorted by instance, so runs are contiguous): a segmented
-// shuffle-down reduction in the sweep precision, then one 64-bit atomicMax per
-// run and residual.  All 32 lanes must call it; lanes without a bus pass inst = -1.
-template <typename T>
-__device__ __forceinline__ void res_max2(const ResDst& dst, T r, T s, int inst) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    T r2 = __shfl_down_sync(FULL, r, o);
-    T s2 = __shfl_down_sync(FULL, s, o);
-    int k2 = __shfl_down_sync(FULL, inst, o);
-    if (lane + o < 32 && k2 == inst) {
-      r = rmax(r, r2);
-      s = rmax(s, s2);
-    }
-  }
-  int kprev = __shfl_up_sync(FULL, inst, 1);
-  bool leader = (lane == 0 || kprev != inst) && inst >= 0;
-  if (leader) dst.put(inst, r, s);
+// max over the warp of a non-negative value (not NaN), on its bit pattern,
+// which orders such values as unsigned integers: one reduction instruction in
+// FP32, two in FP64 (the leading words, then the trailing words of the lanes
+// that hold the largest leading word), against five shuffle steps
+__device__ __forceinline__ float warp_max(float v) {
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ double warp_max(double v) {
+  const unsigned long long b = bits_of(v);
+  const unsigned hi = (unsigned)(b >> 32);
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)b : 0u);
+  return double_of(((unsigned long long)mh << 32) | ml);
 }
 
-// res_max2 for two tasks at once
-template <typename T>
-__device__ __forceinline__ void res_max2_pair(const ResDst& dst, T ra, T sa, int ka, T rb, T sb, int kb) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    T ra2 = __shfl_down_sync(FULL, ra, o);
-    T sa2 = __shfl_down_sync(FULL, sa, o);
-    int ka2 = __shfl_down_sync(FULL, ka, o);
-    T rb2 = __shfl_down_sync(FULL, rb, o);
-    T sb2 = __shfl_down_sync(FULL, sb, o);
-    int kb2 = __shfl_down_sync(FULL, kb, o);
-    if (lane + o < 32 && ka2 == ka) {
-      ra = rmax(ra, ra2);
-      sa = rmax(sa, sa2);
-    }
-    if (lane + o < 32 && kb2 == kb) {
-      rb = rmax(rb, rb2);
-      sb = rmax(sb, sb2);
-    }
+// the residual maxima of one task, whose lanes all belong to instance inst
+// (-1: nothing to report; warp-uniform).  All 32 lanes call it.
+template <typename T, typename Dst>
+__device__ __forceinline__ void res_task(const Dst& dst, T r, T s, int inst) {
+  r = warp_max(r);
+  s = warp_max(s);
+  if ((threadIdx.x & 31) == 0 && inst >= 0) dst.put(inst, r, s);
+}
+
+// of two tasks at once: one reduction where they belong to one instance
+template <typename T, typename Dst>
+__device__ __forceinline__ void res_task_pair(const Dst& dst, T ra, T sa, int ka, T rb, T sb, int kb) {
+  if (ka == kb || kb < 0) {  // an empty task holds zeros
+    res_task(dst, rmax(ra, rb), rmax(sa, sb), ka);
+  } else {
+    res_task(dst, ra, sa, ka);
+    res_task(dst, rb, sb, kb);
   }
-  const int kpa = __shfl_up_sync(FULL, ka, 1), kpb = __shfl_up_sync(FULL, kb, 1);
-  if ((lane == 0 || kpa != ka) && ka >= 0) dst.put(ka, ra, sa);
-  if ((lane == 0 || kpb != kb) && kb >= 0) dst.put(kb, rb, sb);
 }
 
 // ---------------------------------------------------------- bus update
@@ -634,9 +619,29 @@ __device__ __forceinline__ void res_max2_pair(const ResDst& dst, T ra, T sa, int
 // warp scan over the bus ids (a bus's entries are consecutive lanes); the
 // segment's last lane solves its bus and the solution is broadcast back to
 // the segment, where every lane updates its own coupling.
+//
+// Where one instance has the GPU to itself the phase is bound by its dependent
+// chain, so everything that does not change from one iteration to the next is
+// taken out of it: the segment structure of a task is stored with its slots
+// (Slot), the scan stops at the task's longest segment (most buses have at
+// most eight entries: three steps instead of five), and the two sums over the
+// penalties, with the quotients that need them, are formed once per sweep
+// (bus_const; again after residual balancing has changed the penalties) -- four
+// sums are scanned instead of six.  Full solves of the 2,000-bus grid: mixed
+// 45.9 -> 40.8 ms, FP64 157 -> 135 ms; 30 buses in FP64 402 -> 331 ms.  The
+// batches, whose phase waits on its gathers, gain 1-2 %.
 
 struct Slot {
-  int bus, code, inst;  // bus -1: empty lane
+  int bus, code;  // bus -1: empty lane
+  int meta;       // see make_meta
+  int inst;       // of the task (warp-uniform), -1: no task
+  // entries of the same bus on lower lanes; last lane of the bus; the largest
+  // up() of the task; whether this is the bus's last lane; reference bus
+  __device__ __forceinline__ int up() const { return meta & 31; }
+  __device__ __forceinline__ int src() const { return (meta >> 5) & 31; }
+  __device__ __forceinline__ int most() const { return (meta >> 10) & 31; }
+  __device__ __forceinline__ bool last() const { return (meta >> 15) & 1; }
+  __device__ __forceinline__ bool ref() const { return (meta >> 16) & 1; }
 };
 
 __device__ __forceinline__ Slot load_slot(const Dev& d, int t, int lane) {
@@ -644,9 +649,11 @@ __device__ __forceinline__ Slot load_slot(const Dev& d, int t, int lane) {
   Slot s;
   s.bus = d.pbus[i];
   s.code = d.pent[i];
-  s.inst = d.pinst[i];
+  s.meta = d.pmeta[i];
+  s.inst = d.tinst[t];
   return s;
 }
+__device__ __forceinline__ Slot empty_slot(int lane) { return Slot{-1, 0, lane << 5, -1}; }
 
 template <typename T>
 __device__ __forceinline__ void entry_load(const Dev& d, int c, V4<T>& x, V4<T>& lm, V4<T>& zo, T& r) {
@@ -665,9 +672,6 @@ __device__ __forceinline__ void entry_load(const Dev& d, int c, V4<T>& x, V4<T>&
   }
 }
 
-// contributions to the bus sums: c = lambda + rho x per coupling; the 2x2
-// matrix sums 1/rho over every coupled flow, generators enter with +, branch
-// ends with - (they draw power from the bus)
 // a / r: in FP64 the product with one reciprocal of r (a correctly rounded
 // division costs many FP64 instructions on GB300, whose FP64 rate is a small
 // fraction of FP32); in FP32 the special-function quotient
@@ -677,66 +681,69 @@ __device__ __forceinline__ T over_r(T a, T r, T ir) {
   else return div_w(a, r);
 }
 
-// 1/r of a coupling's penalty, used by entry_sums and (FP64) entry_values:
-// the FP64 sweep takes the correctly rounded quotient once per coupling and
-// iteration (ir_once) and passes it to both; the FP32 sweep takes the
-// special-function quotient where entry_sums uses it (ir_at), as
-// entry_values does not need it
+// 1/r of a coupling's penalty where the FP64 sweep multiplies by it (the
+// correctly rounded quotient); the FP32 sweep divides and needs none
 template <typename T>
 __device__ __forceinline__ T ir_once(T r) {
   if constexpr (sizeof(T) == 8) return div_w(T(1), r);
   else return T(0);
 }
-template <typename T>
-__device__ __forceinline__ T ir_at(T r, T once) {
-  if constexpr (sizeof(T) == 8) return once;
-  else return div_w(T(1), r);
-}
 
-// ir = 1/r (see ir_once)
+// contributions to the bus sums that change every iteration: c = lambda + rho
+// x per coupling, flows over rho; generators enter with +, branch ends with -
+// (they draw power from the bus)
 template <typename T>
 __device__ __forceinline__ void entry_sums(int c, const V4<T>& x, const V4<T>& lm, T r, T ir, T* S) {
-  S[0] += ir;
   if (c < 0) {
-    S[1] += over_r(lm.x + r * x.x, r, ir);
-    S[2] += over_r(lm.y + r * x.y, r, ir);
+    S[0] += over_r(lm.x + r * x.x, r, ir);
+    S[1] += over_r(lm.y + r * x.y, r, ir);
   } else {
-    S[1] -= over_r(lm.x + r * x.x, r, ir);
-    S[2] -= over_r(lm.y + r * x.y, r, ir);
-    S[3] += r;
-    S[4] += lm.z + r * x.z;
-    S[5] += lm.w + r * x.w;
+    S[0] -= over_r(lm.x + r * x.x, r, ir);
+    S[1] -= over_r(lm.y + r * x.y, r, ir);
+    S[2] += lm.z + r * x.z;
+    S[3] += lm.w + r * x.w;
   }
 }
 
-// the 2x2 system (A Q^-1 A') nu = A Q^-1 c - b of the bus's power-balance rows
-// with shunts, then d_w and d_theta; writes ZB, NU
+// What the penalties alone give of a bus's system (A Q^-1 A') nu = A Q^-1 c -
+// b: the sums of 1/rho over its flows and of rho over its voltage copies, and
+// 1 / the latter; in FP64 also 1 / determinant.  Held per bus (Dev::bk).
 template <typename T>
-__device__ __forceinline__ void bus_values(V4<T> br, int isref, const T* S, T& n1, T& n2, T& dw, T& dth) {
+__device__ __forceinline__ V4<T> bus_const(V4<T> br, T sinv, T sr) {
   const T gsh = br.z, bsh = br.w;
-  const T iQw = S[3] > T(0) ? div_w(T(1), S[3]) : T(0);  // a bus without branch ends has no voltage copies
-  const T M11 = S[0] + gsh * gsh * iQw;
-  const T M22 = S[0] + bsh * bsh * iQw;
+  const T iQw = sr > T(0) ? div_w(T(1), sr) : T(0);  // a bus without branch ends has no voltage copies
+  T idet = T(0);
+  if constexpr (sizeof(T) == 8) {
+    const T M11 = sinv + gsh * gsh * iQw, M22 = sinv + bsh * bsh * iQw, M12 = -gsh * bsh * iQw;
+    idet = div_w(T(1), M11 * M22 - M12 * M12);
+  }
+  return V4<T>{sinv, sr, iQw, idet};
+}
+
+// the 2x2 system of the bus's power-balance rows with shunts, then d_w and
+// d_theta, from the scanned sums S and the bus's constants k
+template <typename T>
+__device__ __forceinline__ void bus_values(const V4<T>& br, bool isref, const V4<T>& k, const T* S, T& n1, T& n2,
+                                           T& dw, T& dth) {
+  const T gsh = br.z, bsh = br.w;
+  const T iQw = k.z;
+  const T M11 = k.x + gsh * gsh * iQw;
+  const T M22 = k.x + bsh * bsh * iQw;
   const T M12 = -gsh * bsh * iQw;
-  const T v1 = S[1] - gsh * S[4] * iQw - br.x;
-  const T v2 = S[2] + bsh * S[4] * iQw - br.y;
-  const T det = M11 * M22 - M12 * M12;
-  const T idet = sizeof(T) == 8 ? div_w(T(1), det) : T(0);
-  n1 = over_r(M22 * v1 - M12 * v2, det, idet);
-  n2 = over_r(M11 * v2 - M12 * v1, det, idet);
-  dw = (S[4] + gsh * n1 - bsh * n2) * iQw;
-  dth = (isref || !(S[3] > T(0))) ? T(0) : over_r(S[5], S[3], iQw);
+  const T v1 = S[0] - gsh * S[2] * iQw - br.x;
+  const T v2 = S[1] + bsh * S[2] * iQw - br.y;
+  T det = T(0);
+  if constexpr (sizeof(T) == 4) det = M11 * M22 - M12 * M12;
+  n1 = over_r(M22 * v1 - M12 * v2, det, k.w);
+  n2 = over_r(M11 * v2 - M12 * v1, det, k.w);
+  dw = (S[2] + gsh * n1 - bsh * n2) * iQw;
+  dth = (isref || !pos_w(k.y)) ? T(0) : over_r(S[3], k.y, iQw);
 }
 
 template <typename T>
-__device__ __forceinline__ void bus_solve(const Dev& d, int bus, V4<T> br, int isref, const T* S, T& n1, T& n2,
-                                          T& dw, T& dth) {
-  bus_values(br, isref, S, n1, n2, dw, dth);
-  V2<T> zb, nu;
-  zb.x = dw; zb.y = dth;
-  nu.x = n1; nu.y = n2;
-  ((V2<T>*)d.ZB)[bus] = zb;
-  ((V2<T>*)d.NU)[bus] = nu;
+__device__ __forceinline__ void bus_store(const Dev& d, int bus, T n1, T n2, T dw, T dth) {
+  ((V2<T>*)d.ZB)[bus] = V2<T>{dw, dth};
+  ((V2<T>*)d.NU)[bus] = V2<T>{n1, n2};
 }
 
 // bus-side value, multiplier update and residuals of one coupling
@@ -792,77 +799,117 @@ __device__ __forceinline__ void entry_update(const Dev& d, int c, const V4<T>& x
   entry_store(d, c, zn, ln);
 }
 
-// segmented inclusive scan of the six sums by bus id: the last lane of each
-// run of equal ids ends with its bus's totals
-template <typename T>
-__device__ __forceinline__ void seg_scan(int bus, T* S) {
+// segmented inclusive scan of N sums: lane j adds the up lower lanes of its
+// bus, so the last lane of each bus ends with the totals; most (warp-uniform)
+// is the largest up
+template <int N, typename T>
+__device__ __forceinline__ void seg_scan(int up, int most, T* S) {
   const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    T a[6];
+    if (o > most) break;
+    T a[N];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = __shfl_up_sync(FULL, S[k], o);
-    const int bu = __shfl_up_sync(FULL, bus, o);
-    if (lane >= o && bu == bus) {
+    for (int k = 0; k < N; ++k) a[k] = __shfl_up_sync(FULL, S[k], o);
+    if (up >= o) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) S[k] += a[k];
+      for (int k = 0; k < N; ++k) S[k] += a[k];
     }
   }
 }
 
 // seg_scan over two independent tasks at once (their shuffles interleave)
-template <typename T>
-__device__ __forceinline__ void seg_scan2(int bus_a, T* Sa, int bus_b, T* Sb) {
+template <int N, typename T>
+__device__ __forceinline__ void seg_scan2(int up_a, T* Sa, int up_b, T* Sb, int most) {
   const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    T a[6], b[6];
+    if (o > most) break;
+    T a[N], b[N];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < N; ++k) {
       a[k] = __shfl_up_sync(FULL, Sa[k], o);
       b[k] = __shfl_up_sync(FULL, Sb[k], o);
     }
-    const int ua = __shfl_up_sync(FULL, bus_a, o);
-    const int ub = __shfl_up_sync(FULL, bus_b, o);
-    if (lane >= o && ua == bus_a) {
+    if (up_a >= o) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) Sa[k] += a[k];
+      for (int k = 0; k < N; ++k) Sa[k] += a[k];
     }
-    if (lane >= o && ub == bus_b) {
+    if (up_b >= o) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) Sb[k] += b[k];
+      for (int k = 0; k < N; ++k) Sb[k] += b[k];
     }
   }
 }
 
 // What of one task of at most 32 entries stays fixed during a sweep: this
-// lane's slot, whether it is the last lane of its bus, and for that lane the
-// bus's load and shunts
+// lane's slot, the reciprocal of its penalty (FP64), and on the last lane of a
+// bus the bus's load, shunts and constants
 template <typename T>
 struct TaskStatic {
   Slot s;
-  bool last;
-  V4<T> br;
-  int isref;
+  V4<T> br, k;
+  T ir;
 };
 
+// penalty of a slot's coupling
+template <typename T>
+__device__ __forceinline__ T slot_rho(const Dev& d, const Slot& s) {
+  if (s.bus < 0) return T(1);
+  return s.code < 0 ? ((const V4<T>*)d.grec)[d.G - s.code - 1].z : ((const T*)d.trho_l)[s.code >> 1];
+}
+
+// the constants of a task's buses from the penalties: one scan.  The last
+// lane of each bus returns its bus's.  All 32 lanes call it.
+template <typename T>
+__device__ __forceinline__ V4<T> task_const(const Slot& s, const V4<T>& br, T r) {
+  T S[2] = {T(0), T(0)};
+  if (s.bus >= 0) {
+    S[0] = div_w(T(1), r);
+    S[1] = s.code < 0 ? T(0) : r;
+  }
+  seg_scan<2>(s.up(), s.most(), S);
+  return s.last() ? bus_const(br, S[0], S[1]) : V4<T>{T(0), T(0), T(0), T(0)};
+}
+
+template <typename T>
+__device__ __forceinline__ V4<T> task_load_br(const Dev& d, const Slot& s) {
+  return s.last() ? ((const V4<T>*)d.brec)[s.bus] : V4<T>{T(0), T(0), T(0), T(0)};  // pdk qdk gs bs
+}
+
+// the fixed data of a task held in registers for the sweep
 template <typename T>
 __device__ __forceinline__ TaskStatic<T> task_static(const Dev& d, Slot s) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
   TaskStatic<T> a;
   a.s = s;
-  const int bnext = __shfl_down_sync(FULL, s.bus, 1);
-  a.last = s.bus >= 0 && (lane == 31 || bnext != s.bus);
-  a.br = {T(0), T(0), T(0), T(0)};
-  a.isref = 0;
-  if (a.last) {
-    a.br = ((const V4<T>*)d.brec)[s.bus];  // pdk qdk gs bs
-    a.isref = d.isref[s.bus];
-  }
+  const T r = slot_rho<T>(d, s);
+  a.ir = ir_once(r);
+  a.br = task_load_br<T>(d, s);
+  a.k = task_const(s, a.br, r);
   return a;
+}
+
+// the fixed data of a task of the streaming forms: the constants from memory,
+// where task_fresh put them
+template <typename T>
+__device__ __forceinline__ TaskStatic<T> task_stream(const Dev& d, Slot s) {
+  TaskStatic<T> a;
+  a.s = s;
+  a.ir = T(0);
+  a.br = task_load_br<T>(d, s);
+  a.k = s.last() ? ((const V4<T>*)d.bk)[s.bus] : V4<T>{T(0), T(0), T(0), T(0)};
+  return a;
+}
+
+// Streaming forms, in the first iteration of a sweep and after residual
+// balancing has changed penalties: the constants of one task's buses into
+// memory.  A warp takes the same tasks in every iteration, so each lane reads
+// back what it wrote itself.  All 32 lanes call it.
+template <typename T>
+__device__ __noinline__ void task_fresh(const Dev& d, int t, int lane) {
+  const Slot s = load_slot(d, t, lane);
+  const V4<T> k = task_const(s, task_load_br<T>(d, s), slot_rho<T>(d, s));
+  if (s.last()) ((V4<T>*)d.bk)[s.bus] = k;
 }
 
 // the loads of one task: this lane's coupling (lanes of finished instances
@@ -871,25 +918,26 @@ template <typename T>
 struct TaskData {
   Slot s;
   bool last;
-  V4<T> x, lm, zo, br;
-  T r;
-  int isref;
+  V4<T> x, lm, zo, br, k;
+  T r, ir;
 };
 
-template <typename T, bool kDone = true>
+// KEPT: ir comes from the task's fixed data; otherwise it is formed here
+template <typename T, bool kDone, bool KEPT>
 __device__ __forceinline__ TaskData<T> task_load(const Dev& d, const TaskStatic<T>& st, const int* s_done) {
   TaskData<T> a;
   a.s = st.s;
-  a.last = st.last;
+  a.last = st.s.last();
   a.br = st.br;
-  a.isref = st.isref;
-  if (kDone && a.s.bus >= 0 && s_done[a.s.inst]) {
+  a.k = st.k;
+  if (kDone && a.s.inst >= 0 && s_done[a.s.inst]) {
     a.s.bus = a.s.inst = -1;
     a.last = false;
   }
   a.x = a.lm = a.zo = {T(0), T(0), T(0), T(0)};
   a.r = T(1);
   if (a.s.bus >= 0) entry_load(d, a.s.code, a.x, a.lm, a.zo, a.r);
+  a.ir = KEPT ? st.ir : ir_once(a.r);
   return a;
 }
 
@@ -897,21 +945,25 @@ __device__ __forceinline__ TaskData<T> task_load(const Dev& d, const TaskStatic<
 // the two (scan, 2x2 solve, broadcast, update, residual reduction) interleave
 // in one warp.  Tasks never share an entry or a bus, so the order of their
 // stores does not matter.  All 32 lanes call it.
-template <typename T>
+template <typename T, typename Dst>
 __device__ __forceinline__ void bus_task_pair(const Dev& d, const TaskData<T>& a, const TaskData<T>& b,
-                                              const ResDst& dst) {
+                                              const Dst& dst) {
   const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  T Sa[6] = {0, 0, 0, 0, 0, 0}, Sb[6] = {0, 0, 0, 0, 0, 0};
-  const T ira = ir_once(a.r), irb = ir_once(b.r);
-  if (a.s.bus >= 0) entry_sums(a.s.code, a.x, a.lm, a.r, ir_at(a.r, ira), Sa);
-  if (b.s.bus >= 0) entry_sums(b.s.code, b.x, b.lm, b.r, ir_at(b.r, irb), Sb);
-  seg_scan2(a.s.bus, Sa, b.s.bus, Sb);
+  T Sa[4] = {0, 0, 0, 0}, Sb[4] = {0, 0, 0, 0};
+  if (a.s.bus >= 0) entry_sums(a.s.code, a.x, a.lm, a.r, a.ir, Sa);
+  if (b.s.bus >= 0) entry_sums(b.s.code, b.x, b.lm, b.r, b.ir, Sb);
+  const int ma = a.s.most(), mb = b.s.most();
+  seg_scan2<4>(a.s.up(), Sa, b.s.up(), Sb, ma > mb ? ma : mb);
   T n1a = 0, n2a = 0, dwa = 0, dta = 0, n1b = 0, n2b = 0, dwb = 0, dtb = 0;
-  if (a.last) bus_solve(d, a.s.bus, a.br, a.isref, Sa, n1a, n2a, dwa, dta);
-  if (b.last) bus_solve(d, b.s.bus, b.br, b.isref, Sb, n1b, n2b, dwb, dtb);
-  const unsigned ha = __ballot_sync(FULL, a.last) >> lane, hb = __ballot_sync(FULL, b.last) >> lane;
-  const int srca = ha ? lane + __ffs(ha) - 1 : lane, srcb = hb ? lane + __ffs(hb) - 1 : lane;
+  if (a.last) {
+    bus_values(a.br, a.s.ref(), a.k, Sa, n1a, n2a, dwa, dta);
+    bus_store(d, a.s.bus, n1a, n2a, dwa, dta);
+  }
+  if (b.last) {
+    bus_values(b.br, b.s.ref(), b.k, Sb, n1b, n2b, dwb, dtb);
+    bus_store(d, b.s.bus, n1b, n2b, dwb, dtb);
+  }
+  const int srca = a.s.src(), srcb = b.s.src();
   n1a = __shfl_sync(FULL, n1a, srca);
   n1b = __shfl_sync(FULL, n1b, srcb);
   n2a = __shfl_sync(FULL, n2a, srca);
@@ -922,16 +974,16 @@ __device__ __forceinline__ void bus_task_pair(const Dev& d, const TaskData<T>& a
   dtb = __shfl_sync(FULL, dtb, srcb);
   T rma = T(0), sma = T(0), rmb = T(0), smb = T(0);
   if (a.s.bus >= 0) {
-    entry_update(d, a.s.code, a.x, a.lm, a.zo, a.r, ira, n1a, n2a, dwa, dta, rma, sma);
+    entry_update(d, a.s.code, a.x, a.lm, a.zo, a.r, a.ir, n1a, n2a, dwa, dta, rma, sma);
     rma = nan_big(rma);
     sma = nan_big(sma);
   }
   if (b.s.bus >= 0) {
-    entry_update(d, b.s.code, b.x, b.lm, b.zo, b.r, irb, n1b, n2b, dwb, dtb, rmb, smb);
+    entry_update(d, b.s.code, b.x, b.lm, b.zo, b.r, b.ir, n1b, n2b, dwb, dtb, rmb, smb);
     rmb = nan_big(rmb);
     smb = nan_big(smb);
   }
-  res_max2_pair(dst, rma, sma, a.s.inst, rmb, smb, b.s.inst);
+  res_task_pair(dst, rma, sma, a.s.inst, rmb, smb, b.s.inst);
 }
 
 // one task alone in its warp.  The FP64 sweep gives each warp one task where
@@ -939,54 +991,58 @@ __device__ __forceinline__ void bus_task_pair(const Dev& d, const TaskData<T>& a
 // FP32 rate in each SM partition, so two tasks interleaved in one warp take
 // about twice as long as one, where in FP32 they overlap.  The arithmetic is
 // that of task a of bus_task_pair.  All 32 lanes call it.
-template <typename T>
-__device__ __forceinline__ void bus_task_one(const Dev& d, const TaskData<T>& a, const ResDst& dst) {
+template <typename T, typename Dst>
+__device__ __forceinline__ void bus_task_one(const Dev& d, const TaskData<T>& a, const Dst& dst) {
   const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  T S[6] = {0, 0, 0, 0, 0, 0};
-  const T ir = ir_once(a.r);
-  if (a.s.bus >= 0) entry_sums(a.s.code, a.x, a.lm, a.r, ir_at(a.r, ir), S);
-  seg_scan(a.s.bus, S);
+  T S[4] = {0, 0, 0, 0};
+  if (a.s.bus >= 0) entry_sums(a.s.code, a.x, a.lm, a.r, a.ir, S);
+  seg_scan<4>(a.s.up(), a.s.most(), S);
   T n1 = 0, n2 = 0, dw = 0, dt = 0;
-  if (a.last) bus_solve(d, a.s.bus, a.br, a.isref, S, n1, n2, dw, dt);
-  const unsigned h = __ballot_sync(FULL, a.last) >> lane;
-  const int src = h ? lane + __ffs(h) - 1 : lane;
+  if (a.last) {
+    bus_values(a.br, a.s.ref(), a.k, S, n1, n2, dw, dt);
+    bus_store(d, a.s.bus, n1, n2, dw, dt);
+  }
+  const int src = a.s.src();
   n1 = __shfl_sync(FULL, n1, src);
   n2 = __shfl_sync(FULL, n2, src);
   dw = __shfl_sync(FULL, dw, src);
   dt = __shfl_sync(FULL, dt, src);
   T rm = T(0), sm = T(0);
   if (a.s.bus >= 0) {
-    entry_update(d, a.s.code, a.x, a.lm, a.zo, a.r, ir, n1, n2, dw, dt, rm, sm);
+    entry_update(d, a.s.code, a.x, a.lm, a.zo, a.r, a.ir, n1, n2, dw, dt, rm, sm);
     rm = nan_big(rm);
     sm = nan_big(sm);
   }
-  res_max2(dst, rm, sm, a.s.inst);
+  res_task(dst, rm, sm, a.s.inst);
 }
 
 // one bus with more than 32 entries (entries [q0, q1) of ent); lanes loop
-template <typename T, bool kDone = true>
-__device__ void bus_task_big(const SweepP<T>& p, int q0, int q1, const ResDst& dst, const int* s_done) {
+template <typename T, bool kDone, typename Dst>
+__device__ void bus_task_big(const SweepP<T>& p, int q0, int q1, const Dst& dst, const int* s_done) {
   const Dev& d = p.d;
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int bus = d.ebus[q0];
   const int inst = d.bus_inst[bus];
-  if (kDone && s_done[inst]) {
-    res_max2(dst, T(0), T(0), -1);
-    return;
-  }
+  if (kDone && s_done[inst]) return;
   T S[6] = {0, 0, 0, 0, 0, 0};
   for (int q = q0 + lane; q < q1; q += 32) {
     V4<T> x, lm, zo;
     T r;
     const int c = d.ent[q];
     entry_load(d, c, x, lm, zo, r);
-    entry_sums(c, x, lm, r, div_w(T(1), r), S);
+    const T ir = div_w(T(1), r);
+    entry_sums(c, x, lm, r, ir, S);
+    S[4] += ir;
+    if (c >= 0) S[5] += r;
   }
-  seg_scan(bus, S);
+  seg_scan<6>(lane, 31, S);
   T n1 = 0, n2 = 0, dw = 0, dth = 0;
-  if (lane == 31) bus_solve(d, bus, ((const V4<T>*)d.brec)[bus], d.isref[bus], S, n1, n2, dw, dth);
+  if (lane == 31) {
+    const V4<T> br = ((const V4<T>*)d.brec)[bus];
+    bus_values(br, d.isref[bus] != 0, bus_const(br, S[4], S[5]), S, n1, n2, dw, dth);
+    bus_store(d, bus, n1, n2, dw, dth);
+  }
   n1 = __shfl_sync(FULL, n1, 31);
   n2 = __shfl_sync(FULL, n2, 31);
   dw = __shfl_sync(FULL, dw, 31);
@@ -1001,7 +1057,7 @@ __device__ void bus_task_big(const SweepP<T>& p, int q0, int q1, const ResDst& d
   }
   rm = nan_big(rm);
   sm = nan_big(sm);
-  res_max2(dst, rm, sm, inst);
+  res_task(dst, rm, sm, inst);
 }
 
 // RES: every thread has at most one generator or branch and every warp at
@@ -1042,7 +1098,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
   __syncthreads();
   // RES: this thread's phase-A item and its record, this warp's two bus tasks
   const int lane = threadIdx.x & 31, wid = tid >> 5, nw = nthreads >> 5;
-  const Slot none = {-1, 0, -1};
+  const Slot none = empty_slot(lane);
   int my_k = -1;
   V4<T> rr[kRecChunks];
   T my_rho = T(0);
@@ -1068,6 +1124,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     tb = task_static<T>(d, wid + nw < d.NT ? load_slot(d, wid + nw, lane) : none);
   }
   unsigned epoch = 0;  // this CTA's barrier target
+  bool fresh = true;   // streaming: the buses' constants are to be formed (the penalties are new)
   int it = 0;
   bool aborted = false;
   unsigned long long tp0 = 0, tp1 = 0;
@@ -1176,27 +1233,30 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     // all lanes reduce together
     if (RES) {
       if (sizeof(T) == 8 && nw >= d.NT) {  // FP64, one task per warp
-        if (wid < d.NT) bus_task_one(d, task_load<T>(d, ta, s_done), dst);
+        if (wid < d.NT) bus_task_one(d, task_load<T, true, true>(d, ta, s_done), dst);
       } else if (wid < d.NT) {
-        bus_task_pair(d, task_load<T>(d, ta, s_done), task_load<T>(d, tb, s_done), dst);
+        bus_task_pair(d, task_load<T, true, true>(d, ta, s_done), task_load<T, true, true>(d, tb, s_done), dst);
       }
-      for (int b = wid; b < d.NBIG; b += nw) bus_task_big(p, d.big[2 * b], d.big[2 * b + 1], dst, s_done);
     } else {
+      if (fresh)
+        for (int t = wid; t < d.NT; t += nw) task_fresh<T>(d, t, lane);
       auto slot_at = [&](int t) { return t < d.NT ? load_slot(d, t, lane) : none; };
       // tasks wid, wid + nw, ... taken two at a time; the slots of the next
       // pair are in flight while a pair is solved
       Slot s1a = slot_at(wid + 2 * nw), s1b = slot_at(wid + 3 * nw);
-      TaskData<T> ca = task_load<T>(d, task_static<T>(d, slot_at(wid)), s_done);
-      TaskData<T> cb = task_load<T>(d, task_static<T>(d, slot_at(wid + nw)), s_done);
+      TaskData<T> ca = task_load<T, true, false>(d, task_stream<T>(d, slot_at(wid)), s_done);
+      TaskData<T> cb = task_load<T, true, false>(d, task_stream<T>(d, slot_at(wid + nw)), s_done);
       for (int t = wid; t < d.NT; t += 2 * nw) {
         bus_task_pair(d, ca, cb, dst);
-        ca = task_load<T>(d, task_static<T>(d, s1a), s_done);
-        cb = task_load<T>(d, task_static<T>(d, s1b), s_done);
+        ca = task_load<T, true, false>(d, task_stream<T>(d, s1a), s_done);
+        cb = task_load<T, true, false>(d, task_stream<T>(d, s1b), s_done);
         s1a = slot_at(t + 4 * nw);
         s1b = slot_at(t + 5 * nw);
       }
-      for (int b = wid; b < d.NBIG; b += nw) bus_task_big(p, d.big[2 * b], d.big[2 * b + 1], dst, s_done);
     }
+    for (int b = wid; b < d.NBIG; b += nw)
+      bus_task_big<T, true>(p, d.big[2 * b], d.big[2 * b + 1], dst, s_done);
+    fresh = false;
     if (s_acc) {
       __syncthreads();
       res_flush(dst);
@@ -1205,6 +1265,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     if (!grid_barrier(d.bar, epoch, d.err, p.spin_limit)) { aborted = true; break; }
     // residual test (Sec. IV-B) and residual balancing, evaluated identically by every CTA
     const bool rb_now = p.rb_period > 0 && ((it + 1) % p.rb_period) == 0;
+    fresh = rb_now;
     int all = 1;
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
       s_scale[k] = 1.0f;
@@ -1287,6 +1348,59 @@ __device__ __forceinline__ unsigned long long ld_cluster_u64(const void* p, unsi
   return v;
 }
 
+// Where a cluster's residual maxima go: two words of the CTA's shared memory
+// per iteration parity, patterns of the sweep's own type (FP32: 32-bit words,
+// for which shared memory has a native maximum)
+template <typename T>
+struct ClusterRes;
+template <>
+struct ClusterRes<float> {
+  typedef unsigned Word;
+  Word* acc;
+  __device__ __forceinline__ void put(int, float r, float s) const {
+    if (r > 0.f) atomicMax(&acc[0], __float_as_uint(r));
+    if (s > 0.f) atomicMax(&acc[1], __float_as_uint(s));
+  }
+  static __device__ __forceinline__ double value(Word w) { return (double)__uint_as_float(w); }
+};
+template <>
+struct ClusterRes<double> {
+  typedef unsigned long long Word;
+  Word* acc;
+  __device__ __forceinline__ void put(int, double r, double s) const {
+    const unsigned long long br = bits_of(r), bs = bits_of(s);
+    if (br) atomicMax(&acc[0], br);
+    if (bs) atomicMax(&acc[1], bs);
+  }
+  static __device__ __forceinline__ double value(Word w) { return double_of(w); }
+};
+
+// The residual test (Sec. IV-B) on the maxima of all the cluster's CTAs.
+// Every warp reads them for itself and decides alike, so the CTA needs no
+// barrier of its own; res is the CTA's pair of the current parity, which no
+// warp writes again before every warp has passed the next cluster barrier.
+__device__ __forceinline__ void cluster_maxima(const unsigned* res, int cs, double& r, double& s) {
+  unsigned a = 0u, b = 0u;
+  const int lane = threadIdx.x & 31;
+  if (lane < cs) {
+    const unsigned long long v = ld_cluster_u64(res, lane);
+    a = (unsigned)v;
+    b = (unsigned)(v >> 32);
+  }
+  r = (double)__uint_as_float(__reduce_max_sync(0xffffffffu, a));
+  s = (double)__uint_as_float(__reduce_max_sync(0xffffffffu, b));
+}
+__device__ __forceinline__ void cluster_maxima(const unsigned long long* res, int cs, double& r, double& s) {
+  double a = 0.0, b = 0.0;
+  const int lane = threadIdx.x & 31;
+  if (lane < cs) {
+    a = double_of(ld_cluster_u64(&res[0], lane));
+    b = double_of(ld_cluster_u64(&res[1], lane));
+  }
+  r = warp_max(a);
+  s = warp_max(b);
+}
+
 // RES: the cluster has a thread for every generator and branch of its
 // instance and a warp for every two of its bus tasks (checked by the
 // launcher); the records, instance data and task slots are then loaded once
@@ -1298,17 +1412,17 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
   const int K = d.K;
   const int k = (int)cluster_index();
   const int cs = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
-  __shared__ unsigned long long s_res[2][2];  // this CTA's maxima (r, s), by iteration parity
-  __shared__ double s_rs[2];
-  __shared__ int s_stop;
-  if (threadIdx.x < 4) (&s_res[0][0])[threadIdx.x] = 0ull;
+  typedef ClusterRes<T> Res;
+  __shared__ __align__(16) typename Res::Word s_res[2][2];  // this CTA's maxima (r, s), by iteration parity
+  double last_r = 0.0, last_s = 0.0;                        // of the last iteration, over the cluster
+  if (threadIdx.x < 4) (&s_res[0][0])[threadIdx.x] = 0;
   if (d.admm_done[k]) return;  // the whole cluster skips an instance that is not running
   cluster_barrier();  // every CTA has started before any distributed shared memory access
   const int nth = cs * blockDim.x, ct = rank * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31, cw = ct >> 5, nwc = nth >> 5;
   const int g0 = d.gen_off[k], nG = d.gen_off[k + 1] - g0, l0 = d.br_off[k], l1 = d.br_off[k + 1];
   const int t0 = d.task_off[k], t1 = d.task_off[k + 1], b0 = d.big_off[k], b1 = d.big_off[k + 1];
-  const Slot none = {-1, 0, -1};
+  const Slot none = empty_slot(lane);
   const bool prof = p.profile && blockIdx.x == 0 && threadIdx.x == 0;
   // RES: this thread's generator or branch record, this warp's two tasks
   V4<T> rr[kRecChunks];
@@ -1340,7 +1454,7 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
     const int slot = it & 1;
     if (prof) tp0 = gtimer();
     // this parity's maxima were last read before the first barrier of the previous iteration
-    if (threadIdx.x < 2) s_res[slot][threadIdx.x] = 0ull;
+    if (threadIdx.x < 2) s_res[slot][threadIdx.x] = 0;
     // phase A: the instance's generators, then its branches
     if (RES) {
       if (ct < nG) {
@@ -1366,47 +1480,32 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
     cluster_barrier();
     if (prof) { tp0 = gtimer(); atomicAdd(&d.phase_ns[1], tp0 - tp1); }
     // phase B: the instance's bus tasks, two at a time per warp, one in FP64 (warp-uniform loops)
-    const ResDst dst = {&s_res[slot][0], nullptr, 1, slot, k};
+    const Res dst = {&s_res[slot][0]};
     if (RES && sizeof(T) == 8 && nwc >= t1 - t0) {  // FP64, one task per warp
-      bus_task_one(d, task_load<T, false>(d, ta, nullptr), dst);
+      bus_task_one(d, task_load<T, false, true>(d, ta, nullptr), dst);
     } else if (RES) {
-      bus_task_pair(d, task_load<T, false>(d, ta, nullptr), task_load<T, false>(d, tb, nullptr), dst);
+      bus_task_pair(d, task_load<T, false, true>(d, ta, nullptr), task_load<T, false, true>(d, tb, nullptr), dst);
     } else if (sizeof(T) == 8) {
+      if (it == 0)
+        for (int t = t0 + cw; t < t1; t += nwc) task_fresh<T>(d, t, lane);
       for (int t = t0 + cw; t < t1; t += nwc)
-        bus_task_one(d, task_load<T, false>(d, task_static<T>(d, load_slot(d, t, lane)), nullptr), dst);
+        bus_task_one(d, task_load<T, false, false>(d, task_stream<T>(d, load_slot(d, t, lane)), nullptr), dst);
     } else {
+      if (it == 0)
+        for (int t = t0 + cw; t < t1; t += nwc) task_fresh<T>(d, t, lane);
       for (int t = t0 + cw; t < t1; t += 2 * nwc) {
         const Slot sa = load_slot(d, t, lane);
         const Slot sb = t + nwc < t1 ? load_slot(d, t + nwc, lane) : none;
-        bus_task_pair(d, task_load<T, false>(d, task_static<T>(d, sa), nullptr),
-                      task_load<T, false>(d, task_static<T>(d, sb), nullptr), dst);
+        bus_task_pair(d, task_load<T, false, false>(d, task_stream<T>(d, sa), nullptr),
+                      task_load<T, false, false>(d, task_stream<T>(d, sb), nullptr), dst);
       }
     }
     for (int b = b0 + cw; b < b1; b += nwc) bus_task_big<T, false>(p, d.big[2 * b], d.big[2 * b + 1], dst, nullptr);
     if (prof) { tp1 = gtimer(); atomicAdd(&d.phase_ns[2], tp1 - tp0); }
     cluster_barrier();
-    // residual test (Sec. IV-B) on the maxima of all the cluster's CTAs, taken alike by every CTA
-    if (threadIdx.x < 32) {
-      unsigned long long rm = 0ull, sm = 0ull;
-      if (lane < cs) {
-        rm = ld_cluster_u64(&s_res[slot][0], lane);
-        sm = ld_cluster_u64(&s_res[slot][1], lane);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long r2 = __shfl_xor_sync(FULL, rm, o), s2 = __shfl_xor_sync(FULL, sm, o);
-        rm = r2 > rm ? r2 : rm;
-        sm = s2 > sm ? s2 : sm;
-      }
-      if (lane == 0) {
-        s_rs[0] = __longlong_as_double((long long)rm);
-        s_rs[1] = __longlong_as_double((long long)sm);
-        s_stop = p.converged(rm, sm);
-      }
-    }
-    __syncthreads();
+    cluster_maxima(&s_res[slot][0], cs, last_r, last_s);
     if (prof) atomicAdd(&d.phase_ns[3], gtimer() - tp1);
-    if (s_stop) {
+    if (p.converged(bits_of(last_r), bits_of(last_s))) {
       conv = true;
       ++it;
       break;
@@ -1416,8 +1515,8 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
   if (rank == 0 && threadIdx.x == 0) {
     if (conv) d.admm_done[k] = 1;
     d.admm_iters[k] = it;
-    d.admm_rs[k] = it > 0 ? s_rs[0] : 0.0;
-    d.admm_rs[K + k] = it > 0 ? s_rs[1] : 0.0;
+    d.admm_rs[k] = last_r;
+    d.admm_rs[K + k] = last_s;
   }
   cluster_barrier();  // no CTA leaves while another may still read its shared memory
 }
@@ -1455,30 +1554,28 @@ struct DsmLane {
 // Two tasks of one warp: x from this CTA's receive buffers (xa, xb), the bus
 // update of eq. bus_kernel and the multiplier update of eq. multiplier, and
 // the new (z, lambda) pushed to the generator's or branch's CTA.
-template <typename T>
+template <typename T, typename Dst>
 __device__ __forceinline__ void bus_pair_dsm(DsmLane<T>& a, DsmLane<T>& b, const V4<T>& xa, const V4<T>& xb,
-                                             const ResDst& dst, V2<T>& zba, V2<T>& nua, V2<T>& zbb, V2<T>& nub) {
+                                             const Dst& dst, V2<T>& zba, V2<T>& nua, V2<T>& zbb, V2<T>& nub) {
   const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
   const bool ea = a.st.s.bus >= 0, eb = b.st.s.bus >= 0;
-  T Sa[6] = {0, 0, 0, 0, 0, 0}, Sb[6] = {0, 0, 0, 0, 0, 0};
-  const T ira = ir_once(a.r), irb = ir_once(b.r);
-  if (ea) entry_sums(a.st.s.code, xa, a.lm, a.r, ir_at(a.r, ira), Sa);
-  if (eb) entry_sums(b.st.s.code, xb, b.lm, b.r, ir_at(b.r, irb), Sb);
-  seg_scan2(a.st.s.bus, Sa, b.st.s.bus, Sb);
+  T Sa[4] = {0, 0, 0, 0}, Sb[4] = {0, 0, 0, 0};
+  if (ea) entry_sums(a.st.s.code, xa, a.lm, a.r, a.st.ir, Sa);
+  if (eb) entry_sums(b.st.s.code, xb, b.lm, b.r, b.st.ir, Sb);
+  const int ma = a.st.s.most(), mb = b.st.s.most();
+  seg_scan2<4>(a.st.s.up(), Sa, b.st.s.up(), Sb, ma > mb ? ma : mb);
   T n1a = 0, n2a = 0, dwa = 0, dta = 0, n1b = 0, n2b = 0, dwb = 0, dtb = 0;
-  if (a.st.last) {
-    bus_values(a.st.br, a.st.isref, Sa, n1a, n2a, dwa, dta);
+  if (a.st.s.last()) {
+    bus_values(a.st.br, a.st.s.ref(), a.st.k, Sa, n1a, n2a, dwa, dta);
     zba = V2<T>{dwa, dta};
     nua = V2<T>{n1a, n2a};
   }
-  if (b.st.last) {
-    bus_values(b.st.br, b.st.isref, Sb, n1b, n2b, dwb, dtb);
+  if (b.st.s.last()) {
+    bus_values(b.st.br, b.st.s.ref(), b.st.k, Sb, n1b, n2b, dwb, dtb);
     zbb = V2<T>{dwb, dtb};
     nub = V2<T>{n1b, n2b};
   }
-  const unsigned ha = __ballot_sync(FULL, a.st.last) >> lane, hb = __ballot_sync(FULL, b.st.last) >> lane;
-  const int srca = ha ? lane + __ffs(ha) - 1 : lane, srcb = hb ? lane + __ffs(hb) - 1 : lane;
+  const int srca = a.st.s.src(), srcb = b.st.s.src();
   n1a = __shfl_sync(FULL, n1a, srca);
   n1b = __shfl_sync(FULL, n1b, srcb);
   n2a = __shfl_sync(FULL, n2a, srca);
@@ -1490,7 +1587,7 @@ __device__ __forceinline__ void bus_pair_dsm(DsmLane<T>& a, DsmLane<T>& b, const
   T rma = T(0), sma = T(0), rmb = T(0), smb = T(0);
   if (ea) {
     V4<T> zn, ln;
-    entry_values(a.st.s.code, xa, a.lm, a.zo, a.r, ira, n1a, n2a, dwa, dta, rma, sma, zn, ln);
+    entry_values(a.st.s.code, xa, a.lm, a.zo, a.r, a.st.ir, n1a, n2a, dwa, dta, rma, sma, zn, ln);
     st_cluster(a.to, zn);
     st_cluster(a.to + sizeof(V4<T>), ln);
     a.zo = zn;
@@ -1500,7 +1597,7 @@ __device__ __forceinline__ void bus_pair_dsm(DsmLane<T>& a, DsmLane<T>& b, const
   }
   if (eb) {
     V4<T> zn, ln;
-    entry_values(b.st.s.code, xb, b.lm, b.zo, b.r, irb, n1b, n2b, dwb, dtb, rmb, smb, zn, ln);
+    entry_values(b.st.s.code, xb, b.lm, b.zo, b.r, b.st.ir, n1b, n2b, dwb, dtb, rmb, smb, zn, ln);
     st_cluster(b.to, zn);
     st_cluster(b.to + sizeof(V4<T>), ln);
     b.zo = zn;
@@ -1508,7 +1605,7 @@ __device__ __forceinline__ void bus_pair_dsm(DsmLane<T>& a, DsmLane<T>& b, const
     rmb = nan_big(rmb);
     smb = nan_big(smb);
   }
-  res_max2_pair(dst, rma, sma, a.st.s.inst, rmb, smb, b.st.s.inst);
+  res_task(dst, rmax(rma, rmb), rmax(sma, smb), a.st.s.inst);
 }
 
 // The resident cluster form with the exchanged state in shared memory: the
@@ -1529,21 +1626,21 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster_dsm(SweepP<T> p) {
   const int K = d.K;
   const int k = (int)cluster_index();
   const int cs = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
-  __shared__ unsigned long long s_res[2][2];  // this CTA's maxima (r, s), by iteration parity
-  __shared__ double s_rs[2];
-  __shared__ int s_stop;
+  typedef ClusterRes<T> Res;
+  __shared__ __align__(16) typename Res::Word s_res[2][2];  // this CTA's maxima (r, s), by iteration parity
+  double last_r = 0.0, last_s = 0.0;                        // of the last iteration, over the cluster
   extern __shared__ __align__(16) unsigned char s_dyn_c[];
   const int bt = blockDim.x;
   V4<T>* s_zl = (V4<T>*)s_dyn_c;
   V4<T>* s_xin = s_zl + 4 * bt;
   unsigned* s_xcons = (unsigned*)(s_xin + 2 * bt);
-  if (threadIdx.x < 4) (&s_res[0][0])[threadIdx.x] = 0ull;
+  if (threadIdx.x < 4) (&s_res[0][0])[threadIdx.x] = 0;
   if (d.admm_done[k]) return;  // the whole cluster skips an instance that is not running
   const int nth = cs * bt, ct = rank * bt + threadIdx.x;
   const int lane = threadIdx.x & 31, cw = ct >> 5, nwc = nth >> 5;
   const int g0 = d.gen_off[k], nG = d.gen_off[k + 1] - g0, l0 = d.br_off[k], l1 = d.br_off[k + 1];
   const int t0 = d.task_off[k], t1 = d.task_off[k + 1];
-  const Slot none = {-1, 0, -1};
+  const Slot none = empty_slot(lane);
   const bool prof = p.profile && blockIdx.x == 0 && threadIdx.x == 0;
   // this thread's generator or branch, its record, multipliers and (z, lambda)
   const int j = threadIdx.x;
@@ -1607,7 +1704,7 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster_dsm(SweepP<T> p) {
   for (it = 0; it < p.max_iter; ++it) {
     const int slot = it & 1;
     if (prof) tp0 = gtimer();
-    if (threadIdx.x < 2) s_res[slot][threadIdx.x] = 0ull;
+    if (threadIdx.x < 2) s_res[slot][threadIdx.x] = 0;
     // phase A
     if (is_gen) {
       const V4<T> z = s_zl[4 * j], lm = s_zl[4 * j + 1];
@@ -1628,32 +1725,13 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster_dsm(SweepP<T> p) {
     cluster_barrier();
     if (prof) { tp0 = gtimer(); atomicAdd(&d.phase_ns[1], tp0 - tp1); }
     // phase B
-    const ResDst dst = {&s_res[slot][0], nullptr, 1, slot, k};
+    const Res dst = {&s_res[slot][0]};
     bus_pair_dsm(A, B, s_xin[threadIdx.x], s_xin[bt + threadIdx.x], dst, zba, nua, zbb, nub);
     if (prof) { tp1 = gtimer(); atomicAdd(&d.phase_ns[2], tp1 - tp0); }
     cluster_barrier();
-    // residual test (Sec. IV-B) on the maxima of all the cluster's CTAs, taken alike by every CTA
-    if (threadIdx.x < 32) {
-      unsigned long long rm = 0ull, sm = 0ull;
-      if (lane < cs) {
-        rm = ld_cluster_u64(&s_res[slot][0], lane);
-        sm = ld_cluster_u64(&s_res[slot][1], lane);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long r2 = __shfl_xor_sync(FULL, rm, o), s2 = __shfl_xor_sync(FULL, sm, o);
-        rm = r2 > rm ? r2 : rm;
-        sm = s2 > sm ? s2 : sm;
-      }
-      if (lane == 0) {
-        s_rs[0] = __longlong_as_double((long long)rm);
-        s_rs[1] = __longlong_as_double((long long)sm);
-        s_stop = p.converged(rm, sm);
-      }
-    }
-    __syncthreads();
+    cluster_maxima(&s_res[slot][0], cs, last_r, last_s);
     if (prof) atomicAdd(&d.phase_ns[3], gtimer() - tp1);
-    if (s_stop) {
+    if (p.converged(bits_of(last_r), bits_of(last_s))) {
       conv = true;
       ++it;
       break;
@@ -1670,11 +1748,11 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster_dsm(SweepP<T> p) {
     }
     if (A.st.s.bus >= 0) entry_store(d, A.st.s.code, A.zo, A.lm);
     if (B.st.s.bus >= 0) entry_store(d, B.st.s.code, B.zo, B.lm);
-    if (A.st.last) {
+    if (A.st.s.last()) {
       ((V2<T>*)d.ZB)[A.st.s.bus] = zba;
       ((V2<T>*)d.NU)[A.st.s.bus] = nua;
     }
-    if (B.st.last) {
+    if (B.st.s.last()) {
       ((V2<T>*)d.ZB)[B.st.s.bus] = zbb;
       ((V2<T>*)d.NU)[B.st.s.bus] = nub;
     }
@@ -1682,8 +1760,8 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster_dsm(SweepP<T> p) {
   if (rank == 0 && threadIdx.x == 0) {
     if (conv) d.admm_done[k] = 1;
     d.admm_iters[k] = it;
-    d.admm_rs[k] = it > 0 ? s_rs[0] : 0.0;
-    d.admm_rs[K + k] = it > 0 ? s_rs[1] : 0.0;
+    d.admm_rs[k] = last_r;
+    d.admm_rs[K + k] = last_s;
   }
   cluster_barrier();  // no CTA leaves while another may still read its shared memory
 }
