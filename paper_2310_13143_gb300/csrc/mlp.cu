@@ -410,129 +410,245 @@ __global__ void k_splitk(const float* ws, int splits, size_t stride, Epi e) {
 
 // --------------------------------------------------------- other kernels
 // layer-0 input: rows idx[r] of the raw data X (ld = d0), standardised,
-// rounded to bfloat16, stored row-major and transposed; rows >= rows are 0
-__global__ void k_input(const float* X, const int* idx, int rows, int Mb, int d0, const float* mu, const float* sd,
-                        bf16* A, bf16* AT) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)Mb * d0) return;
-  int r = (int)(i / d0), j = (int)(i % d0);
-  float v = 0.0f;
-  if (r < rows) {
-    size_t src = idx ? (size_t)idx[r] : (size_t)r;
-    v = (X[src * d0 + j] - mu[j]) / sd[j];
-  }
-  bf16 h = __float2bfloat16_rn(v);
-  A[i] = h;
-  AT[(size_t)j * Mb + r] = h;
-}
-
-// mean squared error against standardised targets: dY = 2 (Y - T) / (rows * N)
-// in bfloat16, row-major and transposed (32 x 32 tiles transposed through
-// shared memory so both stores coalesce), one sum of squares per block.
-// Grid (ceil(N / 32), Mb / 32), block 32 x 8.
-__global__ void k_mse(const float* Y, const float* T, const int* idx, int rows, int Mb, int N, const float* mu,
-                      const float* sd, bf16* D, bf16* DT, double* part) {
+// rounded to bfloat16, stored row-major and (AT not null) transposed; rows >=
+// rows are 0.  32 x 32 tiles through shared memory, so that both stores
+// coalesce (an element-wise kernel wrote the transpose 2 bytes per sector: 12
+// us for 256 x 4000).  Grid (ceil(d0 / 32), rows of A / 32), block 32 x 8.
+__global__ void __launch_bounds__(256) k_input(const float* X, const int* idx, int rows, int Mb, int d0,
+                                               const float* mu, const float* sd, bf16* A, bf16* AT) {
   __shared__ bf16 tile[32][34];
-  __shared__ double red[256];
-  const int n = blockIdx.x * 32 + threadIdx.x;
-  const int r0 = blockIdx.y * 32;
-  double sq = 0.0;
+  const int j = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 32;
+  const float m = j < d0 ? mu[j] : 0.0f, s = j < d0 ? sd[j] : 1.0f;
+#pragma unroll
   for (int k = threadIdx.y; k < 32; k += 8) {
     const int r = r0 + k;
-    float g = 0.0f;
-    if (n < N && r < rows) {
+    float v = 0.0f;
+    if (j < d0 && r < rows) {
       const size_t src = idx ? (size_t)idx[r] : (size_t)r;
-      const float t = (T[src * N + n] - mu[n]) / sd[n];
-      const float d = Y[(size_t)r * N + n] - t;
-      sq += (double)d * (double)d;
-      g = 2.0f * d / ((float)rows * (float)N);
+      v = (X[src * d0 + j] - m) / s;
     }
-    const bf16 h = __float2bfloat16_rn(g);
-    if (n < N) D[(size_t)r * N + n] = h;
+    const bf16 h = __float2bfloat16_rn(v);
+    if (j < d0) A[(size_t)r * d0 + j] = h;
     tile[k][threadIdx.x] = h;
   }
+  if (!AT) return;
   __syncthreads();
+#pragma unroll
   for (int k = threadIdx.y; k < 32; k += 8) {
-    const int nn = blockIdx.x * 32 + k;
-    if (nn < N) DT[(size_t)nn * Mb + r0 + threadIdx.x] = tile[threadIdx.x][k];
+    const int jj = blockIdx.x * 32 + k;
+    if (jj < d0) AT[(size_t)jj * Mb + r0 + threadIdx.x] = tile[threadIdx.x][k];
   }
-  const int t = threadIdx.y * 32 + threadIdx.x;
-  red[t] = sq;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (t < st) red[t] += red[t + st];
-    __syncthreads();
-  }
-  if (t == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = red[0];
 }
 
-// sum of n partial sums in a fixed order (strided per thread, then a tree);
-// one block of 1024 threads
-__global__ void k_sum(const double* part, int n, double scale, float* out) {
-  __shared__ double red[1024];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-    __syncthreads();
+// Mean squared error against standardised targets: dY = 2 (Y - T) / (rows *
+// N) in bfloat16, row-major and transposed, the output layer's bias gradient
+// (the column sums of dY, in row order) and the loss.
+//
+// One block takes 64 columns over all rows, in tiles of 64 rows transposed
+// through shared memory, each thread two neighbouring columns.  It is bound by
+// its traffic (Y, T, D and D' once: 143 MB for 256 x 46,504).  The squares are
+// accumulated in FP32 pairs (products and sums exact to 2^-48, after Dekker
+// and Knuth) and enter an FP64 sum once per 16 elements: FP64 conversions and
+// additions per element took most of the former kernel's 100 us, and the
+// column sums ran as a kernel of their own (44 us).  Now 47 us for both.  The last block to finish
+// adds the blocks' sums in a fixed order.
+constexpr int kMseCols = 64, kMseRows = 64;
+__global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, const int* idx, int rows, int Mb, int N,
+                                             const float* mu, const float* sd, bf16* D, bf16* DT, float* gb,
+                                             double* part, unsigned* done, float* loss, float* loss_out) {
+  __shared__ __align__(4) bf16 tile[kMseCols][kMseRows + 2];  // [column][row]
+  __shared__ double red[256];
+  __shared__ bool last;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;  // columns n0 + 2 x, + 1; rows y, y + 8, ...
+  const int n0 = blockIdx.x * kMseCols, n = n0 + 2 * x;
+  const bool in = n < N;  // N is a multiple of 8: both columns or none
+  const bool vec = ((uintptr_t)T & 7) == 0;
+  float2 m = make_float2(0.0f, 0.0f), s = make_float2(1.0f, 1.0f);
+  if (in) {
+    m = *(const float2*)(mu + n);
+    s = *(const float2*)(sd + n);
   }
-  if (threadIdx.x == 0) *out = (float)(red[0] * scale);
-}
-
-// column sums of a bfloat16 matrix [rows x N] (bias gradients), fixed order
-__global__ void k_colsum(const bf16* D, int rows, int N, float* out) {
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.0f;
-  for (int r = 0; r < rows; ++r) s += __bfloat162float(D[(size_t)r * N + n]);
-  out[n] = s;
-}
-
-// Adam (bias-corrected) on FP32 master weights W [out x in] with gradient G;
-// writes the bfloat16 copies W16 [out x in] and W16T [in x out] (32 x 32
-// tiles transposed through shared memory)
-__global__ void k_adam_w(float* W, const float* G, float* Mm, float* Vv, int out, int in, float lr, float b1, float b2,
-                         float eps, float c1, float c2, bf16* W16, bf16* W16T) {
-  __shared__ bf16 tile[32][33];
-  int j = blockIdx.x * 32 + threadIdx.x;  // in
-  int i0 = blockIdx.y * 32;               // out
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    int i = i0 + k;
-    bf16 h = __float2bfloat16_rn(0.0f);
-    if (i < out && j < in) {
-      size_t p = (size_t)i * in + j;
-      float g = G[p];
-      float m = b1 * Mm[p] + (1.0f - b1) * g;
-      float v = b2 * Vv[p] + (1.0f - b2) * g * g;
-      Mm[p] = m;
-      Vv[p] = v;
-      float w = W[p] - lr * (m / c1) / (sqrtf(v / c2) + eps);
-      W[p] = w;
-      h = __float2bfloat16_rn(w);
-      W16[p] = h;
+  const float den = (float)rows * (float)N;
+  double sq = 0.0;
+  float col = 0.0f;  // threads 0..63: the sum of column n0 + threadIdx.x
+  for (int r0 = 0; r0 < Mb; r0 += kMseRows) {
+    float hs = 0.0f, ls = 0.0f;  // the squares of this tile, as a sum of two floats
+    auto add = [&](float d) {
+      const float pr = d * d, pe = fmaf(d, d, -pr);
+      const float t = hs + pr, z = t - hs;
+      ls += ((hs - (t - z)) + (pr - z)) + pe;
+      hs = t;
+    };
+#pragma unroll
+    for (int k = 0; k < kMseRows; k += 8) {
+      const int r = r0 + y + k;
+      float2 g = make_float2(0.0f, 0.0f);
+      if (in && r < rows) {
+        const size_t src = idx ? (size_t)idx[r] : (size_t)r;
+        const float* tp = T + src * N + n;
+        const float2 t = vec ? *(const float2*)tp : make_float2(tp[0], tp[1]);
+        const float2 yv = *(const float2*)(Y + (size_t)r * N + n);
+        const float d0 = yv.x - (t.x - m.x) / s.x, d1 = yv.y - (t.y - m.y) / s.y;
+        add(d0);
+        add(d1);
+        g = make_float2(2.0f * d0 / den, 2.0f * d1 / den);
+      }
+      const __nv_bfloat162 h = __floats2bfloat162_rn(g.x, g.y);
+      if (in) *(__nv_bfloat162*)(D + (size_t)r * N + n) = h;
+      tile[2 * x][y + k] = h.x;
+      tile[2 * x + 1][y + k] = h.y;
     }
-    tile[k][threadIdx.x] = h;
+    sq += (double)hs + (double)ls;
+    __syncthreads();
+    for (int c = y; c < kMseCols && n0 + c < N; c += 8)
+      *(__nv_bfloat162*)(DT + (size_t)(n0 + c) * Mb + r0 + 2 * x) = *(const __nv_bfloat162*)&tile[c][2 * x];
+    if (threadIdx.x < kMseCols) {
+#pragma unroll 8
+      for (int r = 0; r < kMseRows; ++r) col += __bfloat162float(tile[threadIdx.x][r]);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < kMseCols && n0 + (int)threadIdx.x < N) gb[n0 + threadIdx.x] = col;
+  auto sum = [&](double v) {
+    red[threadIdx.x] = v;
+    __syncthreads();
+    for (int st = 128; st > 0; st >>= 1) {
+      if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+      __syncthreads();
+    }
+    return red[0];
+  };
+  const double mine = sum(sq);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = mine;
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  int i = i0 + threadIdx.x;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    int jj = blockIdx.x * 32 + k;
-    if (i < out && jj < in) W16T[(size_t)jj * out + i] = tile[threadIdx.x][k];
+  if (!last) return;
+  __threadfence();
+  double t = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) t += ((volatile double*)part)[i];
+  const double total = sum(t);
+  if (threadIdx.x == 0) {
+    const float v = (float)(total * (1.0 / ((double)rows * N)));
+    *loss = v;
+    if (loss_out) *loss_out = v;
+    *done = 0u;  // for the next launch
   }
 }
 
-__global__ void k_adam_b(float* b, const float* G, float* Mm, float* Vv, int n, float lr, float b1, float b2, float eps,
-                         float c1, float c2) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float g = G[i];
-  float m = b1 * Mm[i] + (1.0f - b1) * g;
-  float v = b2 * Vv[i] + (1.0f - b2) * g * g;
-  Mm[i] = m;
-  Vv[i] = v;
-  b[i] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+// Adam (bias-corrected) on every parameter of the network in one launch: FP32
+// master weights W [out x in] with gradient G, the bfloat16 copies W16 [out x
+// in] and W16T [in x out], and the biases, whose gradients of the hidden
+// layers (the column sums of D, in row order) are formed here from D'.
+//
+// A weight block takes a 64 x 64 tile in 16-byte accesses, sixteen loads in
+// flight per thread, and transposes the bfloat16 copy through shared memory.
+// Bound by its traffic, 32 bytes per parameter: the 26.4 M parameters of the
+// 2,000-bus network take 132 us against 220 with 4-byte accesses
+// and one launch per layer (845 MB: 124 us at 6.8 TB/s).
+constexpr int kMaxLayers = 16;
+constexpr int kAdamTile = 64, kAdamBias = 64;  // tile edge; biases per block
+struct AdamLayer {
+  float *W, *G, *mW, *vW, *b, *gb, *mb, *vb;
+  bf16 *W16, *W16T;
+  const bf16* DT;  // hidden layers: D' [out x rows], null where gb is already formed
+  int in, out;
+  int block0, bias0;  // first weight block, first bias block
+};
+struct AdamP {
+  AdamLayer l[kMaxLayers];
+  int nl, rows;
+  float lr, b1, b2, eps, c1, c2;
+};
+// the moments with the roundings written out, so that every instance of this
+// function rounds alike
+__device__ __forceinline__ float adam_one(const AdamP& p, float g, float& m, float& v, float w) {
+  m = fmaf(1.0f - p.b1, g, __fmul_rn(p.b1, m));
+  v = fmaf(__fmul_rn(1.0f - p.b2, g), g, __fmul_rn(p.b2, v));
+  return w - p.lr * (m / p.c1) / (sqrtf(v / p.c2) + p.eps);
+}
+__global__ void __launch_bounds__(256) k_adam(const __grid_constant__ AdamP p) {
+  __shared__ __align__(4) bf16 tile[kAdamTile][kAdamTile + 2];
+  const int blk = blockIdx.x, t = threadIdx.x;
+  if (blk >= p.l[0].bias0) {
+    int q = p.nl - 1;
+    while (q > 0 && blk < p.l[q].bias0) --q;
+    const AdamLayer& y = p.l[q];
+    const int i = (blk - y.bias0) * kAdamBias + t;
+    if (t >= kAdamBias || i >= y.out) return;
+    float g = 0.0f;
+    if (y.DT) {
+      const uint4* src = (const uint4*)(y.DT + (size_t)i * p.rows);  // rows is a multiple of 128
+#pragma unroll 8
+      for (int k = 0; k < p.rows / 8; ++k) {
+        const uint4 u = src[k];
+        const unsigned w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          g += __uint_as_float(w[h] << 16);
+          g += __uint_as_float(w[h] & 0xffff0000u);
+        }
+      }
+      y.gb[i] = g;
+    } else {
+      g = y.gb[i];
+    }
+    float m = y.mb[i], v = y.vb[i];
+    y.b[i] = adam_one(p, g, m, v, y.b[i]);
+    y.mb[i] = m;
+    y.vb[i] = v;
+    return;
+  }
+  int q = p.nl - 1;
+  while (q > 0 && blk < p.l[q].block0) --q;
+  const AdamLayer& y = p.l[q];
+  const int nti = (y.in + kAdamTile - 1) / kAdamTile;
+  const int i0 = (blk - y.block0) / nti * kAdamTile, j0 = (blk - y.block0) % nti * kAdamTile;
+  const int jc = (t & 15) * 4, j = j0 + jc;  // in is a multiple of 8: four columns or none
+  float4 W[4], G[4], M[4], V[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int i = i0 + (t >> 4) + 16 * k;
+    if (i < y.out && j < y.in) {
+      const size_t at = (size_t)i * y.in + j;
+      W[k] = *(const float4*)(y.W + at);
+      G[k] = *(const float4*)(y.G + at);
+      M[k] = *(const float4*)(y.mW + at);
+      V[k] = *(const float4*)(y.vW + at);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int r = (t >> 4) + 16 * k, i = i0 + r;
+    if (i < y.out && j < y.in) {
+      const size_t at = (size_t)i * y.in + j;
+      W[k].x = adam_one(p, G[k].x, M[k].x, V[k].x, W[k].x);
+      W[k].y = adam_one(p, G[k].y, M[k].y, V[k].y, W[k].y);
+      W[k].z = adam_one(p, G[k].z, M[k].z, V[k].z, W[k].z);
+      W[k].w = adam_one(p, G[k].w, M[k].w, V[k].w, W[k].w);
+      *(float4*)(y.mW + at) = M[k];
+      *(float4*)(y.vW + at) = V[k];
+      *(float4*)(y.W + at) = W[k];
+      __nv_bfloat162 h[2] = {__floats2bfloat162_rn(W[k].x, W[k].y), __floats2bfloat162_rn(W[k].z, W[k].w)};
+      *(uint2*)(y.W16 + at) = *(const uint2*)h;
+      *(__nv_bfloat162*)&tile[r][jc] = h[0];
+      *(__nv_bfloat162*)&tile[r][jc + 2] = h[1];
+    }
+  }
+  __syncthreads();
+  // W16T: two neighbouring outputs per lane (out is a multiple of 8)
+  const int x = t & 31, i = i0 + 2 * x;
+  if (i >= y.out) return;
+#pragma unroll
+  for (int k = t >> 5; k < kAdamTile; k += 8) {
+    if (j0 + k >= y.in) break;
+    __nv_bfloat162 h;
+    h.x = tile[2 * x][k];
+    h.y = tile[2 * x + 1][k];
+    *(__nv_bfloat162*)(y.W16T + (size_t)(j0 + k) * y.out + i) = h;
+  }
 }
 
 // de-standardised network outputs: out = y sd + mu (y row-major, N columns)
@@ -669,6 +785,7 @@ struct Net {
   size_t ws_elems = 0;
   double* part = nullptr;
   int nparts = 0;
+  unsigned* done = nullptr;  // blocks of k_mse that have finished (0 between launches)
   int* err = nullptr;
   float* loss = nullptr;
   int step = 0;
@@ -833,8 +950,8 @@ acopf_status acopf_mlp_create(const int32_t* dims, int32_t nlayers, int32_t max_
        dalloc(n, &n->sd_x, dims[0]) && dalloc(n, &n->mu_y, dims[nlayers]) && dalloc(n, &n->sd_y, dims[nlayers]) &&
        dalloc(n, &n->err, 1) && dalloc(n, &n->loss, 1);
   if (ok) {
-    n->nparts = (int)(((size_t)dims[nlayers] + 31) / 32 * ((size_t)Mb / 32));
-    ok = dalloc(n, &n->part, n->nparts);
+    n->nparts = (dims[nlayers] + kMseCols - 1) / kMseCols;
+    ok = dalloc(n, &n->part, n->nparts) && dalloc(n, &n->done, 1);
   }
   if (ok) {
     // identity standardisation until fitted
@@ -971,9 +1088,8 @@ acopf_status acopf_mlp_forward(acopf_mlp_handle h, const float* X, int32_t rows,
   const int d0 = n->dims[0], dn = n->dims[n->nl];
   for (int r0 = 0; r0 < rows; r0 += n->Mb) {
     int rr = rows - r0 < n->Mb ? rows - r0 : n->Mb;
-    size_t tot = (size_t)n->Mb * d0;
-    k_input<<<(unsigned)((tot + 255) / 256), 256, 0, n->stream>>>(X + (size_t)r0 * d0, nullptr, rr, n->Mb, d0,
-                                                                   n->mu_x, n->sd_x, n->A[0], n->AT[0]);
+    k_input<<<dim3((d0 + 31) / 32, n->Mb / 32), dim3(32, 8), 0, n->stream>>>(X + (size_t)r0 * d0, nullptr, rr, n->Mb,
+                                                                             d0, n->mu_x, n->sd_x, n->A[0], nullptr);
     NCK(cudaGetLastError());
     acopf_status s = forward(n, rr);
     if (s) return s;
@@ -991,34 +1107,39 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
   if (!n || !X || !T || rows < 1 || rows > n->Mb || !(lr > 0)) return nfail(n, ACOPF_EINVAL, "mlp_train_step: bad arguments");
   cudaSetDevice(n->device);
   const int nl = n->nl, Mb = n->Mb, d0 = n->dims[0], dn = n->dims[nl];
-  size_t tot = (size_t)Mb * d0;
-  k_input<<<(unsigned)((tot + 255) / 256), 256, 0, n->stream>>>(X, idx, rows, Mb, d0, n->mu_x, n->sd_x, n->A[0],
-                                                                 n->AT[0]);
+  k_input<<<dim3((d0 + 31) / 32, Mb / 32), dim3(32, 8), 0, n->stream>>>(X, idx, rows, Mb, d0, n->mu_x, n->sd_x,
+                                                                        n->A[0], n->AT[0]);
   NCK(cudaGetLastError());
   acopf_status s = forward(n, rows);
   if (s) return s;
-  dim3 mgrid((dn + 31) / 32, Mb / 32);
-  k_mse<<<mgrid, dim3(32, 8), 0, n->stream>>>(n->Y, T, idx, rows, Mb, dn, n->mu_y, n->sd_y, n->D[nl], n->DT[nl],
-                                              n->part);
-  k_sum<<<1, 1024, 0, n->stream>>>(n->part, (int)(mgrid.x * mgrid.y), 1.0 / ((double)rows * dn), n->loss);
+  k_mse<<<n->nparts, 256, 0, n->stream>>>(n->Y, T, idx, rows, Mb, dn, n->mu_y, n->sd_y, n->D[nl], n->DT[nl],
+                                          n->L[nl - 1].gb, n->part, n->done, n->loss, loss);
   NCK(cudaGetLastError());
   for (int l = nl - 1; l >= 0; --l) {
     NCK(run_gemm(n->bwd_w[l], n->ws, n->err, n->stream, n->spin, n->sms));
-    k_colsum<<<(n->dims[l + 1] + 127) / 128, 128, 0, n->stream>>>(n->D[l + 1], Mb, n->dims[l + 1], n->L[l].gb);
-    NCK(cudaGetLastError());
     if (l >= 1) NCK(run_gemm(n->bwd_x[l], n->ws, n->err, n->stream, n->spin, n->sms));
   }
   n->step += 1;
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float c1 = (float)(1.0 - pow(0.9, n->step)), c2 = (float)(1.0 - pow(0.999, n->step));
-  for (auto& y : n->L) {
-    dim3 grid((y.in + 31) / 32, (y.out + 31) / 32);
-    k_adam_w<<<grid, dim3(32, 8), 0, n->stream>>>(y.W, y.gW, y.mW, y.vW, y.out, y.in, lr, b1, b2, eps, c1, c2, y.W16,
-                                                    y.W16T);
-    k_adam_b<<<(y.out + 255) / 256, 256, 0, n->stream>>>(y.b, y.gb, y.mb, y.vb, y.out, lr, b1, b2, eps, c1, c2);
+  AdamP p;
+  p.nl = nl;
+  p.rows = Mb;
+  p.lr = lr; p.b1 = 0.9f; p.b2 = 0.999f; p.eps = 1e-8f;
+  p.c1 = (float)(1.0 - pow(0.9, n->step));
+  p.c2 = (float)(1.0 - pow(0.999, n->step));
+  int blocks = 0;
+  auto tiles = [](int w) { return (w + kAdamTile - 1) / kAdamTile; };
+  for (int l = 0; l < nl; ++l) {
+    const Layer& y = n->L[l];
+    p.l[l] = AdamLayer{y.W, y.gW, y.mW, y.vW, y.b, y.gb, y.mb, y.vb, y.W16, y.W16T,
+                       l < nl - 1 ? n->DT[l + 1] : nullptr, y.in, y.out, blocks, 0};
+    blocks += tiles(y.in) * tiles(y.out);
   }
+  for (int l = 0; l < nl; ++l) {
+    p.l[l].bias0 = blocks;
+    blocks += (n->L[l].out + kAdamBias - 1) / kAdamBias;
+  }
+  k_adam<<<blocks, 256, 0, n->stream>>>(p);
   NCK(cudaGetLastError());
-  if (loss) NCK(cudaMemcpyAsync(loss, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, n->stream));
   return ACOPF_OK;
 }
 
