@@ -7,16 +7,18 @@
 //
 //   C[M x N] = A[M x K] * B[N x K]^T,   A, B bfloat16, K contiguous,
 //
-// with 128 x 256 output tiles in a persistent, warp-specialised kernel: one
+// with 128 x 128 to 128 x 256 output tiles in a persistent, warp-specialised kernel: one
 // CTA per SM loops over tiles; warp 0 streams 128 x 64 and 256 x 64 operand
 // tiles into a four-stage shared-memory ring with TMA (cp.async.bulk.tensor,
 // 128-byte swizzle, completion counted on mbarriers); warp 1 issues
 // tcgen05.mma (kind::f16, BF16 x BF16 -> FP32, 128 x 256 x 16) into one of two
 // 256-column tensor-memory accumulators; warps 2-5 read the other accumulator
 // back with tcgen05.ld for a fused epilogue (bias, GELU, GELU derivative,
-// bfloat16 row-major and transposed stores), so the epilogue of one tile
-// overlaps the main loop of the next.  Long contractions are split over K
-// into FP32 partial tiles summed by k_splitk.
+// bfloat16 row-major and transposed stores, de-standardised outputs), so the
+// epilogue of one tile overlaps the main loop of the next.  Long contractions
+// are split over K: products with few output tiles run as k_gemm_small, 128 x
+// 64 tiles whose CTA keeps every split in an accumulator of its own; the rest
+// write FP32 partial tiles summed by k_splitk.
 //
 // Layout convention: the backward pass needs every operand with its
 // contraction index contiguous, so the forward epilogue stores each hidden
@@ -43,18 +45,24 @@ namespace nn {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
+constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;  // BN: widest tile of k_gemm_tc (tile_width)
 constexpr uint32_t kABytes = BM * BK * 2;  // A tile: 128 rows x 128 bytes
 constexpr uint32_t kBBytes = BN * BK * 2;  // B tile: 256 rows x 128 bytes
 constexpr int kGemmThreads = 192;          // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
+constexpr int kScratch = 32 * 33;          // floats of epilogue scratch per warp: one 32 x 32 block
 constexpr size_t kGemmSmem = 1024 + (size_t)STAGES * (kABytes + kBBytes) + 256;
 constexpr uint32_t kTmemCols = 512;        // two 256-column FP32 accumulators
+
+// k_gemm_small
+constexpr int SN = 64, kSmallStages = 6, kSmallThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
+constexpr uint32_t kSBytes = SN * BK * 2;
+constexpr size_t kSmallSmem = 1024 + (size_t)kSmallStages * (kABytes + kSBytes) + 256;
+constexpr int kSmallSplits = 512 / SN;  // accumulators that tensor memory holds
 
 // Instruction descriptor of tcgen05.mma kind::f16: D in FP32 (bits 4-5 = 1),
 // A and B bfloat16 (bits 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0),
 // N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                            ((uint32_t)(BM >> 4) << 24);
+constexpr uint32_t kIdescM = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
 
 enum { EPI_F32 = 0, EPI_GELU = 1, EPI_GELU_BWD = 2, EPI_PARTIAL = 3 };
 
@@ -63,15 +71,16 @@ struct Epi {
   int M, N;             // output extent
   int rows_valid;       // bf16 outputs of rows >= rows_valid are written as 0
   const float* bias;    // [N] or null
-  float* f32;           // FP32 row-major output (EPI_F32, EPI_PARTIAL; EPI_GELU: the pre-activation)
+  float* f32;           // FP32 row-major output (EPI_F32, EPI_PARTIAL; EPI_GELU: the pre-activation, or null)
   int ld_f32;
   size_t split_stride;  // EPI_PARTIAL: elements between the partial tiles of consecutive K splits
   bf16* bf;             // bfloat16 row-major output
   int ld_bf;
-  bf16* bt;             // bfloat16 transposed output: (m, n) at bt[n * ld_bt + m]
+  bf16* bt;             // bfloat16 transposed output: (m, n) at bt[n * ld_bt + m] (EPI_GELU: or null)
   int ld_bt;
   const float* z;       // EPI_GELU_BWD: saved pre-activation
   int ld_z;
+  const float *mu, *sd; // EPI_F32: not null: outputs de-standardised, y sd + mu (inference)
 };
 
 // --------------------------------------------------------------- PTX helpers
@@ -117,11 +126,12 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
   d |= (uint64_t)2 << 61;
   return d;
 }
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+__device__ __forceinline__ uint32_t idesc(int n) { return kIdescM | ((uint32_t)(n >> 3) << 17); }
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate));
+      "l"(a), "l"(b), "r"(id), "r"(accumulate));
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
@@ -130,18 +140,20 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 16 consecutive FP32 accumulator columns of this thread's lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
-  uint32_t r[16];
+// 32 consecutive FP32 accumulator columns of this thread's lane
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
+  uint32_t r[32];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // ------------------------------------------------------------------ epilogue
@@ -150,31 +162,31 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
 
-__device__ __forceinline__ void epi_one(const Epi& e, int m, int n, float acc, int split) {
-  if (m >= e.M || n >= e.N) return;
+// one element, after the K-split partial tiles have been summed
+__device__ __forceinline__ void epi_one(const Epi& e, int m, int n, float acc) {
   switch (e.op) {
     case EPI_F32: {
-      e.f32[(size_t)m * e.ld_f32 + n] = acc + (e.bias ? e.bias[n] : 0.0f);
+      float y = acc;
+      if (e.bias) y += e.bias[n];
+      if (e.sd) y = fmaf(y, e.sd[n], e.mu[n]);
+      e.f32[(size_t)m * e.ld_f32 + n] = y;
       break;
     }
     case EPI_GELU: {
-      float zz = acc + e.bias[n];
-      e.f32[(size_t)m * e.ld_f32 + n] = zz;
-      bf16 h = __float2bfloat16_rn(m < e.rows_valid ? gelu_f(zz) : 0.0f);
+      const float zz = acc + e.bias[n];
+      if (e.f32) e.f32[(size_t)m * e.ld_f32 + n] = zz;
+      const bf16 h = __float2bfloat16_rn(m < e.rows_valid ? gelu_f(zz) : 0.0f);
+      e.bf[(size_t)m * e.ld_bf + n] = h;
+      if (e.bt) e.bt[(size_t)n * e.ld_bt + m] = h;
+      break;
+    }
+    default: {  // EPI_GELU_BWD
+      const float v = m < e.rows_valid ? acc * gelu_grad_f(e.z[(size_t)m * e.ld_z + n]) : 0.0f;
+      const bf16 h = __float2bfloat16_rn(v);
       e.bf[(size_t)m * e.ld_bf + n] = h;
       e.bt[(size_t)n * e.ld_bt + m] = h;
       break;
     }
-    case EPI_GELU_BWD: {
-      float v = m < e.rows_valid ? acc * gelu_grad_f(e.z[(size_t)m * e.ld_z + n]) : 0.0f;
-      bf16 h = __float2bfloat16_rn(v);
-      e.bf[(size_t)m * e.ld_bf + n] = h;
-      e.bt[(size_t)n * e.ld_bt + m] = h;
-      break;
-    }
-    default:  // EPI_PARTIAL
-      e.f32[(size_t)split * e.split_stride + (size_t)m * e.ld_f32 + n] = acc;
-      break;
   }
 }
 
@@ -182,62 +194,126 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(b)) : "memory");
 }
 
-// 16 consecutive accumulator columns [n, n + 16) of row m: vector stores when
-// the whole group is in range, the per-element epilogue otherwise
-__device__ __forceinline__ void epi_store16(const Epi& e, int m, int n, const float v[16], int split) {
-  if (m >= e.M) return;
-  if (n + 16 > e.N) {
+// EPI_F32: bias, deviation and mean of output columns n0 .. n0 + n - 1 into a
+// warp's part of shared memory (stride floats each), fetched before the
+// accumulator is waited for.  All 32 lanes call it.
+__device__ __forceinline__ void epi_consts(const Epi& e, int n0, int n, float* cst, int stride) {
+  if (e.op != EPI_F32) return;
+  __syncwarp();
+  for (int j = threadIdx.x & 31; j < n && n0 + j < e.N; j += 32) {
+    if (e.bias) cst[j] = e.bias[n0 + j];
+    if (e.sd) {
+      cst[stride + j] = e.sd[n0 + j];
+      cst[2 * stride + j] = e.mu[n0 + j];
+    }
+  }
+  __syncwarp();
+}
+
+// One warp's 32 x 32 block of the accumulator: lane holds row m0 + lane,
+// columns n0 .. n0 + 31.  FP32 outputs are stored from the lanes, 16 bytes of
+// a row at a time (through shared memory, in whole rows, the 46,504 x 512
+// weight gradient took 49 us against 37).  Pre-activations and row-major
+// bfloat16 go through the warp's scratch in shared memory; transposed outputs
+// come straight from the lanes, which hold consecutive rows.  A block is read
+// back into registers as a whole before it is stored (and a pre-activation
+// block read as a whole before it goes to the scratch): the compiler cannot
+// move a load past a store that may alias it, and one load per store would pay
+// its latency 32 times.  cst: what epi_consts put into shared memory for these
+// columns.  All 32 lanes call it.
+__device__ __forceinline__ void epi_block(const Epi& e, int m0, int n0, float v[32], int split, float* scratch,
+                                          const float* cst, int stride) {
+  const int lane = threadIdx.x & 31;
+  const int m = m0 + lane, n = n0 + lane;
+  const int rows = e.M - m0 < 32 ? e.M - m0 : 32;  // rows of the block that exist (may be <= 0)
+  if (e.op == EPI_F32 || e.op == EPI_PARTIAL) {
+    if (lane >= rows) return;
+    float* dst = e.f32 + (e.op == EPI_PARTIAL ? (size_t)split * e.split_stride : 0) + (size_t)m * e.ld_f32 + n0;
+    if (n0 + 32 <= e.N && ((uintptr_t)dst & 15) == 0) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) epi_one(e, m, n + j, v[j], split);
+      for (int j = 0; j < 32; j += 4) {
+        float4 y = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        if (e.op == EPI_F32 && e.bias) {
+          const float4 q = *(const float4*)(cst + j);
+          y.x += q.x; y.y += q.y; y.z += q.z; y.w += q.w;
+        }
+        if (e.op == EPI_F32 && e.sd) {
+          const float4 q = *(const float4*)(cst + stride + j), u = *(const float4*)(cst + 2 * stride + j);
+          y.x = fmaf(y.x, q.x, u.x); y.y = fmaf(y.y, q.y, u.y); y.z = fmaf(y.z, q.z, u.z); y.w = fmaf(y.w, q.w, u.w);
+        }
+        *(float4*)(dst + j) = y;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (n0 + j < e.N) {
+          float y = v[j];
+          if (e.op == EPI_F32 && e.bias) y += cst[j];
+          if (e.op == EPI_F32 && e.sd) y = fmaf(y, cst[stride + j], cst[2 * stride + j]);
+          dst[j] = y;
+        }
+    }
     return;
   }
-  switch (e.op) {
-    case EPI_F32:
-    case EPI_PARTIAL: {
-      float* dst = e.op == EPI_PARTIAL ? e.f32 + (size_t)split * e.split_stride + (size_t)m * e.ld_f32 + n
-                                       : e.f32 + (size_t)m * e.ld_f32 + n;
-      float w[16];
+  uint32_t h[16];  // the block's rows in bfloat16, two columns per word
+  if (e.op == EPI_GELU) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        w[j] = v[j] + (e.op == EPI_F32 && e.bias ? e.bias[n + j] : 0.0f);
+    for (int j = 0; j < 32; ++j) v[j] += n0 + j < e.N ? e.bias[n0 + j] : 0.0f;
+    if (e.f32) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) scratch[lane * 33 + j] = v[j];
+      __syncwarp();
+      float t[32];
+#pragma unroll
+      for (int r = 0; r < 32; ++r) t[r] = scratch[r * 33 + lane];
+      __syncwarp();
+      if (n < e.N) {
+        float* dst = e.f32 + (size_t)m0 * e.ld_f32 + n;
+#pragma unroll
+        for (int r = 0; r < 32; ++r)
+          if (r < rows) dst[(size_t)r * e.ld_f32] = t[r];
       }
-      if (((uintptr_t)dst & 15) == 0) {
-#pragma unroll
-        for (int j = 0; j < 16; j += 4) *(float4*)(dst + j) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) dst[j] = w[j];
-      }
-      break;
     }
-    case EPI_GELU:
-    case EPI_GELU_BWD: {
-      bf16 h[16];
-      if (e.op == EPI_GELU) {
-        float* zd = e.f32 + (size_t)m * e.ld_f32 + n;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float zz = v[j] + e.bias[n + j];
-          zd[j] = zz;
-          h[j] = __float2bfloat16_rn(m < e.rows_valid ? gelu_f(zz) : 0.0f);
-        }
-      } else {
-        const float* zs = e.z + (size_t)m * e.ld_z + n;
+    for (int j = 0; j < 32; ++j) v[j] = m < e.rows_valid ? gelu_f(v[j]) : 0.0f;
+  } else {  // EPI_GELU_BWD: the saved pre-activations, read in rows
+    float t[32];
+    const float* src = e.z + (size_t)m0 * e.ld_z + n;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) h[j] = __float2bfloat16_rn(m < e.rows_valid ? v[j] * gelu_grad_f(zs[j]) : 0.0f);
-      }
-      bf16* dst = e.bf + (size_t)m * e.ld_bf + n;
-      if (((uintptr_t)dst & 15) == 0) {
-        *(uint4*)dst = *(const uint4*)&h[0];
-        *(uint4*)(dst + 8) = *(const uint4*)&h[8];
-      } else {
+    for (int r = 0; r < 32; ++r) t[r] = r < rows && n < e.N ? src[(size_t)r * e.ld_z] : 0.0f;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) dst[j] = h[j];
-      }
-      // transposed: lanes hold consecutive rows, so each column's stores coalesce
+    for (int r = 0; r < 32; ++r) scratch[r * 33 + lane] = t[r];
+    __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) e.bt[(size_t)(n + j) * e.ld_bt + m] = h[j];
-      break;
+    for (int j = 0; j < 32; ++j)
+      v[j] = m < e.rows_valid && n0 + j < e.N ? v[j] * gelu_grad_f(scratch[lane * 33 + j]) : 0.0f;
+    __syncwarp();
+  }
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const __nv_bfloat162 w = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    h[j] = *(const uint32_t*)&w;
+  }
+  if (e.bt && lane < rows) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (n0 + j < e.N)
+        e.bt[(size_t)(n0 + j) * e.ld_bt + m] = __ushort_as_bfloat16((unsigned short)(h[j >> 1] >> (16 * (j & 1))));
+  }
+  // row-major bfloat16 (N and ld_bf are multiples of 8): two rows per store instruction
+  uint32_t* sw = (uint32_t*)scratch;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) sw[lane * 17 + j] = h[j];
+  __syncwarp();
+  const int w = lane & 15;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) h[i] = sw[(2 * i + (lane >> 4)) * 17 + w];
+  __syncwarp();
+  if (n0 + 2 * w < e.N) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int r = 2 * i + (lane >> 4);
+      if (r < rows) *(uint32_t*)(e.bf + (size_t)(m0 + r) * e.ld_bf + n0 + 2 * w) = h[i];
     }
   }
 }
@@ -264,19 +340,21 @@ __device__ __forceinline__ void decode_item(int w, int mt, int nt, int& z, int& 
 // on time-out the waiting role records *err and stops.
 __global__ void __launch_bounds__(kGemmThreads, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int K, int kts,
-              int splits, Epi e, int* err, long long spin) {
+              int splits, int bn, Epi e, int* err, long long spin) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
   uint8_t* sB = smem + STAGES * kABytes;
+  __shared__ __align__(16) float scratch[4][kScratch];
   uint64_t* full = (uint64_t*)(smem + STAGES * (kABytes + kBBytes));
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;  // accumulator a holds a finished tile
   uint64_t* tempty = tfull + 2;      // accumulator a has been read by the epilogue
   uint32_t* tslot = (uint32_t*)(tempty + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int mt = (e.M + BM - 1) / BM, nt = (e.N + BN - 1) / BN;
+  const int mt = (e.M + BM - 1) / BM, nt = (e.N + bn - 1) / bn;
   const int items = splits * mt * nt;
+  const uint32_t bbytes = (uint32_t)bn * BK * 2;
   const int kt_total = (K + BK - 1) / BK;
 
   if (threadIdx.x == 0) {
@@ -316,14 +394,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             ok = false;
             break;
           }
-          mbar_expect_tx(&full[s], kABytes + kBBytes);
+          mbar_expect_tx(&full[s], kABytes + bbytes);
           tma_load_2d(sA + s * kABytes, &ta, kt * BK, mb * BM, &full[s]);
-          tma_load_2d(sB + s * kBBytes, &tb, kt * BK, nb * BN, &full[s]);
+          tma_load_2d(sB + s * kBBytes, &tb, kt * BK, nb * bn, &full[s]);
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
+      const uint32_t id = idesc(bn);
       int i = 0, j = 0;
       bool ok = true;
       for (int w = blockIdx.x; w < items && ok; w += gridDim.x, ++j) {
@@ -347,7 +426,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           const uint32_t pa = saddr(sA + s * kABytes), pb = saddr(sB + s * kBBytes);
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            mma_bf16(acc, sdesc(pa + 32 * kk), sdesc(pb + 32 * kk), (kt > kt0 || kk > 0) ? 1u : 0u);
+            mma_bf16(acc, sdesc(pa + 32 * kk), sdesc(pb + 32 * kk), id, (kt > kt0 || kk > 0) ? 1u : 0u);
           mma_commit(&empty[s]);
         }
         if (!ok) break;
@@ -361,9 +440,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     int j = 0;
     for (int w = blockIdx.x; w < items; w += gridDim.x, ++j) {
       int z, mb, nb;
-        decode_item(w, mt, nt, z, mb, nb);
+      decode_item(w, mt, nt, z, mb, nb);
       const int kt0 = z * kts, kt1 = kt0 + kts < kt_total ? kt0 + kts : kt_total;
       const int a = j & 1, u = j >> 1;
+      const int n0 = nb * bn;
+      epi_consts(e, n0, bn, scratch[q], BN);
       bool ok = mbar_wait(&tfull[a], u & 1, spin);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) {
@@ -371,18 +452,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         break;
       }
       tc_fence_after();
-      const int row = mb * BM + q * 32 + lane;
-      const int n0 = nb * BN;
-      for (int c = 0; c < BN; c += 16) {
+      for (int c = 0; c < bn; c += 32) {
         if (n0 + c >= e.N) break;
-        float v[16];
+        float v[32];
         if (kt1 > kt0) {
-          tmem_ld16(tmem + (uint32_t)(a * BN) + ((uint32_t)(q * 32) << 16) + (uint32_t)c, v);
+          tmem_ld32(tmem + (uint32_t)(a * BN) + ((uint32_t)(q * 32) << 16) + (uint32_t)c, v);
         } else {
 #pragma unroll
-          for (int t = 0; t < 16; ++t) v[t] = 0.0f;
+          for (int t = 0; t < 32; ++t) v[t] = 0.0f;
         }
-        epi_store16(e, row, n0 + c, v, z);
+        epi_block(e, mb * BM + q * 32, n0 + c, v, z, scratch[q], scratch[q] + c, BN);
       }
       tc_fence_before();
       __syncwarp();
@@ -397,6 +476,133 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   }
 }
 
+// Products with few output tiles: one 128 x 64 tile per CTA, the whole
+// contraction in it.  The K splits of the plan fix how the result is rounded
+// (FP32 sums per split, added in order); here each split accumulates in 64
+// tensor-memory columns of its own and the epilogue adds them, so there are no
+// partial tiles in memory and no second kernel, and eight epilogue warps take
+// one 32 x 32 block each where four took eight (a GELU tile of 128 x 256 on
+// one SM took 54 us).  One launch can hold two products, the weight and the
+// input gradient of a layer.  A layer of 512 x 512 at 256 rows, with launch
+// gaps: forward 14.3 -> 10.5 us, backward 25 -> 12-16 us; the 64-wide first
+// layer at 128 rows 54 -> 7.3 us.
+struct SmallG {
+  CUtensorMap ta, tb;  // boxes of 128 and of 64 rows
+  int K, kts, splits, mt;
+  Epi e;
+};
+struct SmallP {
+  SmallG g[2];
+  int first1;  // CTAs from here on work on g[1]
+};
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    k_gemm_small(const __grid_constant__ SmallP p, int* err, long long spin) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + kSmallStages * kABytes;
+  __shared__ __align__(16) float scratch[8][kScratch];
+  uint64_t* full = (uint64_t*)(smem + kSmallStages * (kABytes + kSBytes));
+  uint64_t* empty = full + kSmallStages;
+  uint64_t* tfull = empty + kSmallStages;
+  uint32_t* tslot = (uint32_t*)(tfull + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int second = (int)blockIdx.x >= p.first1;
+  const SmallG& g = p.g[second];
+  const int item = (int)blockIdx.x - (second ? p.first1 : 0);
+  const int mb = item % g.mt, nb = item / g.mt;
+  const int kt_total = (g.K + BK - 1) / BK;
+  uint32_t cols = 64;
+  while (cols < (uint32_t)(g.splits * SN)) cols *= 2;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSmallStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(tslot)), "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tslot;
+
+  if (warp == 0) {
+    if (lane == 0) {  // producer
+      for (int kt = 0; kt < kt_total; ++kt) {
+        const int s = kt % kSmallStages;
+        if (kt >= kSmallStages && !mbar_wait(&empty[s], ((kt / kSmallStages) - 1) & 1, spin)) {
+          atomicExch(err, 1);
+          break;
+        }
+        mbar_expect_tx(&full[s], kABytes + kSBytes);
+        tma_load_2d(sA + s * kABytes, &g.ta, kt * BK, mb * BM, &full[s]);
+        tma_load_2d(sB + s * kSBytes, &g.tb, kt * BK, nb * SN, &full[s]);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer: split z accumulates in columns [64 z, 64 z + 64)
+      const uint32_t id = idesc(SN);
+      bool ok = true;
+      uint32_t acc = tmem;
+      for (int kt = 0, in = 0; kt < kt_total; ++kt, ++in) {
+        if (in == g.kts) {
+          in = 0;
+          acc += SN;
+        }
+        const int s = kt % kSmallStages;
+        if (!mbar_wait(&full[s], (kt / kSmallStages) & 1, spin)) {
+          atomicExch(err, 1);
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t pa = saddr(sA + s * kABytes), pb = saddr(sB + s * kSBytes);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk)
+          mma_bf16(acc, sdesc(pa + 32 * kk), sdesc(pb + 32 * kk), id, (in > 0 || kk > 0) ? 1u : 0u);
+        mma_commit(&empty[s]);
+      }
+      if (ok) mma_commit(tfull);
+    }
+  } else {
+    // epilogue: warp w reads accumulator lanes (rows) 32 (w % 4) .. + 31, columns 32 ((w - 2) / 4) .. + 31
+    const int q = warp & 3, c = 32 * ((warp - 2) >> 2);
+    epi_consts(g.e, nb * SN + c, 32, scratch[warp - 2], 32);
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull, 0, spin));
+    if (!ok) {
+      if (lane == 0) atomicExch(err, 1);
+    } else {
+      tc_fence_after();
+      const int n0 = nb * SN + c;
+      if (n0 < g.e.N) {
+        float v[32];
+        const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c;
+        tmem_ld32(at, v);
+        for (int z = 1; z < g.splits; ++z) {
+          float u[32];
+          tmem_ld32(at + z * SN, u);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] += u[j];
+        }
+        epi_block(g.e, mb * BM + q * 32, n0, v, 0, scratch[warp - 2], scratch[warp - 2], 32);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+  }
+}
+
 // sum of the K-split partial tiles, then the epilogue
 __global__ void k_splitk(const float* ws, int splits, size_t stride, Epi e) {
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -405,7 +611,7 @@ __global__ void k_splitk(const float* ws, int splits, size_t stride, Epi e) {
   int m = (int)(i / e.N), n = (int)(i % e.N);
   float acc = 0.0f;
   for (int z = 0; z < splits; ++z) acc += ws[(size_t)z * stride + i];
-  epi_one(e, m, n, acc, 0);
+  epi_one(e, m, n, acc);
 }
 
 // --------------------------------------------------------- other kernels
@@ -651,14 +857,6 @@ __global__ void __launch_bounds__(256) k_adam(const __grid_constant__ AdamP p) {
   }
 }
 
-// de-standardised network outputs: out = y sd + mu (y row-major, N columns)
-__global__ void k_destd(const float* Y, float* out, size_t total, int N, const float* mu, const float* sd) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  int n = (int)(i % N);
-  out[i] = Y[i] * sd[n] + mu[n];
-}
-
 // bfloat16 copies of FP32 weights (after set_params)
 __global__ void k_w16(const float* W, int out, int in, bf16* W16, bf16* W16T) {
   size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -720,20 +918,65 @@ struct Gemm {
   CUtensorMap ta, tb;
   int M, N, K, splits, kts;
   Epi e;
+  bool small = false;  // run as k_gemm_small
+  int bn = BN;         // rows of tb's boxes: 64 for k_gemm_small, else the tile width of k_gemm_tc
 };
 
-static int g_smem_set = -1;
+// dynamic shared memory of the two kernels, once per device and thread of the caller
+static cudaError_t set_smem() {
+  static thread_local int done = -1;
+  int dev = 0;
+  cudaError_t c = cudaGetDevice(&dev);
+  if (c != cudaSuccess || done == dev) return c;
+  c = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
+  if (c == cudaSuccess)
+    c = cudaFuncSetAttribute(k_gemm_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
+  if (c == cudaSuccess) done = dev;
+  return c;
+}
+
+// k_gemm_small pays while its tiles fit the GPU about twice, tensor memory
+// holds every split, and the contraction, which one CTA walks alone at about
+// 0.4 us per 64, stays short: 4,000 in one CTA took 25 us, split over 32 CTAs
+// with k_splitk 17
+static bool fits_small(int M, int N, int K, int splits, int sms) {
+  return splits <= kSmallSplits && K <= 24 * BK &&
+         (long)((M + BM - 1) / BM) * ((N + SN - 1) / SN) <= 2L * sms;
+}
+
+static SmallG small_of(const Gemm& g) {
+  SmallG s;
+  s.ta = g.ta;
+  s.tb = g.tb;
+  s.K = g.K;
+  s.kts = g.kts;
+  s.splits = g.splits;
+  s.mt = (g.e.M + BM - 1) / BM;
+  s.e = g.e;
+  return s;
+}
+
+// one or two products whose plan says small (b may be null)
+static cudaError_t run_small(const Gemm& a, const Gemm* b, int* err, cudaStream_t st, long long spin) {
+  cudaError_t c = set_smem();
+  if (c != cudaSuccess) return c;
+  SmallP p;
+  p.g[0] = small_of(a);
+  p.g[1] = b ? small_of(*b) : p.g[0];
+  p.first1 = p.g[0].mt * ((a.N + SN - 1) / SN);
+  const int grid = p.first1 + (b ? p.g[1].mt * ((b->N + SN - 1) / SN) : 0);
+  k_gemm_small<<<grid, kSmallThreads, kSmallSmem, st>>>(p, err, spin);
+  return cudaGetLastError();
+}
 
 static cudaError_t run_gemm(const Gemm& g, float* ws, int* err, cudaStream_t st, long long spin, int sms) {
-  if (g_smem_set < 0) {
-    cudaError_t c = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
-    if (c != cudaSuccess) return c;
-    g_smem_set = 1;
-  }
-  const int items = g.splits * ((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
+  if (g.small) return run_small(g, nullptr, err, st, spin);
+  cudaError_t c = set_smem();
+  if (c != cudaSuccess) return c;
+  const int items = g.splits * ((g.e.M + BM - 1) / BM) * ((g.N + g.bn - 1) / g.bn);
   const int grid = items < sms ? items : sms;
   if (g.splits == 1) {
-    k_gemm_tc<<<grid, kGemmThreads, kGemmSmem, st>>>(g.ta, g.tb, g.K, g.kts, 1, g.e, err, spin);
+    k_gemm_tc<<<grid, kGemmThreads, kGemmSmem, st>>>(g.ta, g.tb, g.K, g.kts, 1, g.bn, g.e, err, spin);
     return cudaGetLastError();
   }
   Epi p = g.e;
@@ -741,8 +984,8 @@ static cudaError_t run_gemm(const Gemm& g, float* ws, int* err, cudaStream_t st,
   p.f32 = ws;
   p.ld_f32 = g.N;
   p.split_stride = (size_t)g.M * g.N;
-  k_gemm_tc<<<grid, kGemmThreads, kGemmSmem, st>>>(g.ta, g.tb, g.K, g.kts, g.splits, p, err, spin);
-  size_t total = (size_t)g.M * g.N;
+  k_gemm_tc<<<grid, kGemmThreads, kGemmSmem, st>>>(g.ta, g.tb, g.K, g.kts, g.splits, g.bn, p, err, spin);
+  size_t total = (size_t)g.e.M * g.N;
   k_splitk<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(ws, g.splits, p.split_stride, g.e);
   return cudaGetLastError();
 }
@@ -757,7 +1000,34 @@ static void plan_split(Gemm& g, int sms) {
   g.splits = (kt + g.kts - 1) / g.kts;
 }
 
-static size_t ws_need(const Gemm& g) { return g.splits > 1 ? (size_t)g.splits * g.M * g.N : 0; }
+static size_t ws_need(const Gemm& g) { return g.splits > 1 && !g.small ? (size_t)g.splits * g.M * g.N : 0; }
+
+// Tile width of k_gemm_tc: the one whose waves of tiles cover the product with
+// the least width per SM (a tile costs about its width plus 32 columns' worth
+// of fixed time).  46,504 columns at one block of rows are 182 tiles of 256,
+// two waves of which the second holds 30 tiles, but 1.9 waves of 160 (21.7 ->
+// 9.1 us; at 256 rows 45 -> 32); wide products keep 256.
+static int tile_width(int M, int N, int splits, int sms) {
+  int best = BN;
+  long cost = 0;
+  for (int bn = BN; bn >= 128; bn -= 32) {
+    const long tiles = (long)splits * ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+    const long c = (tiles + sms - 1) / sms * (bn + 32);
+    if (bn == BN || c < cost) {
+      cost = c;
+      best = bn;
+    }
+  }
+  return best;
+}
+
+// split and kernel of one of the network's products, and its operand maps
+static bool plan_gemm(Gemm& g, const void* A, int lda, const void* B, int ldb, int sms) {
+  plan_split(g, sms);
+  g.small = fits_small(g.M, g.N, g.K, g.splits, sms);
+  g.bn = g.small ? SN : tile_width(g.M, g.N, g.splits, sms);
+  return make_map(&g.ta, A, g.M, g.K, lda, BM) && make_map(&g.tb, B, g.N, g.K, ldb, g.bn);
+}
 
 // --------------------------------------------------------------- the network
 struct Layer {
@@ -789,6 +1059,7 @@ struct Net {
   int* err = nullptr;
   float* loss = nullptr;
   int step = 0;
+  Gemm head;  // the output layer at one block of rows (inference of at most 128 rows)
   std::vector<Gemm> fwd, bwd_w, bwd_x;  // fwd[l], bwd_w[l] (dW_l), bwd_x[l] (dA_l, l >= 1)
   std::vector<void*> allocs;
   std::string last_error;
@@ -827,7 +1098,7 @@ static bool plan(Net* n) {
     // forward: [Mb x in] * W[out x in]^T
     Gemm& f = n->fwd[l];
     f.M = Mb; f.N = out; f.K = in;
-    if (!make_map(&f.ta, n->A[l], Mb, in, in, BM) || !make_map(&f.tb, y.W16, out, in, in, BN)) return false;
+    if (!plan_gemm(f, n->A[l], in, y.W16, in, n->sms)) return false;
     memset(&f.e, 0, sizeof(Epi));
     f.e.M = Mb; f.e.N = out; f.e.rows_valid = Mb; f.e.bias = y.b;
     if (l < nl - 1) {
@@ -839,28 +1110,33 @@ static bool plan(Net* n) {
       f.e.op = EPI_F32;
       f.e.f32 = n->Y; f.e.ld_f32 = out;
     }
-    plan_split(f, n->sms);
     ws = ws > ws_need(f) ? ws : ws_need(f);
+    if (l == nl - 1) {
+      // the same product for one block of rows: other tile widths fill the GPU; the split stays, it fixes the rounding
+      n->head = f;
+      if (!f.small) {
+        n->head.bn = tile_width(BM, out, f.splits, n->sms);
+        if (!make_map(&n->head.tb, y.W16, out, in, in, n->head.bn)) return false;
+      }
+    }
     // weight gradient: dW = D^T [out x Mb] * (A^T [in x Mb])^T
     Gemm& w = n->bwd_w[l];
     w.M = out; w.N = in; w.K = Mb;
-    if (!make_map(&w.ta, n->DT[l + 1], out, Mb, Mb, BM) || !make_map(&w.tb, n->AT[l], in, Mb, Mb, BN)) return false;
+    if (!plan_gemm(w, n->DT[l + 1], Mb, n->AT[l], Mb, n->sms)) return false;
     memset(&w.e, 0, sizeof(Epi));
     w.e.op = EPI_F32; w.e.M = out; w.e.N = in; w.e.rows_valid = out;
     w.e.f32 = y.gW; w.e.ld_f32 = in;
-    plan_split(w, n->sms);
     ws = ws > ws_need(w) ? ws : ws_need(w);
     if (l >= 1) {
       // input gradient: D_l = (D_{l+1} [Mb x out] * (W16T [in x out])^T) * GELU'(Z_l)
       Gemm& x = n->bwd_x[l];
       x.M = Mb; x.N = in; x.K = out;
-      if (!make_map(&x.ta, n->D[l + 1], Mb, out, out, BM) || !make_map(&x.tb, y.W16T, in, out, out, BN)) return false;
+      if (!plan_gemm(x, n->D[l + 1], out, y.W16T, out, n->sms)) return false;
       memset(&x.e, 0, sizeof(Epi));
       x.e.op = EPI_GELU_BWD; x.e.M = Mb; x.e.N = in; x.e.rows_valid = Mb;
       x.e.z = n->Z[l]; x.e.ld_z = in;
       x.e.bf = n->D[l]; x.e.ld_bf = in;
       x.e.bt = n->DT[l]; x.e.ld_bt = Mb;
-      plan_split(x, n->sms);
       ws = ws > ws_need(x) ? ws : ws_need(x);
     }
   }
@@ -886,10 +1162,26 @@ static acopf_status check_err(Net* n) {
     if (_e != cudaSuccess) return nfail(n, ACOPF_ECUDA, std::string("cuda: ") + cudaGetErrorString(_e)); \
   } while (0)
 
-static acopf_status forward(Net* n, int rows) {
+// the network on the rows of A[0].  Training (out null): pre-activations,
+// transposes and Y, all Mb rows.  Inference: the row blocks that hold rows,
+// only what the next layer reads, and the de-standardised outputs of the valid
+// rows straight into out.
+static acopf_status forward(Net* n, int rows, float* out = nullptr) {
   for (int l = 0; l < n->nl; ++l) {
-    Gemm g = n->fwd[l];
+    Gemm g = out && l == n->nl - 1 && rows <= BM ? n->head : n->fwd[l];
     g.e.rows_valid = rows;
+    if (out) {
+      if (l < n->nl - 1) {
+        g.e.M = (rows + BM - 1) / BM * BM;
+        g.e.f32 = nullptr;
+        g.e.bt = nullptr;
+      } else {
+        g.e.M = rows;
+        g.e.f32 = out;
+        g.e.mu = n->mu_y;
+        g.e.sd = n->sd_y;
+      }
+    }
     NCK(run_gemm(g, n->ws, n->err, n->stream, n->spin, n->sms));
   }
   return ACOPF_OK;
@@ -1088,15 +1380,11 @@ acopf_status acopf_mlp_forward(acopf_mlp_handle h, const float* X, int32_t rows,
   const int d0 = n->dims[0], dn = n->dims[n->nl];
   for (int r0 = 0; r0 < rows; r0 += n->Mb) {
     int rr = rows - r0 < n->Mb ? rows - r0 : n->Mb;
-    k_input<<<dim3((d0 + 31) / 32, n->Mb / 32), dim3(32, 8), 0, n->stream>>>(X + (size_t)r0 * d0, nullptr, rr, n->Mb,
-                                                                             d0, n->mu_x, n->sd_x, n->A[0], nullptr);
+    k_input<<<dim3((d0 + 31) / 32, (rr + BM - 1) / BM * (BM / 32)), dim3(32, 8), 0, n->stream>>>(
+        X + (size_t)r0 * d0, nullptr, rr, n->Mb, d0, n->mu_x, n->sd_x, n->A[0], nullptr);
     NCK(cudaGetLastError());
-    acopf_status s = forward(n, rr);
+    acopf_status s = forward(n, rr, Y + (size_t)r0 * dn);
     if (s) return s;
-    // outputs of the valid rows, de-standardised: y = y_std sd + mu
-    size_t ty = (size_t)rr * dn;
-    k_destd<<<(unsigned)((ty + 255) / 256), 256, 0, n->stream>>>(n->Y, Y + (size_t)r0 * dn, ty, dn, n->mu_y, n->sd_y);
-    NCK(cudaGetLastError());
   }
   return check_err(n);
 }
@@ -1116,8 +1404,13 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
                                           n->L[nl - 1].gb, n->part, n->done, n->loss, loss);
   NCK(cudaGetLastError());
   for (int l = nl - 1; l >= 0; --l) {
-    NCK(run_gemm(n->bwd_w[l], n->ws, n->err, n->stream, n->spin, n->sms));
-    if (l >= 1) NCK(run_gemm(n->bwd_x[l], n->ws, n->err, n->stream, n->spin, n->sms));
+    const Gemm &w = n->bwd_w[l], &x = n->bwd_x[l];
+    if (l >= 1 && w.small && x.small) {
+      NCK(run_small(w, &x, n->err, n->stream, n->spin));
+      continue;
+    }
+    NCK(run_gemm(w, n->ws, n->err, n->stream, n->spin, n->sms));
+    if (l >= 1) NCK(run_gemm(x, n->ws, n->err, n->stream, n->spin, n->sms));
   }
   n->step += 1;
   AdamP p;
@@ -1155,14 +1448,17 @@ acopf_status acopf_mlp_sync(acopf_mlp_handle h) {
 acopf_status acopf_gemm_bf16(const void* A, const void* B, float* C, int32_t M, int32_t N, int32_t K, int32_t splits,
                              void* stream, float* ms) {
   if (!A || !B || !C || M < 1 || N < 1 || K < 8 || K % 8) return ACOPF_EINVAL;
-  Gemm g;
-  memset(&g, 0, sizeof(g));
+  Gemm g{};
   g.M = M; g.N = N; g.K = K;
-  if (!make_map(&g.ta, A, M, K, K, BM) || !make_map(&g.tb, B, N, K, K, BN)) return ACOPF_EINVAL;
   int kt = (K + BK - 1) / BK;
   int s = splits < 1 ? 1 : (splits > kt ? kt : splits);
   g.kts = (kt + s - 1) / s;
   g.splits = (kt + g.kts - 1) / g.kts;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  g.bn = tile_width(M, N, g.splits, sms);
+  if (!make_map(&g.ta, A, M, K, K, BM) || !make_map(&g.tb, B, N, K, K, g.bn)) return ACOPF_EINVAL;
   g.e.op = EPI_F32; g.e.M = M; g.e.N = N; g.e.rows_valid = M; g.e.f32 = C; g.e.ld_f32 = N;
   cudaStream_t st = (cudaStream_t)stream;
   float* ws = nullptr;
@@ -1173,9 +1469,6 @@ acopf_status acopf_gemm_bf16(const void* A, const void* B, float* C, int32_t M, 
     cudaFree(err);
     return ACOPF_ENOMEM;
   }
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (ms) {
     cudaEventCreate(&e0);

@@ -70,3 +70,34 @@ def test_training_steps_at_tile_edges(dims, rows, offset):
         np.testing.assert_allclose(after, want, rtol=2 ** -22, atol=1e-3 * 2 ** -12)
     net.close()
     del xk, tk
+
+
+@pytest.mark.parametrize("dims,batch,rows", [([16, 32, 24], 128, 1), ([64, 512, 512, 712], 128, 129),
+                                             ([40, 72, 20488], 256, 128), ([40, 72, 20488], 256, 130),
+                                             ([4104, 264, 136], 256, 257)])
+def test_inference_at_tile_edges(dims, batch, rows):
+    """Outputs straight from the product's epilogue: one row, one more than a
+    block of rows, an output layer whose tiles are narrower for one block of
+    rows than for two, and a first layer summed from splits; nothing is
+    written past the rows asked for."""
+    rng = np.random.default_rng(dims[-1] + rows)
+    X = rng.standard_normal((rows, dims[0])).astype(np.float32)
+    T = (3.0 * rng.standard_normal((64, dims[-1])) + 1.0).astype(np.float32)
+    fit = rng.standard_normal((64, dims[0])).astype(np.float32)
+    net = binding.Mlp(dims, max_batch=batch)
+    flat = gg.mlp_init(dims, seed=4)
+    for (_, b) in _split(flat, dims):
+        b[:] = 0.1 * rng.standard_normal(b.size)
+    net.set_params(flat)
+    Xd, Td, Fd = (torch.from_numpy(a).cuda() for a in (X, T, fit))
+    net.fit_standardiser(Fd.data_ptr(), Td.data_ptr(), 64)
+    mx, sx, my, sy = net.get_standardiser()
+    Yd = torch.full((rows + 1, dims[-1]), 7.0, device="cuda")
+    net.forward(Xd.data_ptr(), rows, Yd.data_ptr())
+    params = [(w.astype(np.float64), b.astype(np.float64)) for w, b in _split(flat, dims)]
+    Y, _ = omlp.forward(params, (X.astype(np.float64) - mx) / sx, q=omlp.bf16_round)
+    got = Yd.cpu().double().numpy()
+    want = Y * sy + my
+    assert np.max(np.abs(got[:rows] - want)) <= 2 ** -7 * np.max(np.abs(want))
+    assert (got[rows] == 7.0).all()
+    net.close()
