@@ -208,7 +208,7 @@ struct Ctx {
   int sweep_stages = 0;  // record access of the sweep (acopf_tune), 4: one thread-block cluster per instance
   int cluster_cs = 1;         // cluster size of sweep_stages 4, chosen for
   int cluster_threads = -1;   // this CTA size (-1: not chosen yet)
-  bool cluster_res = false;   // and whether every component of an instance has a thread (static data in registers)
+  int cluster_res = 0;        // and how many threads every branch of an instance has (0: static data not in registers)
   bool cluster_dsm = false;   // and whether the state it exchanges stays in distributed shared memory
   std::vector<int> h_task_off, h_big_off;  // host copies of d.task_off, d.big_off
   // warm start staged by acopf_set_warm_start / acopf_set_warm_start_device

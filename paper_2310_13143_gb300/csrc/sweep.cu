@@ -23,6 +23,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string>
 #include <vector>
@@ -395,35 +396,77 @@ __device__ __forceinline__ void line_compute_to(const SweepP<T>& p, int l, const
 }
 
 // FP64 resident forms: the line update with the branch's active set and the
-// set's operator kept from one iteration to the next (line_eval; op in shared
-// memory, one column per thread).  The set is corrected up to three times; a
-// subproblem that this does not settle, and line_solver = 1, take the general
-// solves above.  Bound by the count of FP64 instructions on the slowest warp
-// (see line_qp.cuh); full FP64 solves: 2,000 buses 244 -> 157 ms (30.5 -> 19.7
-// us per iteration), 30 buses 638 -> 402 ms (22 -> 14).
-__device__ __noinline__ bool line_operator_call(const LineQP<double>& P, unsigned set, double* op, int stride) {
+// set's operator kept from one iteration to the next (line_operator,
+// line_eval).  The set is corrected up to three times; a subproblem that this
+// does not settle, and line_solver = 1, take the general solves above.
+//
+// What bounds it is the number of FP64 instructions on a warp's path: one takes
+// its SM partition's pipe for some 64 cycles whether the warp has one lane at
+// work or 32.  So where the launch allows it four lanes share a branch
+// (line_compute_quad): lane q holds row q of each matrix and takes variable q,
+// flow q and row q of the constraints, the vectors pass between the lanes by
+// shuffles, and a matrix product costs four FP64 instructions instead of
+// sixteen -- about 50 on the usual path against 150.  Full FP64 solves: 2,000
+// buses 135 -> 101 ms, 30 buses 331 -> 223 ms against one lane per branch (and 244
+// and 638 ms with a factorisation per iteration).
+//
+// What few iterations need -- a new operator, the general solves -- is called
+// out of line and reads the branch again from global memory, so that it costs
+// the common path no registers.
+__device__ __noinline__ bool line_operator_slow(const Dev& d, int l, unsigned set, double* op, int stride) {
+  const V4<double> zero = {0.0, 0.0, 0.0, 0.0};
+  LineQP<double> P;
+  line_problem(GRec<double>{(const double*)((const V4<double>*)d.lrec + l), d.L}, zero, zero, zero, zero, 0.0, P);
   return line_operator(P, set, op, stride);
 }
-__device__ __noinline__ void line_general_call(const LineQP<double>& P, const double* z, double* x, double* u,
-                                               int exact, double beta_scale, double tol, int outer, int newton) {
-  const double u_in[4] = {u[0], u[1], u[2], u[3]};
+// the set shown by the branch's last point, where a launch starts
+__device__ __noinline__ unsigned line_set_slow(const Dev& d, int l) {
+  const V4<double> zero = {0.0, 0.0, 0.0, 0.0};
+  LineQP<double> P;
+  line_problem(GRec<double>{(const double*)((const V4<double>*)d.lrec + l), d.L}, zero, zero, zero, zero, 0.0, P);
+  const V4<double> x0 = ((const V4<double>*)d.X)[2 * l], x1 = ((const V4<double>*)d.X)[2 * l + 1];
+  const V4<double> uu = ((const V4<double>*)d.U)[l];
+  const double x[4] = {x0.z, x0.w, x1.z, x1.w}, u[4] = {uu.x, uu.y, uu.z, uu.w};
+  return line_set_of(P, x, u);
+}
+// the whole line update of branch l by the general solves, from and to global
+// memory; returns the solution's set
+__device__ __noinline__ unsigned line_general_slow(const Dev& d, int l, int exact, double beta_scale, double tol,
+                                                   int outer, int newton) {
+  const V4<double>* Z = (const V4<double>*)d.Z;
+  const V4<double>* LM = (const V4<double>*)d.LAM;
+  const V4<double> z0 = Z[2 * l], z1 = Z[2 * l + 1], uu = ((const V4<double>*)d.U)[l];
+  const GRec<double> rec{(const double*)((const V4<double>*)d.lrec + l), d.L};
+  LineQP<double> P;
+  line_problem(rec, z0, z1, LM[2 * l], LM[2 * l + 1], ((const double*)d.trho_l)[l], P);
+  const double z[4] = {z0.z, z0.w, z1.z, z1.w};
+  double x[4], u[4] = {uu.x, uu.y, uu.z, uu.w};
+#pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = clampv(z[i], P.lo[i], P.hi[i]);
-  if (exact) {
-    if (line_pred_call(P, x, u)) return;
-    for (int i = 0; i < 4; ++i) u[i] = u_in[i];
-    if (line_exact_call(P, x, u) >= 0) return;
-    for (int i = 0; i < 4; ++i) {
-      x[i] = clampv(z[i], P.lo[i], P.hi[i]);
-      u[i] = u_in[i];
-    }
+  bool done = exact && line_pred_call(P, x, u);
+  if (exact && !done) {
+    u[0] = uu.x; u[1] = uu.y; u[2] = uu.z; u[3] = uu.w;
+    done = line_exact_call(P, x, u) >= 0;
   }
-  const double beta = beta_scale * fmax(fmax(P.q[0], P.q[4]), fmax(P.q[7], P.q[9]));
-  line_alm_call(P, x, u, beta, tol, outer, newton);
+  if (!done) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = clampv(z[i], P.lo[i], P.hi[i]);
+    u[0] = uu.x; u[1] = uu.y; u[2] = uu.z; u[3] = uu.w;
+    const double beta = beta_scale * fmax(fmax(P.q[0], P.q[4]), fmax(P.q[7], P.q[9]));
+    line_alm_call(P, x, u, beta, tol, outer, newton);
+  }
+  V4<double> o0, o1, ou;
+  line_outputs(rec, x, u, o0, o1, ou);
+  ((V4<double>*)d.X)[2 * l] = o0;
+  ((V4<double>*)d.X)[2 * l + 1] = o1;
+  ((V4<double>*)d.U)[l] = ou;
+  return line_set_of(P, x, u);
 }
 
+// one lane per branch: op in shared memory, one column per thread
 template <typename Rec>
-__device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, int l, const Rec& rec, V4<double> z0,
-                                                  V4<double> z1, V4<double> l0, V4<double> l1, V4<double> uu,
+__device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, const Dev& d, int l, const Rec& rec,
+                                                  V4<double> z0, V4<double> z1, V4<double> l0, V4<double> l1,
                                                   double rho, unsigned& set, double* op, int stride) {
   LineQP<double> P;
   line_problem(rec, z0, z1, l0, l1, rho, P);
@@ -432,8 +475,7 @@ __device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, int l
   if (p.line_exact) {
     for (int attempt = 0; attempt < 4; ++attempt) {
       if (!(set & kSetValid)) {
-        const LineQP<double> Q = P;  // a copy for the call: P itself stays in registers
-        if (!line_operator_call(Q, set, op, stride)) break;
+        if (!line_operator_slow(d, l, set, op, stride)) break;
         set |= kSetValid;
       }
       unsigned next;
@@ -443,16 +485,8 @@ __device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, int l
     }
   }
   if (!ok) {
-    const LineQP<double> Q = P;
-    const double zv[4] = {z0.z, z0.w, z1.z, z1.w};
-    double xs[4], us[4] = {uu.x, uu.y, uu.z, uu.w};
-    line_general_call(Q, zv, xs, us, p.line_exact, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
-    set = line_set_of(Q, xs, us);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      x[i] = xs[i];
-      u[i] = us[i];
-    }
+    set = line_general_slow(d, l, p.line_exact, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
+    return;
   }
   V4<double> o0, o1, ou;
   line_outputs(rec, x, u, o0, o1, ou);
@@ -462,17 +496,170 @@ __device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, int l
   ((V4<double>*)p.d.U)[l] = ou;
 }
 
-// the set shown by the branch's last point (from global memory), where a
-// launch starts
-template <typename Rec>
-__device__ __forceinline__ unsigned line_set_start(const Dev& d, int l, const Rec& rec) {
-  LineQP<double> P;
-  const V4<double> zero = {0.0, 0.0, 0.0, 0.0};
-  line_problem(rec, zero, zero, zero, zero, 0.0, P);
-  const V4<double> x0 = ((const V4<double>*)d.X)[2 * l], x1 = ((const V4<double>*)d.X)[2 * l + 1];
-  const V4<double> uu = ((const V4<double>*)d.U)[l];
-  const double x[4] = {x0.z, x0.w, x1.z, x1.w}, u[4] = {uu.x, uu.y, uu.z, uu.w};
-  return line_set_of(P, x, u);
+// Four lanes per branch: what lane q of branch l holds for the sweep.
+struct QuadRec {
+  double Q[4], Fc[4], Fr[4];       // row q of Q; column q and row q of F
+  double c0, f0, lo, hi, rho;      // of variable q, flow q
+  double n[4], b, b1, R0, R1, qm;  // row q of the constraints, 1 + |b|; entry q of the line-limit rows; max |Q|
+  double P[4], p0, M[4], m0;       // row q of the operator; row q's multiplier
+  bool on;                         // whether constraint row q exists
+  unsigned set;
+};
+
+__device__ __forceinline__ void quad_load(const Dev& d, int l, int q, QuadRec& a) {
+  const GRec<double> rec{(const double*)((const V4<double>*)d.lrec + l), d.L};
+  a.qm = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    a.Q[j] = rec(pk(q, j));
+    a.Fc[j] = rec(10 + 4 * j + q);
+    a.Fr[j] = rec(10 + 4 * q + j);
+  }
+  for (int k = 0; k < 10; ++k) a.qm = fmax(a.qm, fabs(rec(k)));
+  a.f0 = rec(26 + q);
+  a.c0 = rec(30 + q);
+  a.lo = rec(34 + q);
+  a.hi = rec(38 + q);
+  a.R0 = rec(42 + q);
+  a.R1 = rec(46 + q);
+  const double s = q == 2 ? 1.0 : -1.0;  // angle rows: x1 - x3 <= ahi, x3 - x1 <= -alo
+#pragma unroll
+  for (int j = 0; j < 4; ++j) a.n[j] = q < 2 ? rec(42 + 4 * q + j) : (j == 1 ? s : (j == 3 ? -s : 0.0));
+  a.b = q < 2 ? rec(50 + q) : (q == 2 ? rec(53) : -rec(52));
+  a.b1 = 1.0 + fabs(a.b);
+  a.on = q < 2 ? rec(54 + q) > 0.0 : rec(53) < 1e29;
+  a.rho = ((const double*)d.trho_l)[l];
+  a.p0 = a.m0 = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) a.P[j] = a.M[j] = 0.0;
+}
+
+__device__ __forceinline__ double quad_get(double v, int j) { return __shfl_sync(0xffffffffu, v, j, 4); }
+__device__ __forceinline__ unsigned quad_max(unsigned v) {
+  unsigned w = __shfl_xor_sync(0xffffffffu, v, 1);
+  v = w > v ? w : v;
+  w = __shfl_xor_sync(0xffffffffu, v, 2);
+  return w > v ? w : v;
+}
+__device__ __forceinline__ double quad_dot(const double* a, double v, double s) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) s = fma(a[j], quad_get(v, j), s);
+  return s;
+}
+
+// The line update of the warp's eight branches.  All 32 lanes call it; quads
+// without a branch (is = false) go along on zeros.  op: the quad's column of
+// operators in shared memory.
+__device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const Dev& d, bool is, int l, QuadRec& a,
+                                                  double* op, int stride) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, q = lane & 3, qb = lane & ~3;
+  // coupling (end q / 2, component q % 2): flow q and variable q
+  const size_t at = is ? 8 * (size_t)l + 4 * (q >> 1) + (q & 1) : 0;
+  double zf = 0.0, zv = 0.0, lf = 0.0, lv = 0.0;
+  if (is) {
+    const double *Z = (const double*)d.Z + at, *LM = (const double*)d.LAM + at;
+    zf = Z[0];
+    zv = Z[2];
+    lf = LM[0];
+    lv = LM[2];
+  }
+  const double c = quad_dot(a.Fc, lf - a.rho * zf, a.c0 + lv - a.rho * zv);
+  const unsigned ch = quad_max(abs_hi(c));
+  double x = 0.0, mu = 0.0;
+  bool general = !p.line_exact;  // of the quad: left to the general solves
+  // every exit from the loop is warp-uniform: all lanes take part in its shuffles
+  for (int attempt = 0; attempt < 4; ++attempt) {
+    // operators that are missing, by the quads' first lanes
+    const bool build = is && !general && !(a.set & kSetValid);
+    if (__any_sync(FULL, build)) {
+      bool good = true;
+      if (build && q == 0) good = line_operator_slow(d, l, a.set, op, stride);
+      __syncwarp();
+      good = __shfl_sync(FULL, (int)good, 0, 4) != 0;
+      if (build) {
+        if (good) {
+          int r0, r1;
+          set_rows((a.set >> 8) & 15u, r0, r1);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            a.P[j] = op[pk(q, j) * stride];
+            a.M[j] = q == r0 ? op[(14 + j) * stride] : (q == r1 ? op[(18 + j) * stride] : 0.0);
+          }
+          a.p0 = op[(10 + q) * stride];
+          a.m0 = q == r0 ? op[22 * stride] : (q == r1 ? op[23 * stride] : 0.0);
+          a.set |= kSetValid;
+        } else {
+          general = true;
+        }
+      }
+      __syncwarp();
+    }
+    // the point, one refinement step, and the row multipliers (the steps of line_eval)
+    x = a.p0 - quad_dot(a.P, c, 0.0);
+    double g = quad_dot(a.Q, x, c);
+    mu = 0.0;
+    if (__any_sync(FULL, is && (a.set & 0xf00u))) {
+      mu = a.m0 - quad_dot(a.M, c, 0.0);
+      const double m0 = quad_get(mu, 0), m1 = quad_get(mu, 1), ma = quad_get(mu, 2) - quad_get(mu, 3);
+      g += m0 * a.R0 + m1 * a.R1;
+      if (q & 1) g += q == 1 ? ma : -ma;
+      mu -= quad_dot(a.M, g, 0.0);
+    }
+    x -= quad_dot(a.P, g, 0.0);
+    // KKT check
+    const unsigned xh = quad_max(abs_hi(x)), gh = quad_max(abs_hi(g));
+    const bool finite = xh < 0x7ff00000u && ch < 0x7ff00000u && gh < 0x7ff00000u;
+    const double xm = double_of((unsigned long long)xh << 32), cm = double_of((unsigned long long)ch << 32);
+    const double tx = 1e-11 * (xm + 1.0);
+    const double tol = 1e-11 * (cm + 1.0) + 1e-11 * a.qm * xm;
+    const unsigned th = hi_of(tol), txh = hi_of(tx);
+    const double v = quad_dot(a.n, x, -a.b);
+    const double below = a.lo - x, above = x - a.hi;
+    bool fx = (a.set >> q) & 1u, hs = (a.set >> (4 + q)) & 1u, act = (a.set >> (8 + q)) & 1u;
+    bool bad = !finite;
+    const bool feas = !a.on || le_tol(v, hi_of(tx * a.b1));
+    if (!feas) bad = true;
+    if (act) {
+      if (!le_tol(-mu, th)) { bad = true; act = false; }
+    } else if (!feas) {
+      act = true;
+    }
+    if (!fx) {
+      if (abs_hi(g) > th) bad = true;
+      if (!le_tol(below, txh)) { bad = true; fx = true; hs = false; }
+      else if (!le_tol(above, txh)) { bad = true; fx = true; hs = true; }
+      if ((long long)bits_of(below) > 0) x = a.lo;
+      if ((long long)bits_of(above) > 0) x = a.hi;
+    } else if (bits_of(a.lo) != bits_of(a.hi) && ((bits_of(a.lo) | bits_of(a.hi)) << 1)) {
+      if (!le_tol(hs ? g : -g, th)) { bad = true; fx = false; hs = false; }
+    }
+    const unsigned fail = __ballot_sync(FULL, bad && is && !general);
+    if (!fail) break;
+    const unsigned nfx = (__ballot_sync(FULL, fx) >> qb) & 15u, nhs = (__ballot_sync(FULL, hs) >> qb) & 15u,
+                   nact = (__ballot_sync(FULL, act) >> qb) & 15u;
+    const bool whole = __shfl_sync(FULL, (int)finite, 0, 4) != 0;
+    if ((fail >> qb) & 15u) {
+      const unsigned next = nfx | (nhs << 4) | (nact << 8);
+      if (!whole || attempt == 3 || next == (a.set & ~kSetValid)) general = true;
+      else a.set = next;
+    }
+    if (!__any_sync(FULL, is && !general && !(a.set & kSetValid))) break;  // nothing is left to correct
+  }
+  if (__any_sync(FULL, is && general)) {
+    unsigned s = a.set;
+    if (is && general && q == 0)
+      s = line_general_slow(d, l, p.line_exact, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
+    s = __shfl_sync(FULL, s, 0, 4);
+    if (general) a.set = s;
+  }
+  const double xf = quad_dot(a.Fr, x, a.f0);
+  if (is && !general) {
+    double* X = (double*)d.X + at;
+    X[0] = xf;
+    X[2] = x;
+    ((double*)d.U)[4 * (size_t)l + q] = ((a.set >> (8 + q)) & 1u) && pos_w(mu) ? mu : 0.0;
+  }
 }
 
 // line update of branch l reading its record from global memory (rs, stride L)
@@ -1064,8 +1251,10 @@ __device__ void bus_task_big(const SweepP<T>& p, int q0, int q1, const Dst& dst,
 // most two bus tasks (checked by the launcher); their static data -- the
 // branch record, the generator record, instance ids, task slots and bus data
 // -- is loaded once, before the first iteration, and held in registers.
-template <typename T, bool RES>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep(SweepP<T> p) {
+// RES is the number of lanes that share a branch: 1, or 4 in FP64
+// (line_compute_quad); 0: not resident.
+template <typename T, int RES>
+__global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep(const __grid_constant__ SweepP<T> p) {
   const Dev& d = p.d;
   // dynamic shared memory: residual accumulators (2K 64-bit, when smem_res),
   // finished flags (K ints), penalty factors (K floats), branch tiles
@@ -1105,21 +1294,30 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
   unsigned my_wset = 0u;  // the box bounds held at the end of the branch's last solve; FP64: its active set
   double* s_op = (double*)(((uintptr_t)(s_scale + K) + 15) & ~(uintptr_t)15);  // RES FP64: kLineOp values per thread
   TaskStatic<T> ta, tb;
+  // this thread's generator or branch: with four lanes per branch the branches come first
+  const int gen = RES == 4 ? tid - 4 * d.L : tid, br = RES == 4 ? tid >> 2 : tid - d.G;
+  const bool is_gen = gen >= 0 && gen < d.G, is_br = br >= 0 && br < d.L;
+  QuadRec qr;
   if (RES) {
-    if (tid < d.G) {
-      my_k = d.gen_inst[tid];
-      rr[0] = ((const V4<T>*)d.grec)[tid];
-      rr[1] = ((const V4<T>*)d.grec)[d.G + tid];
+    if (is_gen) {
+      my_k = d.gen_inst[gen];
+      rr[0] = ((const V4<T>*)d.grec)[gen];
+      rr[1] = ((const V4<T>*)d.grec)[d.G + gen];
       if (sizeof(T) == 8) rr[2] = {T(1) / (rr[0].y + rr[1].z), T(1) / rr[1].z, T(0), T(0)};
-    } else if (tid < d.G + d.L) {
-      const int l = tid - d.G;
-      my_k = d.br_inst[l];
+    } else if (is_br) {
+      my_k = d.br_inst[br];
+      if constexpr (RES == 4) {
+        quad_load(d, br, lane & 3, qr);
+        qr.set = line_set_slow(d, br);
+      } else {
 #pragma unroll
-      for (int c = 0; c < kRecChunks; ++c) rr[c] = ((const V4<T>*)d.lrec)[(size_t)c * d.L + l];
-      my_rho = ((const T*)d.trho_l)[l];
-      if constexpr (sizeof(T) == 8) my_wset = line_set_start(d, l, RRec<T>{rr});
-      else my_wset = d.wset[l];
+        for (int c = 0; c < kRecChunks; ++c) rr[c] = ((const V4<T>*)d.lrec)[(size_t)c * d.L + br];
+        my_rho = ((const T*)d.trho_l)[br];
+        if constexpr (sizeof(T) == 8) my_wset = line_set_slow(d, br);
+        else my_wset = d.wset[br];
+      }
     }
+    if constexpr (RES == 4) if (!is_br) qr = QuadRec{};
     ta = task_static<T>(d, wid < d.NT ? load_slot(d, wid, lane) : none);
     tb = task_static<T>(d, wid + nw < d.NT ? load_slot(d, wid + nw, lane) : none);
   }
@@ -1134,20 +1332,25 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     if (prof) tp0 = gtimer();
     // phase A: generators then branches
     if (RES) {
-      if (my_k >= 0 && !s_done[my_k]) {
-        if (tid < d.G) {
-          if constexpr (sizeof(T) == 8) gen_compute_kept(d, tid, rr[0], rr[1], rr[2].x, rr[2].y);
-          else gen_compute(d, tid, rr[0], rr[1]);
-        } else {
-          const int l = tid - d.G;
-          const V4<T>* Z = (const V4<T>*)d.Z;
-          const V4<T>* LM = (const V4<T>*)d.LAM;
-          if constexpr (sizeof(T) == 8)
-            line_compute_kept(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1],
-                              ((const V4<T>*)d.U)[l], my_rho, my_wset, s_op + threadIdx.x, blockDim.x);
+      const bool go = my_k >= 0 && !s_done[my_k];
+      const V4<T>* Z = (const V4<T>*)d.Z;
+      const V4<T>* LM = (const V4<T>*)d.LAM;
+      if constexpr (RES == 4) {
+        if (go && is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+        line_compute_quad(p, d, go && is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
+      } else if (go) {
+        if constexpr (sizeof(T) == 8) {
+          if (is_gen)
+            gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
           else
-            line_compute(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1], ((const V4<T>*)d.U)[l],
-                         my_rho, &my_wset);
+            line_compute_kept(p, d, br, RRec<T>{rr}, Z[2 * br], Z[2 * br + 1], LM[2 * br], LM[2 * br + 1], my_rho,
+                              my_wset, s_op + threadIdx.x, blockDim.x);
+        } else {
+          if (is_gen)
+            gen_compute(d, gen, rr[0], rr[1]);
+          else
+            line_compute(p, br, RRec<T>{rr}, Z[2 * br], Z[2 * br + 1], LM[2 * br], LM[2 * br + 1],
+                         ((const V4<T>*)d.U)[br], my_rho, &my_wset);
         }
       }
     } else if (!kTiled) {
@@ -1298,7 +1501,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     if (prof) atomicAdd(&d.phase_ns[3], gtimer() - tp1);
     if (all && !p.fixed) { ++it; break; }
   }
-  if (RES && sizeof(T) == 4 && tid >= d.G && tid < d.G + d.L) d.wset[tid - d.G] = (uint16_t)my_wset;
+  if (RES && sizeof(T) == 4 && is_br) d.wset[br] = (uint16_t)my_wset;
   // record the residuals of unfinished instances
   if (blockIdx.x == 0 && !aborted) {
     int last = (it - 1) & 1;
@@ -1405,10 +1608,9 @@ __device__ __forceinline__ void cluster_maxima(const unsigned long long* res, in
 // instance and a warp for every two of its bus tasks (checked by the
 // launcher); the records, instance data and task slots are then loaded once
 // and held in registers, as in the resident form of k_sweep.
-template <typename T, bool RES>
-__global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
+template <typename T, int RES>
+__global__ void __launch_bounds__(256, 1) k_sweep_cluster(const __grid_constant__ SweepP<T> p) {
   const Dev& d = p.d;
-  const unsigned FULL = 0xffffffffu;
   const int K = d.K;
   const int k = (int)cluster_index();
   const int cs = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
@@ -1431,19 +1633,29 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
   extern __shared__ __align__(16) unsigned char s_dyn_c[];
   double* s_op = (double*)s_dyn_c;  // RES FP64: kLineOp values per thread
   TaskStatic<T> ta, tb;
+  // this thread's generator or branch: with four lanes per branch the branches come first
+  const int gi = RES == 4 ? ct - 4 * (l1 - l0) : ct, bi = RES == 4 ? ct >> 2 : ct - nG;
+  const bool is_gen = gi >= 0 && gi < nG, is_br = bi >= 0 && bi < l1 - l0;
+  const int gen = g0 + gi, br = l0 + bi;
+  QuadRec qr;
   if (RES) {
-    if (ct < nG) {
-      rr[0] = ((const V4<T>*)d.grec)[g0 + ct];
-      rr[1] = ((const V4<T>*)d.grec)[d.G + g0 + ct];
+    if (is_gen) {
+      rr[0] = ((const V4<T>*)d.grec)[gen];
+      rr[1] = ((const V4<T>*)d.grec)[d.G + gen];
       if (sizeof(T) == 8) rr[2] = {T(1) / (rr[0].y + rr[1].z), T(1) / rr[1].z, T(0), T(0)};
-    } else if (l0 + ct - nG < l1) {
-      const int l = l0 + ct - nG;
+    } else if (is_br) {
+      if constexpr (RES == 4) {
+        quad_load(d, br, lane & 3, qr);
+        qr.set = line_set_slow(d, br);
+      } else {
 #pragma unroll
-      for (int c = 0; c < kRecChunks; ++c) rr[c] = ((const V4<T>*)d.lrec)[(size_t)c * d.L + l];
-      my_rho = ((const T*)d.trho_l)[l];
-      if constexpr (sizeof(T) == 8) my_wset = line_set_start(d, l, RRec<T>{rr});
-      else my_wset = d.wset[l];
+        for (int c = 0; c < kRecChunks; ++c) rr[c] = ((const V4<T>*)d.lrec)[(size_t)c * d.L + br];
+        my_rho = ((const T*)d.trho_l)[br];
+        if constexpr (sizeof(T) == 8) my_wset = line_set_slow(d, br);
+        else my_wset = d.wset[br];
+      }
     }
+    if constexpr (RES == 4) if (!is_br) qr = QuadRec{};
     ta = task_static<T>(d, t0 + cw < t1 ? load_slot(d, t0 + cw, lane) : none);
     tb = task_static<T>(d, t0 + cw + nwc < t1 ? load_slot(d, t0 + cw + nwc, lane) : none);
   }
@@ -1457,19 +1669,23 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
     if (threadIdx.x < 2) s_res[slot][threadIdx.x] = 0;
     // phase A: the instance's generators, then its branches
     if (RES) {
-      if (ct < nG) {
-        if constexpr (sizeof(T) == 8) gen_compute_kept(d, g0 + ct, rr[0], rr[1], rr[2].x, rr[2].y);
-        else gen_compute(d, g0 + ct, rr[0], rr[1]);
-      } else if (l0 + ct - nG < l1) {
-        const int l = l0 + ct - nG;
-        const V4<T>* Z = (const V4<T>*)d.Z;
-        const V4<T>* LM = (const V4<T>*)d.LAM;
-        if constexpr (sizeof(T) == 8)
-          line_compute_kept(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1],
-                            ((const V4<T>*)d.U)[l], my_rho, my_wset, s_op + threadIdx.x, blockDim.x);
-        else
-          line_compute(p, l, RRec<T>{rr}, Z[2 * l], Z[2 * l + 1], LM[2 * l], LM[2 * l + 1], ((const V4<T>*)d.U)[l],
-                       my_rho, &my_wset);
+      const V4<T>* Z = (const V4<T>*)d.Z;
+      const V4<T>* LM = (const V4<T>*)d.LAM;
+      if constexpr (RES == 4) {
+        if (is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+        line_compute_quad(p, d, is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
+      } else if constexpr (sizeof(T) == 8) {
+        if (is_gen)
+          gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+        else if (is_br)
+          line_compute_kept(p, d, br, RRec<T>{rr}, Z[2 * br], Z[2 * br + 1], LM[2 * br], LM[2 * br + 1], my_rho,
+                            my_wset, s_op + threadIdx.x, blockDim.x);
+      } else {
+        if (is_gen)
+          gen_compute(d, gen, rr[0], rr[1]);
+        else if (is_br)
+          line_compute(p, br, RRec<T>{rr}, Z[2 * br], Z[2 * br + 1], LM[2 * br], LM[2 * br + 1],
+                       ((const V4<T>*)d.U)[br], my_rho, &my_wset);
       }
     } else {
       int u = ct;
@@ -1511,7 +1727,7 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(SweepP<T> p) {
       break;
     }
   }
-  if (RES && sizeof(T) == 4 && ct >= nG && l0 + ct - nG < l1) d.wset[l0 + ct - nG] = (uint16_t)my_wset;
+  if (RES && sizeof(T) == 4 && is_br) d.wset[br] = (uint16_t)my_wset;
   if (rank == 0 && threadIdx.x == 0) {
     if (conv) d.admm_done[k] = 1;
     d.admm_iters[k] = it;
@@ -1622,7 +1838,6 @@ __device__ __forceinline__ void bus_pair_dsm(DsmLane<T>& a, DsmLane<T>& b, const
 template <typename T>
 __global__ void __launch_bounds__(256, 1) k_sweep_cluster_dsm(SweepP<T> p) {
   const Dev& d = p.d;
-  const unsigned FULL = 0xffffffffu;
   const int K = d.K;
   const int k = (int)cluster_index();
   const int cs = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
@@ -1836,17 +2051,20 @@ static size_t sweep_smem(int K, int threads, int stages) {
   return b;
 }
 
-// dynamic shared memory of the kept line operators (FP64 resident forms)
+// dynamic shared memory of the kept line operators (FP64 resident forms), one per branch of the CTA
 template <typename T>
-static size_t op_smem(int threads) {
-  return sizeof(T) == 8 ? (size_t)kLineOp * sizeof(double) * threads : 0;
+static size_t op_smem(int threads, int lanes) {
+  return sizeof(T) == 8 ? (size_t)kLineOp * sizeof(double) * (threads / lanes) : 0;
 }
 
 // Launch shape of k_sweep<T>.  The resident form (sweep_stages 3) is used when
 // residual balancing is off and a co-resident grid gives every generator and
-// branch a thread of its own and every warp at most two bus tasks; otherwise
+// branch threads of its own and every warp at most two bus tasks; otherwise
 // (and for sweep_stages 0-2) the streaming form, with enough CTAs for one pass
-// over the larger of the two phases, capped at the co-resident maximum.
+// over the larger of the two phases, capped at the co-resident maximum.  FP64:
+// four threads per branch where they fit, which is up to 9,600 branches (255
+// registers: two warps per SM partition, some 100 FP64 instructions on its
+// pipe per iteration), else one (one warp per partition, 150).
 struct SweepShape {
   void* fn;
   int blocks;
@@ -1858,30 +2076,36 @@ static acopf_status sweep_shape(Ctx& c, const SweepP<T>& p, SweepShape& sh) {
   const Dev& d = c.d;
   const int threads = c.block_threads;
   if (c.sweep_stages == 3 && p.rb_period == 0) {
-    const size_t smem = sweep_smem<T>(d.K, threads, 0) + 16 + op_smem<T>(threads);
-    cudaFuncSetAttribute(k_sweep<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, true>, threads, smem);
-    if (c.ctas_per_sm > 0 && c.ctas_per_sm < per_sm) per_sm = c.ctas_per_sm;
-    const long cap = (long)per_sm * c.num_sms;
     const long wpb = threads / 32;
-    long need = ((long)d.G + d.L + threads - 1) / threads;
     const long need_b = ((long)d.NT + 2 * wpb - 1) / (2 * wpb);
     // the FP64 sweep gives each warp one bus task when the grid still fits
     // (two interleaved FP64 tasks take about twice as long as one)
     const long need_b1 = ((long)d.NT + wpb - 1) / wpb;
-    if (sizeof(T) == 8 && need_b1 > need && need_b1 <= cap) need = need_b1;
-    if (need_b > need) need = need_b;
-    if (need < 1) need = 1;
-    if (per_sm >= 1 && need <= cap) {
-      sh = {(void*)k_sweep<T, true>, (int)need, smem};
-      return ACOPF_OK;
+    for (int lanes = sizeof(T) == 8 ? 4 : 1; lanes >= 1; lanes -= 3) {
+      void* fn = (void*)k_sweep<T, 1>;
+      if constexpr (sizeof(T) == 8) if (lanes == 4) fn = (void*)k_sweep<T, 4>;
+      const size_t smem = sweep_smem<T>(d.K, threads, 0) + 16 + op_smem<T>(threads, lanes);
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      int per_sm = 0;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
+      if (c.ctas_per_sm > 0 && c.ctas_per_sm < per_sm) per_sm = c.ctas_per_sm;
+      const long cap = (long)per_sm * c.num_sms;
+      const long items = (long)d.G + (long)lanes * d.L;
+      long need = (items + threads - 1) / threads;
+      if (sizeof(T) == 8 && need_b1 > need && need_b1 <= cap) need = need_b1;
+      if (need_b > need) need = need_b;
+      if (need < 1) need = 1;
+      if (per_sm >= 1 && need <= cap) {
+        sh = {fn, (int)need, smem};
+        return ACOPF_OK;
+      }
     }
+    cudaGetLastError();
   }
   const size_t smem = sweep_smem<T>(d.K, threads, p.stages);
-  cudaFuncSetAttribute(k_sweep<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_sweep<T, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, false>, threads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, 0>, threads, smem);
   if (per_sm < 1) {
     c.last_error = "sweep: the kernel does not fit on a multiprocessor";
     return ACOPF_ECUDA;
@@ -1893,55 +2117,55 @@ static acopf_status sweep_shape(Ctx& c, const SweepP<T>& p, SweepShape& sh) {
   long maxb = (long)per_sm * c.num_sms;
   int blocks = (int)(need < maxb ? need : maxb);
   if (blocks < 1) blocks = 1;
-  sh = {(void*)k_sweep<T, false>, blocks, smem};
+  sh = {(void*)k_sweep<T, 0>, blocks, smem};
   return ACOPF_OK;
 }
 
-// Cluster size of sweep_stages 4: enough CTAs for one thread per generator or
-// branch of the largest instance, at most 16, fewer when a cluster of that
-// size cannot be resident.  The FP64 sweep takes one bus task per warp when a
-// resident cluster of at most 16 CTAs allows it (as in sweep_shape).
+// Cluster size of sweep_stages 4, and in res how many threads it gives a
+// branch: enough CTAs for every generator and branch of the largest instance,
+// at most 16, fewer (and res 0) when a cluster of that size cannot be resident.
+// The FP64 sweep takes four threads per branch, and one bus task per warp,
+// when a resident cluster of at most 16 CTAs allows it (as in sweep_shape).
 template <typename T>
-static int cluster_size(Ctx& c, int threads, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, bool& res) {
-  long items = 1, tasks = 0;
+static int cluster_size(Ctx& c, int threads, cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int& res) {
+  long items = 1, items4 = 1, tasks = 0;
   for (int k = 0; k < c.d.K; ++k) {
-    long n = (long)(c.h_gen_off[k + 1] - c.h_gen_off[k]) + (c.h_br_off[k + 1] - c.h_br_off[k]);
-    items = n > items ? n : items;
+    const long g = c.h_gen_off[k + 1] - c.h_gen_off[k], l = c.h_br_off[k + 1] - c.h_br_off[k];
+    items = std::max(items, g + l);
+    items4 = std::max(items4, g + 4 * l);
+    tasks = std::max(tasks, (long)(c.h_task_off[k + 1] - c.h_task_off[k]));
   }
-  const std::vector<int>& toff = c.h_task_off;
-  for (int k = 0; k < c.d.K; ++k) tasks = toff[k + 1] - toff[k] > tasks ? toff[k + 1] - toff[k] : tasks;
-  int cs = (int)((items + threads - 1) / threads);
   const long wpb = threads / 32;
-  const int cs_b = (int)((tasks + 2 * wpb - 1) / (2 * wpb));
-  if (cs_b > cs) cs = cs_b;
-  if (cs < 1) cs = 1;
-  res = cs <= 16;
-  if (cs > 16) cs = 16;
-  void* fn = res ? (void*)k_sweep_cluster<T, true> : (void*)k_sweep_cluster<T, false>;
-  cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  cfg.dynamicSmemBytes = res ? op_smem<T>(threads) : 0;
-  if (cfg.dynamicSmemBytes) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
-  const long cs_b1 = (tasks + wpb - 1) / wpb;
-  if (sizeof(T) == 8 && res && cs_b1 > cs && cs_b1 <= 16) {
-    cfg.gridDim = dim3((unsigned)cs_b1);
-    attr.val.clusterDim.x = (unsigned)cs_b1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) return (int)cs_b1;
-    cudaGetLastError();
-  }
-  for (; cs > 1; --cs) {
-    cfg.gridDim = dim3(cs);
-    attr.val.clusterDim.x = cs;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) break;
-    cudaGetLastError();
-    res = false;  // a smaller cluster no longer covers every component
-    cfg.dynamicSmemBytes = 0;
-    fn = (void*)k_sweep_cluster<T, false>;
+  auto fits = [&](long n, void* fn, size_t smem) {
     cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (smem) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3((unsigned)n);
+    attr.val.clusterDim.x = (unsigned)n;
+    int clusters = 0;
+    const bool ok = cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters >= 1;
+    cudaGetLastError();
+    return ok;
+  };
+  const long cs_b1 = (tasks + wpb - 1) / wpb;
+  if constexpr (sizeof(T) == 8) {
+    // four lanes per branch where 16 CTAs hold them (one bus task per warp comes with it)
+    res = 4;
+    const long n4 = std::max(std::max((items4 + threads - 1) / threads, cs_b1), 1L);
+    if (n4 <= 16 && fits(n4, (void*)k_sweep_cluster<T, 4>, op_smem<T>(threads, 4))) return (int)n4;
   }
-  if (res && (long)cs * threads < items) res = false;
-  return cs;
+  long cs = std::max(std::max((items + threads - 1) / threads, (tasks + 2 * wpb - 1) / (2 * wpb)), 1L);
+  if (cs <= 16) {
+    res = 1;
+    if (sizeof(T) == 8 && cs_b1 > cs && cs_b1 <= 16 && fits(cs_b1, (void*)k_sweep_cluster<T, 1>, op_smem<T>(threads, 1)))
+      return (int)cs_b1;
+    if (fits(cs, (void*)k_sweep_cluster<T, 1>, op_smem<T>(threads, 1))) return (int)cs;
+  }
+  res = 0;  // a smaller cluster does not cover every component
+  for (cs = std::min(cs, 16L); cs > 1; --cs)
+    if (fits(cs, (void*)k_sweep_cluster<T, 0>, 0)) break;
+  cfg.dynamicSmemBytes = 0;
+  return (int)cs;
 }
 
 template <typename T>
@@ -1960,12 +2184,13 @@ static acopf_status run_sweep_cluster(Ctx& c, const SweepP<T>& p) {
   cfg.numAttrs = 1;
   const size_t dsm_smem = (size_t)threads * (6 * sizeof(V4<T>) + 2 * sizeof(unsigned));
   if (c.cluster_threads != threads) {
-    bool res = false;
+    int res = 0;
     c.cluster_cs = cluster_size<T>(c, threads, cfg, attr[0], res);
+    cfg.dynamicSmemBytes = 0;
     c.cluster_res = res;
     c.cluster_threads = threads;
     // the shared-memory form: FP32, resident, and no bus of more than 32 entries
-    bool dsm = res && sizeof(T) == 4;
+    bool dsm = res == 1 && sizeof(T) == 4;
     for (int k = 0; dsm && k < c.d.K; ++k) dsm = c.h_big_off[k + 1] == c.h_big_off[k];
     if constexpr (sizeof(T) == 4) if (dsm) {
       cudaFuncSetAttribute(k_sweep_cluster_dsm<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1982,7 +2207,7 @@ static acopf_status run_sweep_cluster(Ctx& c, const SweepP<T>& p) {
   }
   const int cs = c.cluster_cs;
   attr[0].val.clusterDim.x = cs;
-  cfg.dynamicSmemBytes = c.cluster_dsm ? dsm_smem : (c.cluster_res ? op_smem<T>(threads) : 0);
+  cfg.dynamicSmemBytes = c.cluster_dsm ? dsm_smem : (c.cluster_res ? op_smem<T>(threads, c.cluster_res) : 0);
   if (!c.capturing) cudaMemsetAsync(c.d.err, 0, sizeof(int), c.stream);
   cfg.gridDim = dim3((unsigned)(c.d.K * cs));
   const bool prof = c.profiling && !c.capturing;
@@ -1990,11 +2215,12 @@ static acopf_status run_sweep_cluster(Ctx& c, const SweepP<T>& p) {
   cudaError_t e;
   if constexpr (sizeof(T) == 4) {
     e = c.cluster_dsm   ? cudaLaunchKernelEx(&cfg, k_sweep_cluster_dsm<T>, p)
-        : c.cluster_res ? cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, true>, p)
-                        : cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, false>, p);
+        : c.cluster_res ? cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, 1>, p)
+                        : cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, 0>, p);
   } else {
-    e = c.cluster_res ? cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, true>, p)
-                      : cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, false>, p);
+    e = c.cluster_res == 4   ? cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, 4>, p)
+        : c.cluster_res == 1 ? cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, 1>, p)
+                             : cudaLaunchKernelEx(&cfg, k_sweep_cluster<T, 0>, p);
   }
   c.launches++;
   if (e != cudaSuccess) {
