@@ -124,6 +124,31 @@ static void drop_graph(Ctx* c) {
   c->graph = nullptr;
 }
 
+// One instance's variables, pi (when wanted) and objective into c->h_stage;
+// synchronises the handle's stream.
+static acopf_status stage_instance(Ctx* c, int inst, const PackSrc& src) {
+  const size_t nb = c->h_bus_off[inst + 1] - c->h_bus_off[inst], nl = c->h_br_off[inst + 1] - c->h_br_off[inst],
+               ng = c->h_gen_off[inst + 1] - c->h_gen_off[inst];
+  const size_t n = 2 * ng + 2 * nb + 6 * nl + 1;
+  struct OnDevice {  // a read-out works whatever device the caller has current
+    int was = 0;
+    explicit OnDevice(int dev) { cudaGetDevice(&was); if (was != dev) cudaSetDevice(dev); else was = -1; }
+    ~OnDevice() { if (was >= 0) cudaSetDevice(was); }
+  } on(c->device);
+  if (n > c->stage_values) {
+    CK(cudaStreamSynchronize(c->stream));
+    if (c->h_stage) cudaFreeHost(c->h_stage);
+    c->h_stage = nullptr;
+    c->stage_values = 0;
+    CK(cudaMallocHost(&c->h_stage, sizeof(double) * n));
+    c->stage_values = n;
+  }
+  launch_pack(*c, src, inst, c->h_stage);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(c->stream));
+  return ACOPF_OK;
+}
+
 // oracle slot s of a branch -> (end, component) of the end-major layout
 static const int kSlotEnd[8] = {0, 0, 1, 1, 0, 0, 1, 1};
 static const int kSlotComp[8] = {0, 1, 0, 1, 2, 3, 2, 3};
@@ -437,7 +462,7 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   cudaError_t e = cudaSuccess;
   size_t T = c->precision == ACOPF_MIXED ? sizeof(float) : sizeof(double);
 #define A(ptr, n) if (e == cudaSuccess) e = dalloc(c, &(ptr), (n))
-  A(d.bus_off, K + 1); A(d.br_off, K + 1); A(d.gen_off, K + 1);
+  A(d.bus_off, K + 1); A(d.br_off, K + 1); A(d.gen_off, K + 1); A(c->d_gen_iperm, G);
   A(d.bus_inst, B); A(d.br_inst, L); A(d.gen_inst, G);
   A(d.pd, B); A(d.qd, B); A(d.gs, B); A(d.bs, B); A(d.wmin, B); A(d.wmax, B); A(d.isref, B);
   A(d.end_ptr, B + 1); A(d.end_idx, 2 * (size_t)L); A(d.gen_ptr, B + 1);
@@ -480,7 +505,7 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   std::vector<int> pd_dummy;
   e = cudaSuccess;
 #define U(dst, v) if (e == cudaSuccess && !(v).empty()) e = upload(c, dst, (v).data(), (v).size())
-  U(d.bus_off, bus_off); U(d.br_off, br_off); U(d.gen_off, gen_off);
+  U(d.bus_off, bus_off); U(d.br_off, br_off); U(d.gen_off, gen_off); U(c->d_gen_iperm, iperm);
   U(d.bus_inst, bus_inst); U(d.br_inst, br_inst); U(d.gen_inst, gen_inst_s);
   U(d.pd, pd); U(d.qd, qd); U(d.gs, gs); U(d.bs, bs); U(d.wmin, wmin); U(d.wmax, wmax); U(d.isref, isref);
   U(d.end_ptr, end_ptr); U(d.end_idx, end_idx); U(d.gen_ptr, gen_ptr);
@@ -549,6 +574,7 @@ acopf_status acopf_destroy(acopf_handle h) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   if (c->graph) cudaGraphDestroy(c->graph);
   if (c->h_running) cudaFreeHost(c->h_running);
+  if (c->h_stage) cudaFreeHost(c->h_stage);
   if (c->gstream) cudaStreamDestroy(c->gstream);
   free(c->h_bus_off); free(c->h_br_off); free(c->h_gen_off); free(c->h_gen_perm); free(c->h_gen_iperm);
   delete c;
@@ -709,31 +735,14 @@ acopf_status acopf_set_iterate(acopf_handle h, int32_t inst, const double* x, co
 acopf_status acopf_get_iterate(acopf_handle h, int32_t inst, double* x, double* pi) {
   Ctx* c = (Ctx*)h;
   if (!c || !inst_ok(c, inst) || !x) return fail(c, ACOPF_EINVAL, "acopf_get_iterate: bad arguments");
-  Dev& d = c->d;
-  CK(cudaStreamSynchronize(c->stream));
-  int b0 = c->h_bus_off[inst], nb = c->h_bus_off[inst + 1] - b0;
-  int l0 = c->h_br_off[inst], nl = c->h_br_off[inst + 1] - l0;
-  int g0 = c->h_gen_off[inst], ng = c->h_gen_off[inst + 1] - g0;
-  std::vector<double> pg(ng), qg(ng);
-  CK(cudaMemcpy(pg.data(), d.pg + g0, sizeof(double) * ng, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(qg.data(), d.qg + g0, sizeof(double) * ng, cudaMemcpyDeviceToHost));
-  for (int q = 0; q < ng; ++q) {
-    int internal = c->h_gen_iperm[g0 + q] - g0;
-    x[q] = pg[internal];
-    x[ng + q] = qg[internal];
-  }
-  double* w = x + 2 * ng;
-  CK(cudaMemcpy(w, d.w + b0, sizeof(double) * nb, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(w + nb, d.th + b0, sizeof(double) * nb, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(w + 2 * nb, d.wr + l0, sizeof(double) * nl, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(w + 2 * nb + nl, d.wi + l0, sizeof(double) * nl, cudaMemcpyDeviceToHost));
-  if (pi) {
-    std::vector<double> col(nl);
-    for (int r = 0; r < 4; ++r) {
-      CK(cudaMemcpy(col.data(), d.pi + (size_t)r * d.L + l0, sizeof(double) * nl, cudaMemcpyDeviceToHost));
-      for (int l = 0; l < nl; ++l) pi[4 * l + r] = col[l];
-    }
-  }
+  const Dev& d = c->d;
+  acopf_status s = stage_instance(c, inst, PackSrc{d.pg, d.qg, d.w, d.th, d.wr, d.wi, pi ? d.pi : nullptr});
+  if (s) return s;
+  const size_t nl = c->h_br_off[inst + 1] - c->h_br_off[inst];
+  const size_t nx = 2 * (size_t)(c->h_gen_off[inst + 1] - c->h_gen_off[inst]) +
+                    2 * (size_t)(c->h_bus_off[inst + 1] - c->h_bus_off[inst]) + 2 * nl;
+  memcpy(x, c->h_stage, sizeof(double) * nx);
+  if (pi) memcpy(pi, c->h_stage + nx, sizeof(double) * 4 * nl);
   return ACOPF_OK;
 }
 
@@ -1264,33 +1273,18 @@ acopf_status acopf_get_step(acopf_handle h, int32_t inst, double* dx, double* pi
   Ctx* c = (Ctx*)h;
   if (!c || !inst_ok(c, inst)) return fail(c, ACOPF_EINVAL, "acopf_get_step: bad arguments");
   if (!c->have_step) return fail(c, ACOPF_ENOTREADY, "acopf_get_step: no QP has been solved");
-  Dev& d = c->d;
-  CK(cudaStreamSynchronize(c->stream));
-  int b0 = c->h_bus_off[inst], nb = c->h_bus_off[inst + 1] - b0;
-  int l0 = c->h_br_off[inst], nl = c->h_br_off[inst + 1] - l0;
-  int g0 = c->h_gen_off[inst], ng = c->h_gen_off[inst + 1] - g0;
-  if (dx) {
-    std::vector<double> pg(ng), qg(ng);
-    CK(cudaMemcpy(pg.data(), d.dpg + g0, sizeof(double) * ng, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(qg.data(), d.dqg + g0, sizeof(double) * ng, cudaMemcpyDeviceToHost));
-    for (int q = 0; q < ng; ++q) {
-      int internal = c->h_gen_iperm[g0 + q] - g0;
-      dx[q] = pg[internal];
-      dx[ng + q] = qg[internal];
-    }
-    double* w = dx + 2 * ng;
-    CK(cudaMemcpy(w, d.dw + b0, sizeof(double) * nb, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(w + nb, d.dth + b0, sizeof(double) * nb, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(w + 2 * nb, d.dwr + l0, sizeof(double) * nl, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(w + 2 * nb + nl, d.dwi + l0, sizeof(double) * nl, cudaMemcpyDeviceToHost));
+  if (!dx && !pi) {
+    CK(cudaStreamSynchronize(c->stream));
+    return ACOPF_OK;
   }
-  if (pi) {
-    std::vector<double> col(nl);
-    for (int r = 0; r < 4; ++r) {
-      CK(cudaMemcpy(col.data(), d.pi_new + (size_t)r * d.L + l0, sizeof(double) * nl, cudaMemcpyDeviceToHost));
-      for (int l = 0; l < nl; ++l) pi[4 * l + r] = col[l];
-    }
-  }
+  const Dev& d = c->d;
+  acopf_status s = stage_instance(c, inst, PackSrc{d.dpg, d.dqg, d.dw, d.dth, d.dwr, d.dwi, pi ? d.pi_new : nullptr});
+  if (s) return s;
+  const size_t nl = c->h_br_off[inst + 1] - c->h_br_off[inst];
+  const size_t nx = 2 * (size_t)(c->h_gen_off[inst + 1] - c->h_gen_off[inst]) +
+                    2 * (size_t)(c->h_bus_off[inst + 1] - c->h_bus_off[inst]) + 2 * nl;
+  if (dx) memcpy(dx, c->h_stage, sizeof(double) * nx);
+  if (pi) memcpy(pi, c->h_stage + nx, sizeof(double) * 4 * nl);
   return ACOPF_OK;
 }
 
@@ -1300,10 +1294,10 @@ acopf_status acopf_get_solution(acopf_handle h, int32_t inst, acopf_solution* ou
   int nb = c->h_bus_off[inst + 1] - c->h_bus_off[inst];
   int nl = c->h_br_off[inst + 1] - c->h_br_off[inst];
   int ng = c->h_gen_off[inst + 1] - c->h_gen_off[inst];
-  std::vector<double> x(2 * (size_t)ng + 2 * (size_t)nb + 2 * (size_t)nl);
-  acopf_status s = acopf_get_iterate(h, inst, x.data(), nullptr);
+  const Dev& d = c->d;
+  acopf_status s = stage_instance(c, inst, PackSrc{d.pg, d.qg, d.w, d.th, d.wr, d.wi, nullptr});
   if (s) return s;
-  const double* v = x.data();
+  const double* v = c->h_stage;
   if (out->pg) memcpy(out->pg, v, sizeof(double) * ng);
   if (out->qg) memcpy(out->qg, v + ng, sizeof(double) * ng);
   const double* w = v + 2 * ng;
@@ -1312,9 +1306,7 @@ acopf_status acopf_get_solution(acopf_handle h, int32_t inst, acopf_solution* ou
   if (out->va) memcpy(out->va, w + nb, sizeof(double) * nb);
   if (out->wr) memcpy(out->wr, w + 2 * nb, sizeof(double) * nl);
   if (out->wi) memcpy(out->wi, w + 2 * nb + nl, sizeof(double) * nl);
-  InstCtl q;
-  CK(cudaMemcpy(&q, c->d.ctl + inst, sizeof(q), cudaMemcpyDeviceToHost));
-  out->obj = q.obj;
+  out->obj = w[2 * nb + 2 * nl];  // the value after the variables
   return ACOPF_OK;
 }
 
@@ -1409,10 +1401,6 @@ acopf_status acopf_set_warm_start_device(acopf_handle h, const float* pred, int6
       return fail(c, ACOPF_EINVAL, "acopf_set_warm_start_device: instances of different sizes");
   const int64_t width = 5LL * ng + 2LL * nb + 15LL * nl;
   if (ld < width) return fail(c, ACOPF_EINVAL, "acopf_set_warm_start_device: ld below the row width 5G + 2B + 15L");
-  if (!c->d_gen_iperm) {
-    CK(dalloc(c, &c->d_gen_iperm, (size_t)c->d.G));
-    CK(upload(c, c->d_gen_iperm, c->h_gen_iperm, (size_t)c->d.G));
-  }
   launch_warm_scatter(*c, pred, ld, nb, nl, ng, base_rho, use_x, use_pi, use_lambda, use_rho);
   CK(cudaGetLastError());
   if (use_x) c->warm_x = true;

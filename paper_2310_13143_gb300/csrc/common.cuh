@@ -213,7 +213,7 @@ struct Ctx {
   std::vector<int> h_task_off, h_big_off;  // host copies of d.task_off, d.big_off
   // warm start staged by acopf_set_warm_start / acopf_set_warm_start_device
   bool warm_x = false, warm_lam = false, warm_rho = false;
-  int* d_gen_iperm = nullptr;  // device copy of h_gen_iperm (allocated on first use)
+  int* d_gen_iperm = nullptr;  // device copy of h_gen_iperm
   // CUDA graph of one SQP iteration (sqp_solve_graph)
   bool capturing = false;          // launches are being captured: no host reads, no per-sweep error reset
   cudaGraph_t graph = nullptr;
@@ -221,6 +221,11 @@ struct Ctx {
   sqp_options gopts{};             // options the graph was captured with
   int gkernels = 0;                // kernel nodes per replay
   int* h_running = nullptr;        // pinned host copy of n_running
+  // read-outs (acopf_get_iterate, _step, _solution): pinned host memory that
+  // k_pack writes one instance's values into; as large as the largest instance
+  // read so far needs, freed with the handle
+  double* h_stage = nullptr;
+  size_t stage_values = 0;
   cudaStream_t gstream = nullptr;  // capture stream when the handle has none
 };
 
@@ -234,6 +239,11 @@ void launch_step(Ctx& c, int pass = 0);
 void launch_merit(Ctx& c, int pass = 0);
 void launch_accept_and_kkt(Ctx& c);
 void launch_fill_rho(Ctx& c, double rho);
+// what a read-out packs: the six variable blocks and pi (null: left out)
+struct PackSrc {
+  const double *pg, *qg, *w, *th, *wr, *wi, *pi;
+};
+void launch_pack(Ctx& c, const PackSrc& s, int inst, double* out);
 void launch_commit_rho(Ctx& c);
 acopf_status project_linear(Ctx& c, double rho, double eps, int max_iter, int check, int* iters, double* rs);
 void launch_warm_scatter(Ctx& c, const float* pred, long long ld, int nb, int nl, int ng, double base_rho, int use_x,
