@@ -354,7 +354,8 @@ acopf_status acopf_get_profile_phases(acopf_handle h, double* ns);
 
 /* Launch shape of the ADMM sweep (the autotuner's knobs): threads per CTA
  * (32..256, multiple of 32; 0 keeps), resident CTAs per SM (0 = as many as
- * fit; -1 keeps), and how branch records reach the line solves (-1 keeps):
+ * fit; -1 keeps), and how branch records reach the line solves (-1 keeps; a
+ * new handle has 3):
  * 0 = read in place from global memory every iteration; 1 or 2 (FP32 sweep)
  * = shared-memory tile buffers filled by bulk async copies; 3 = loaded once
  * per sweep into registers, together with every other piece of static data
@@ -366,9 +367,10 @@ acopf_status acopf_get_profile_phases(acopf_handle h, double* ns);
  * barriers are the cluster's hardware barrier and whose residual maxima are
  * combined in distributed shared memory, so instances never wait on one
  * another (residual balancing off -- otherwise as with 0).  With 3 and 4 the
- * FP64 sweep sizes the grid (or cluster) for one bus task per warp where it
- * still fits: FP64 arithmetic issues at a small fraction of the FP32 rate,
- * so two tasks interleaved in a warp take twice as long as one. */
+ * FP64 sweep gives every branch four threads and every warp one bus task
+ * where the grid (or cluster) still fits, else one thread per branch: FP64
+ * arithmetic issues at a small fraction of the FP32 rate, so what counts is
+ * the number of FP64 instructions in a warp. */
 acopf_status acopf_tune(acopf_handle h, int32_t block_threads, int32_t ctas_per_sm, int32_t sweep_stages);
 
 /* Autotuner of the sweep's launch shape.  If cache_path (may be NULL) names a
