@@ -67,21 +67,22 @@ static void release_block(const Ctx::Block& b) {
   else cudaFree(b.p);
 }
 
-// a zeroed block owned by the handle; *slot (a field of the handle) points to it
-static cudaError_t dalloc_bytes(Ctx* c, void** slot, size_t bytes) {
+// a block owned by the handle, zeroed unless the caller fills all of it;
+// *slot (a field of the handle) points to it
+static cudaError_t dalloc_bytes(Ctx* c, void** slot, size_t bytes, bool zero = true) {
   if (c->nblocks >= (int)(sizeof(c->blocks) / sizeof(c->blocks[0]))) return cudaErrorInvalidValue;
   void* v = nullptr;
   cudaError_t e = ctx_alloc(*c, &v, bytes);
   if (e != cudaSuccess) return e;
-  cudaMemsetAsync(v, 0, bytes, c->stream);
+  if (zero) cudaMemsetAsync(v, 0, bytes, c->stream);
   c->blocks[c->nblocks++] = Ctx::Block{v, bytes, slot, c->ualloc ? c->ufree : nullptr, c->uctx};
   *slot = v;
   return cudaSuccess;
 }
 
 template <typename P>
-static cudaError_t dalloc(Ctx* c, P** p, size_t count) {
-  return dalloc_bytes(c, (void**)p, sizeof(P) * (count > 0 ? count : 1));
+static cudaError_t dalloc(Ctx* c, P** p, size_t count, bool zero = true) {
+  return dalloc_bytes(c, (void**)p, sizeof(P) * (count > 0 ? count : 1), zero);
 }
 
 template <typename P>
@@ -462,18 +463,19 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   cudaError_t e = cudaSuccess;
   size_t T = c->precision == ACOPF_MIXED ? sizeof(float) : sizeof(double);
 #define A(ptr, n) if (e == cudaSuccess) e = dalloc(c, &(ptr), (n))
-  A(d.bus_off, K + 1); A(d.br_off, K + 1); A(d.gen_off, K + 1); A(c->d_gen_iperm, G);
-  A(d.bus_inst, B); A(d.br_inst, L); A(d.gen_inst, G);
-  A(d.pd, B); A(d.qd, B); A(d.gs, B); A(d.bs, B); A(d.wmin, B); A(d.wmax, B); A(d.isref, B);
-  A(d.end_ptr, B + 1); A(d.end_idx, 2 * (size_t)L); A(d.gen_ptr, B + 1);
-  A(d.ent, E); A(d.ebus, E); A(d.pent, pent.size()); A(d.pbus, pbus.size()); A(d.pmeta, pmeta.size());
-  A(d.tinst, tinst.size());
-  A(d.big, big.size()); A(d.task_off, K + 1); A(d.big_off, K + 1); A(d.wset, L);
+#define AU(ptr, n) if (e == cudaSuccess) e = dalloc(c, &(ptr), (n), false)  // uploaded below
+  AU(d.bus_off, K + 1); AU(d.br_off, K + 1); AU(d.gen_off, K + 1); AU(c->d_gen_iperm, G);
+  AU(d.bus_inst, B); AU(d.br_inst, L); AU(d.gen_inst, G);
+  AU(d.pd, B); AU(d.qd, B); AU(d.gs, B); AU(d.bs, B); AU(d.wmin, B); AU(d.wmax, B); AU(d.isref, B);
+  AU(d.end_ptr, B + 1); AU(d.end_idx, 2 * (size_t)L); AU(d.gen_ptr, B + 1);
+  AU(d.ent, E); AU(d.ebus, E); AU(d.pent, pent.size()); AU(d.pbus, pbus.size()); AU(d.pmeta, pmeta.size());
+  AU(d.tinst, tinst.size());
+  AU(d.big, big.size()); AU(d.task_off, K + 1); AU(d.big_off, K + 1); A(d.wset, L);
   d.E = (int)E;
   d.NT = (int)(pbus.size() / 32);
   d.NBIG = (int)(big.size() / 2);
-  A(d.f, L); A(d.t, L); A(d.Y, 8 * (size_t)L); A(d.s2, L); A(d.angmin, L); A(d.angmax, L);
-  A(d.gbus, G); A(d.pmin, G); A(d.pmax, G); A(d.qmin, G); A(d.qmax, G); A(d.cq, G); A(d.cl, G); A(d.cc, G);
+  AU(d.f, L); AU(d.t, L); A(d.Y, 8 * (size_t)L); AU(d.s2, L); AU(d.angmin, L); AU(d.angmax, L);
+  AU(d.gbus, G); AU(d.pmin, G); AU(d.pmax, G); AU(d.qmin, G); AU(d.qmax, G); AU(d.cq, G); AU(d.cl, G); AU(d.cc, G);
   A(d.pg, G); A(d.qg, G); A(d.w, B); A(d.th, B); A(d.wr, L); A(d.wi, L); A(d.pi, 4 * (size_t)L);
   A(d.dpg, G); A(d.dqg, G); A(d.dw, B); A(d.dth, B); A(d.dwr, L); A(d.dwi, L); A(d.pi_new, 4 * (size_t)L);
   A(d.flow, 4 * (size_t)L); A(d.aR, 4 * (size_t)L); A(d.aI, 4 * (size_t)L); A(d.bR, L); A(d.bI, L);
@@ -493,6 +495,7 @@ acopf_status acopf_create(const acopf_grid* grids, int32_t ngrids, const acopf_o
   A(d.dend, 2 * 2 * (size_t)L); A(d.red, 16 * (size_t)K); A(d.ctl, K); A(d.n_running, 1);
   A(d.hist, (size_t)K * ACOPF_HIST_MAX * kHistW); A(d.rho_fac, K); A(d.phase_ns, 4);
 #undef A
+#undef AU
 #undef AR
   double *d_r = nullptr, *d_x = nullptr, *d_b = nullptr, *d_tap = nullptr, *d_sh = nullptr;
   if (e == cudaSuccess) e = cudaMalloc(&d_r, sizeof(double) * 5 * (size_t)(L > 0 ? L : 1));
@@ -1142,7 +1145,10 @@ acopf_status acopf_get_qp(acopf_handle h, int32_t inst, acopf_qp_view* v) {
   int l0 = c->h_br_off[inst], nl = c->h_br_off[inst + 1] - l0;
   int g0 = c->h_gen_off[inst], ng = c->h_gen_off[inst + 1] - g0;
   std::vector<double> br((size_t)110 * nl), gn((size_t)6 * ng), bu((size_t)2 * nb);
-  if (nl) CK(cudaMemcpy(br.data(), d.xbr + (size_t)110 * l0, sizeof(double) * br.size(), cudaMemcpyDeviceToHost));
+  // the instance's part of each of the 110 value rows (value k of branch l at xbr[k L + l])
+  if (nl)
+    CK(cudaMemcpy2D(br.data(), sizeof(double) * nl, d.xbr + l0, sizeof(double) * (size_t)d.L, sizeof(double) * nl, 110,
+                    cudaMemcpyDeviceToHost));
   CK(cudaMemcpy(gn.data(), d.xgen + (size_t)6 * g0, sizeof(double) * gn.size(), cudaMemcpyDeviceToHost));
   CK(cudaMemcpy(bu.data(), d.xbus + (size_t)2 * b0, sizeof(double) * bu.size(), cudaMemcpyDeviceToHost));
   struct F { double* dst; int off, n; } fs[] = {{v->flow, 0, 4}, {v->H, 4, 36}, {v->aR, 40, 4}, {v->aI, 44, 4},
@@ -1152,7 +1158,7 @@ acopf_status acopf_get_qp(acopf_handle h, int32_t inst, acopf_qp_view* v) {
   for (auto& fld : fs) {
     if (!fld.dst) continue;
     for (int l = 0; l < nl; ++l)
-      for (int k = 0; k < fld.n; ++k) fld.dst[(size_t)fld.n * l + k] = br[(size_t)110 * l + fld.off + k];
+      for (int k = 0; k < fld.n; ++k) fld.dst[(size_t)fld.n * l + k] = br[(size_t)(fld.off + k) * nl + l];
   }
   if (v->gen)
     for (int q = 0; q < ng; ++q) {
