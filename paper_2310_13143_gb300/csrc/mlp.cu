@@ -84,6 +84,16 @@ struct Epi {
 };
 
 // --------------------------------------------------------------- PTX helpers
+// Programmatic dependent launch: every kernel of a step is launched so that it
+// may start while the one before it still runs.  It lets its own successor
+// start (pdl_go), sets up what touches no global memory, and then waits until
+// the kernel before it has completed and its writes are visible (pdl_wait);
+// every kernel waits, so completion carries over from one to the next.  The
+// gaps and prologues between the small kernels of a step were a third of its
+// time: 64 steps of the 30-bus network 7.8 -> 6.6 ms, a prediction for one
+// scenario 73 -> 61 us.
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t n) {
@@ -352,6 +362,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint64_t* tempty = tfull + 2;      // accumulator a has been read by the epilogue
   uint32_t* tslot = (uint32_t*)(tempty + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_go();
   const int mt = (e.M + BM - 1) / BM, nt = (e.N + bn - 1) / bn;
   const int items = splits * mt * nt;
   const uint32_t bbytes = (uint32_t)bn * BK * 2;
@@ -378,6 +389,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {  // producer: operand tiles into the ring of stages
@@ -507,6 +519,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   uint64_t* tfull = empty + kSmallStages;
   uint32_t* tslot = (uint32_t*)(tfull + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_go();
   const int second = (int)blockIdx.x >= p.first1;
   const SmallG& g = p.g[second];
   const int item = (int)blockIdx.x - (second ? p.first1 : 0);
@@ -532,6 +545,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {  // producer
@@ -605,6 +619,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 
 // sum of the K-split partial tiles, then the epilogue
 __global__ void k_splitk(const float* ws, int splits, size_t stride, Epi e) {
+  pdl_go();
+  pdl_wait();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   size_t total = (size_t)e.M * e.N;
   if (i >= total) return;
@@ -623,6 +639,8 @@ __global__ void k_splitk(const float* ws, int splits, size_t stride, Epi e) {
 __global__ void __launch_bounds__(256) k_input(const float* X, const int* idx, int rows, int Mb, int d0,
                                                const float* mu, const float* sd, bf16* A, bf16* AT) {
   __shared__ bf16 tile[32][34];
+  pdl_go();
+  pdl_wait();
   const int j = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 32;
   const float m = j < d0 ? mu[j] : 0.0f, s = j < d0 ? sd[j] : 1.0f;
 #pragma unroll
@@ -665,6 +683,8 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
   __shared__ __align__(4) bf16 tile[kMseCols][kMseRows + 2];  // [column][row]
   __shared__ double red[256];
   __shared__ bool last;
+  pdl_go();
+  pdl_wait();
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;  // columns n0 + 2 x, + 1; rows y, y + 8, ...
   const int n0 = blockIdx.x * kMseCols, n = n0 + 2 * x;
   const bool in = n < N;  // N is a multiple of 8: both columns or none
@@ -778,6 +798,8 @@ __device__ __forceinline__ float adam_one(const AdamP& p, float g, float& m, flo
 __global__ void __launch_bounds__(256) k_adam(const __grid_constant__ AdamP p) {
   __shared__ __align__(4) bf16 tile[kAdamTile][kAdamTile + 2];
   const int blk = blockIdx.x, t = threadIdx.x;
+  pdl_go();
+  pdl_wait();
   if (blk >= p.l[0].bias0) {
     int q = p.nl - 1;
     while (q > 0 && blk < p.l[q].bias0) --q;
@@ -922,6 +944,22 @@ struct Gemm {
   int bn = BN;         // rows of tb's boxes: 64 for k_gemm_small, else the tile width of k_gemm_tc
 };
 
+// launch with programmatic dependence on the kernel before it in the stream
+template <typename... P, typename... A>
+static cudaError_t launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, P(a)...);
+}
+
 // dynamic shared memory of the two kernels, once per device and thread of the caller
 static cudaError_t set_smem() {
   static thread_local int done = -1;
@@ -965,8 +1003,7 @@ static cudaError_t run_small(const Gemm& a, const Gemm* b, int* err, cudaStream_
   p.g[1] = b ? small_of(*b) : p.g[0];
   p.first1 = p.g[0].mt * ((a.N + SN - 1) / SN);
   const int grid = p.first1 + (b ? p.g[1].mt * ((b->N + SN - 1) / SN) : 0);
-  k_gemm_small<<<grid, kSmallThreads, kSmallSmem, st>>>(p, err, spin);
-  return cudaGetLastError();
+  return launch(k_gemm_small, grid, kSmallThreads, kSmallSmem, st, p, err, spin);
 }
 
 static cudaError_t run_gemm(const Gemm& g, float* ws, int* err, cudaStream_t st, long long spin, int sms) {
@@ -976,18 +1013,17 @@ static cudaError_t run_gemm(const Gemm& g, float* ws, int* err, cudaStream_t st,
   const int items = g.splits * ((g.e.M + BM - 1) / BM) * ((g.N + g.bn - 1) / g.bn);
   const int grid = items < sms ? items : sms;
   if (g.splits == 1) {
-    k_gemm_tc<<<grid, kGemmThreads, kGemmSmem, st>>>(g.ta, g.tb, g.K, g.kts, 1, g.bn, g.e, err, spin);
-    return cudaGetLastError();
+    return launch(k_gemm_tc, grid, kGemmThreads, kGemmSmem, st, g.ta, g.tb, g.K, g.kts, 1, g.bn, g.e, err, spin);
   }
   Epi p = g.e;
   p.op = EPI_PARTIAL;
   p.f32 = ws;
   p.ld_f32 = g.N;
   p.split_stride = (size_t)g.M * g.N;
-  k_gemm_tc<<<grid, kGemmThreads, kGemmSmem, st>>>(g.ta, g.tb, g.K, g.kts, g.splits, g.bn, p, err, spin);
+  c = launch(k_gemm_tc, grid, kGemmThreads, kGemmSmem, st, g.ta, g.tb, g.K, g.kts, g.splits, g.bn, p, err, spin);
+  if (c != cudaSuccess) return c;
   size_t total = (size_t)g.e.M * g.N;
-  k_splitk<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(ws, g.splits, p.split_stride, g.e);
-  return cudaGetLastError();
+  return launch(k_splitk, (unsigned)((total + 255) / 256), 256, 0, st, (const float*)ws, g.splits, p.split_stride, g.e);
 }
 
 // K split so that the grid covers the GPU's SMs about once
@@ -1380,9 +1416,8 @@ acopf_status acopf_mlp_forward(acopf_mlp_handle h, const float* X, int32_t rows,
   const int d0 = n->dims[0], dn = n->dims[n->nl];
   for (int r0 = 0; r0 < rows; r0 += n->Mb) {
     int rr = rows - r0 < n->Mb ? rows - r0 : n->Mb;
-    k_input<<<dim3((d0 + 31) / 32, (rr + BM - 1) / BM * (BM / 32)), dim3(32, 8), 0, n->stream>>>(
-        X + (size_t)r0 * d0, nullptr, rr, n->Mb, d0, n->mu_x, n->sd_x, n->A[0], nullptr);
-    NCK(cudaGetLastError());
+    NCK(launch(k_input, dim3((d0 + 31) / 32, (rr + BM - 1) / BM * (BM / 32)), dim3(32, 8), 0, n->stream,
+               X + (size_t)r0 * d0, (const int*)nullptr, rr, n->Mb, d0, n->mu_x, n->sd_x, n->A[0], (bf16*)nullptr));
     acopf_status s = forward(n, rr, Y + (size_t)r0 * dn);
     if (s) return s;
   }
@@ -1395,14 +1430,12 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
   if (!n || !X || !T || rows < 1 || rows > n->Mb || !(lr > 0)) return nfail(n, ACOPF_EINVAL, "mlp_train_step: bad arguments");
   cudaSetDevice(n->device);
   const int nl = n->nl, Mb = n->Mb, d0 = n->dims[0], dn = n->dims[nl];
-  k_input<<<dim3((d0 + 31) / 32, Mb / 32), dim3(32, 8), 0, n->stream>>>(X, idx, rows, Mb, d0, n->mu_x, n->sd_x,
-                                                                        n->A[0], n->AT[0]);
-  NCK(cudaGetLastError());
+  NCK(launch(k_input, dim3((d0 + 31) / 32, Mb / 32), dim3(32, 8), 0, n->stream, X, idx, rows, Mb, d0, n->mu_x,
+             n->sd_x, n->A[0], n->AT[0]));
   acopf_status s = forward(n, rows);
   if (s) return s;
-  k_mse<<<n->nparts, 256, 0, n->stream>>>(n->Y, T, idx, rows, Mb, dn, n->mu_y, n->sd_y, n->D[nl], n->DT[nl],
-                                          n->L[nl - 1].gb, n->part, n->done, n->loss, loss);
-  NCK(cudaGetLastError());
+  NCK(launch(k_mse, n->nparts, 256, 0, n->stream, n->Y, T, idx, rows, Mb, dn, n->mu_y, n->sd_y, n->D[nl], n->DT[nl],
+             n->L[nl - 1].gb, n->part, n->done, n->loss, loss));
   for (int l = nl - 1; l >= 0; --l) {
     const Gemm &w = n->bwd_w[l], &x = n->bwd_x[l];
     if (l >= 1 && w.small && x.small) {
@@ -1431,8 +1464,7 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
     p.l[l].bias0 = blocks;
     blocks += (n->L[l].out + kAdamBias - 1) / kAdamBias;
   }
-  k_adam<<<blocks, 256, 0, n->stream>>>(p);
-  NCK(cudaGetLastError());
+  NCK(launch(k_adam, blocks, 256, 0, n->stream, p));
   return ACOPF_OK;
 }
 
