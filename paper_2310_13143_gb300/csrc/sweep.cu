@@ -1359,7 +1359,10 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
         }
       }
     } else if (!kTiled) {
-      for (int u = tid; u < d.G + d.L; u += nthreads) {
+      // warps take runs of 32 components round the CTAs, so that the last,
+      // partial pass is spread over all SMs (in CTA order it went to the first
+      // CTAs only, and the others waited for half a pass)
+      for (int u = (((int)threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x) * 32 + lane; u < d.G + d.L; u += nthreads) {
         if (u < d.G) {
           int k = d.gen_inst[u];
           if (!s_done[k]) gen_phase(p, u, s_scale[k]);
@@ -1446,20 +1449,25 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
         bus_task_pair(d, task_load<T, true, true>(d, ta, s_done), task_load<T, true, true>(d, tb, s_done), dst);
       }
     } else {
+      // a CTA takes a contiguous run of tasks, whose warps gather from
+      // neighbouring branches at the same time; the runs differ by one task
+      const int tb = (int)((long long)d.NT * blockIdx.x / gridDim.x),
+                te = (int)((long long)d.NT * (blockIdx.x + 1) / gridDim.x);
+      const int wpb = blockDim.x >> 5, tw = tb + (threadIdx.x >> 5);
       if (fresh)
-        for (int t = wid; t < d.NT; t += nw) task_fresh<T>(d, t, lane);
-      auto slot_at = [&](int t) { return t < d.NT ? load_slot(d, t, lane) : none; };
-      // tasks wid, wid + nw, ... taken two at a time; the slots of the next
-      // pair are in flight while a pair is solved
-      Slot s1a = slot_at(wid + 2 * nw), s1b = slot_at(wid + 3 * nw);
-      TaskData<T> ca = task_load<T, true, false>(d, task_stream<T>(d, slot_at(wid)), s_done);
-      TaskData<T> cb = task_load<T, true, false>(d, task_stream<T>(d, slot_at(wid + nw)), s_done);
-      for (int t = wid; t < d.NT; t += 2 * nw) {
+        for (int t = tw; t < te; t += wpb) task_fresh<T>(d, t, lane);
+      auto slot_at = [&](int t) { return t < te ? load_slot(d, t, lane) : none; };
+      // the warp's tasks two at a time; the slots of the next pair are in
+      // flight while a pair is solved
+      Slot s1a = slot_at(tw + 2 * wpb), s1b = slot_at(tw + 3 * wpb);
+      TaskData<T> ca = task_load<T, true, false>(d, task_stream<T>(d, slot_at(tw)), s_done);
+      TaskData<T> cb = task_load<T, true, false>(d, task_stream<T>(d, slot_at(tw + wpb)), s_done);
+      for (int t = tw; t < te; t += 2 * wpb) {
         bus_task_pair(d, ca, cb, dst);
         ca = task_load<T, true, false>(d, task_stream<T>(d, s1a), s_done);
         cb = task_load<T, true, false>(d, task_stream<T>(d, s1b), s_done);
-        s1a = slot_at(t + 4 * nw);
-        s1b = slot_at(t + 5 * nw);
+        s1a = slot_at(t + 4 * wpb);
+        s1b = slot_at(t + 5 * wpb);
       }
     }
     for (int b = wid; b < d.NBIG; b += nw)
