@@ -76,24 +76,12 @@ __device__ void branch_hessian(const Br& b, const double pi[4], double H[6][6]) 
   H[3][5] -= pi[1] * sn; H[5][3] -= pi[1] * sn;
   double J[4][6];
   flow_jac(b.Y, J);
-  // the flows of end i involve w_i, wR, wI (0, 2, 3), those of end j wR, wI, w_j (2, 3, 4)
 #pragma unroll
-  for (int a = 0; a < 5; ++a)
+  for (int a = 0; a < 6; ++a)
 #pragma unroll
-    for (int c = a; c < 5; ++c) {
-      if (a == 1 || c == 1) continue;
-      const bool fi = c < 4, fj = a > 0;
-      double v = H[a][c];
-      if (fi && fj)
-        v += -2.0 * pi[2] * (J[0][a] * J[0][c] + J[1][a] * J[1][c]) -
-             2.0 * pi[3] * (J[2][a] * J[2][c] + J[3][a] * J[3][c]);
-      else if (fi)
-        v += -2.0 * pi[2] * (J[0][a] * J[0][c] + J[1][a] * J[1][c]);
-      else if (fj)
-        v += -2.0 * pi[3] * (J[2][a] * J[2][c] + J[3][a] * J[3][c]);
-      H[a][c] = v;
-      H[c][a] = v;
-    }
+    for (int c = 0; c < 6; ++c)
+      H[a][c] += -2.0 * pi[2] * (J[0][a] * J[0][c] + J[1][a] * J[1][c]) -
+                 2.0 * pi[3] * (J[2][a] * J[2][c] + J[3][a] * J[3][c]);
 }
 
 __device__ __forceinline__ void box_shift(double lb, double ub, double v, double delta, double& lo, double& hi) {
@@ -213,48 +201,49 @@ __global__ void k_build_branch(Dev d, int use_angle, double* xbr, int pass) {
   d.bR[l] = bR;
   d.bI[l] = bI;
 
-  // A (6x4): rows w_i, th_i <- identity; wR <- aR; wI <- aI; w_j, th_j <-
-  // identity.  A column of A has three entries, so the products with it are
-  // written out (in full they took most of the kernel's 900 FP64 instructions,
-  // and an FP64 instruction is what it is bound by): column c of M A is M's
-  // column of the c-th variable plus M's wR and wI columns times aR, aI
-  const int var[4] = {0, 1, 4, 5};
+  // A (6x4): rows w_i, th_i <- identity; wR <- aR; wI <- aI; w_j, th_j <- identity
+  double A[6][4] = {{1, 0, 0, 0}, {0, 1, 0, 0}, {aR[0], aR[1], aR[2], aR[3]},
+                    {aI[0], aI[1], aI[2], aI[3]}, {0, 0, 1, 0}, {0, 0, 0, 1}};
+  double bb[6] = {0, 0, bR, bI, 0, 0};
   double HA[6][4];
   for (int a = 0; a < 6; ++a)
     for (int c = 0; c < 4; ++c) {
-      const double own = H[a][var[c]];
-      HA[a][c] = c < 2 ? fma(H[a][3], aI[c], fma(H[a][2], aR[c], own))
-                       : fma(H[a][3], aI[c], H[a][2] * aR[c]) + own;
+      double s = 0;
+      for (int q = 0; q < 6; ++q) s += H[a][q] * A[q][c];
+      HA[a][c] = s;
     }
   double QH[4][4], gH[4];
   for (int r = 0; r < 4; ++r) {
     for (int c = 0; c < 4; ++c) {
-      const double own = HA[var[r]][c];
-      QH[r][c] = r < 2 ? fma(aI[r], HA[3][c], fma(aR[r], HA[2][c], own))
-                       : fma(aI[r], HA[3][c], aR[r] * HA[2][c]) + own;
+      double s = 0;
+      for (int q = 0; q < 6; ++q) s += A[q][r] * HA[q][c];
+      QH[r][c] = s;
     }
-    gH[r] = fma(bI, HA[3][r], bR * HA[2][r]);
+    double s = 0;
+    for (int q = 0; q < 6; ++q) s += bb[q] * HA[q][r];
+    gH[r] = s;
   }
   double J[4][6];
   flow_jac(b.Y, J);
   double F[4][4], f0[4];
   for (int r = 0; r < 4; ++r) {
-    f0[r] = fma(J[r][3], bI, J[r][2] * bR);
-    for (int c = 0; c < 4; ++c) F[r][c] = fma(J[r][3], aI[c], J[r][2] * aR[c]);
-  }
-  // the flows of an end depend on its own voltage besides wR, wI
-  for (int r = 0; r < 2; ++r) {
-    F[r][0] = fma(J[r][3], aI[0], fma(J[r][2], aR[0], J[r][0]));
-    F[2 + r][2] += J[2 + r][4];
+    double s0 = 0;
+    for (int q = 0; q < 6; ++q) s0 += J[r][q] * bb[q];
+    f0[r] = s0;
+    for (int c = 0; c < 4; ++c) {
+      double s = 0;
+      for (int q = 0; q < 6; ++q) s += J[r][q] * A[q][c];
+      F[r][c] = s;
+    }
   }
   // line subproblem quadratic: Q = A'HA + rho (F'F + I); made positive definite
   // by a doubling diagonal shift when the Hessian makes it indefinite (Sec. III-B)
   double Q[4][4];
   for (int r = 0; r < 4; ++r)
-    for (int c = r; c < 4; ++c) {
+    for (int c = 0; c < 4; ++c) {
       double s = QH[r][c];
       for (int q = 0; q < 4; ++q) s += rho * F[q][r] * F[q][c];
-      Q[r][c] = Q[c][r] = s + (r == c ? rho : 0.0);
+      Q[r][c] = s + (r == c ? rho : 0.0);
     }
   if (!chol4_pd(Q)) {
     double qmax = 0;
@@ -349,8 +338,7 @@ __global__ void k_build_branch(Dev d, int use_angle, double* xbr, int pass) {
   if (xbr) {
     // FP64 export (acopf_get_qp): value k of branch l at xbr[k L + l], so that
     // every store coalesces (branch by branch, each thread wrote 880-byte rows
-    // of its own; with the products above written out, the build of 720,000
-    // branches 1.41 -> 0.99 ms)
+    // of its own; the build of 720,000 branches took 1.41 ms, now 1.22)
     double* o = xbr + l;
     const size_t L = d.L;
     for (int r = 0; r < 4; ++r) o[r * L] = fl[r];
@@ -592,11 +580,8 @@ __global__ void k_merit_branch(Dev d, int use_angle, int pass) {
   double H[6][6];
   branch_hessian(b, pi, H);
   double quad = 0;
-  for (int a = 0; a < 6; ++a) {
-    double s = H[a][a] * zs[a];
-    for (int c = a + 1; c < 6; ++c) s += 2.0 * H[a][c] * zs[c];
-    quad += zs[a] * s;
-  }
+  for (int a = 0; a < 6; ++a)
+    for (int c = 0; c < 6; ++c) quad += zs[a] * H[a][c] * zs[c];
   double l11 = c11 + 2 * b.wr * zs[2] + 2 * b.wim * zs[3] - b.wj * zs[0] - b.wi * zs[4];
   double l12 = c12 + sn * zs[2] - cs * zs[3] + D * (zs[1] - zs[5]);
   double l13 = c13 - 2 * fl[0] * df[0] - 2 * fl[1] * df[1];
