@@ -215,6 +215,7 @@ struct Ctx {
   int sweep_stages = 3;
   int cluster_cs = 1;         // cluster size of sweep_stages 4, chosen for
   int cluster_threads = -1;   // this CTA size (-1: not chosen yet)
+  int cluster_exact = -1;     // and way to solve the lines (SweepP::line_exact)
   int cluster_res = 0;        // and how many threads every branch of an instance has (0: static data not in registers)
   bool cluster_dsm = false;   // and whether the state it exchanges stays in distributed shared memory
   std::vector<int> h_task_off, h_big_off;  // host copies of d.task_off, d.big_off
