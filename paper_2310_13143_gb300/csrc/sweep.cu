@@ -1283,12 +1283,18 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     mbar_init(&tbar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  int live = 0;  // whether an instance of this thread's takes part
   for (int k = threadIdx.x; k < K; k += blockDim.x) {
     s_done[k] = d.admm_done[k];
+    live += s_done[k] ? 0 : 1;
     s_scale[k] = 1.0f;
     if (s_acc) s_acc[k] = s_acc[K + k] = 0ull;
   }
-  __syncthreads();
+  // whether most instances take part: of the threads that have any, at least
+  // three in four have one that does.  Every CTA decides alike: admm_done only
+  // changes behind the first device-wide barrier
+  const int have = K < (int)blockDim.x ? K : (int)blockDim.x;
+  const bool mostly = 4 * __syncthreads_count(live > 0) >= 3 * have;
   // RES: this thread's phase-A item and its record, this warp's two bus tasks
   const int lane = threadIdx.x & 31, wid = tid >> 5, nw = nthreads >> 5;
   const Slot none = empty_slot(lane);
@@ -1458,8 +1464,11 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
       // neighbouring branches at the same time; the runs differ by one task.
       // With few tasks per warp a run's remainder would cost every CTA a round
       // of its own, so there the tasks go round all warps (64 x 2,000 buses, 5
-      // tasks per warp: 29.4 -> 27.8 us per iteration in runs)
-      const bool runs = d.NT >= 4 * nw;
+      // tasks per warp: 29.4 -> 27.8 us per iteration in runs), as they do when
+      // only a batch's last instances take part, whose tasks lie together and
+      // would all fall to a few CTAs (256 scenarios and 64 grids of 118-10,000
+      // buses solved to the end: 1,727 ms in runs throughout, 1,597 ms so)
+      const bool runs = mostly && d.NT >= 4 * nw;
       const int tb = runs ? (int)((long long)d.NT * blockIdx.x / gridDim.x) : 0;
       const int te = runs ? (int)((long long)d.NT * (blockIdx.x + 1) / gridDim.x) : d.NT;
       const int wpb = runs ? (int)blockDim.x >> 5 : nw, tw = runs ? tb + ((int)threadIdx.x >> 5) : wid;

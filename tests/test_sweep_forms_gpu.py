@@ -82,3 +82,23 @@ def test_bus_tasks_of_a_full_warp(spokes, shape, precision):
     tol = 1e-7 if precision == "fp64" else 3e-4
     for k, ok in (("x", "xl"), ("z", "zl"), ("lam", "ll"), ("zb", "zb"), ("nu", "nu")):
         np.testing.assert_allclose(got[k], st[ok], rtol=0, atol=tol * max(1.0, np.abs(st[ok]).max()), err_msg=k)
+
+
+def test_bus_tasks_of_a_batch_that_thins_out():
+    """Bus tasks in runs per CTA while most instances take part, round all
+    warps after that, or (many warps) round all warps throughout: an instance's
+    arithmetic is the same, bit for bit."""
+    grids = [gg.grid_30bus()] * 6 + gg.scenarios_cholesky(gg.grid_2000bus(), 6, 1)
+    o = binding.default_sqp(tol=1e-2, max_sqp=8, admm=dict(rho=2e4, max_iter=200, eps=1e-3, eps_dual=5e-3))
+    out = []
+    for shape in ((64, 1, 0), (256, 0, 0)):
+        s = binding.Solver(grids, precision="mixed")
+        s.tune(*shape)
+        s.sqp_solve(o)
+        out.append([(s.get_residuals(k), s.get_iterate(k)) for k in range(len(grids))])
+        s.close()
+    assert len({r["sqp_iter"] for r, _ in out[0]}) > 1  # the batch did thin out
+    for (ra, ia), (rb, ib) in zip(*out):
+        assert (ra["sqp_iter"], ra["admm_iter"]) == (rb["sqp_iter"], rb["admm_iter"])
+        for a, b in zip(ia, ib):
+            np.testing.assert_array_equal(a, b)
