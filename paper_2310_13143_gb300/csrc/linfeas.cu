@@ -24,9 +24,9 @@
 // rounding:
 //   - The branch's 4x4 matrix rho F'F + diag(rho, 2, 2, rho) does not change
 //     from one iteration to the next, and its (wR, wI) block is a multiple of
-//     the identity (the two columns of F are orthogonal and of equal norm).
-//     wR and wI have no bounds, so they are eliminated once per call; what is
-//     left per iteration is a 2-variable box QP in closed form.
+//     the identity.  wR and wI have no bounds, so they are eliminated once per
+//     call; what is left per iteration is a 2-variable box QP in closed form
+//     (linfeas_qp.cuh).
 //   - A coupling's multiplier after the bus update is -nu (branch flow) or +nu
 //     (generator) of its bus, so flows carry no multiplier of their own; the
 //     primal residual of a flow is |nu - nu_old| / rho, a bus quantity.
@@ -44,7 +44,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "line_qp.cuh"
+#include "linfeas_qp.cuh"
 
 namespace acopf {
 
@@ -56,7 +56,6 @@ __device__ __forceinline__ D4 d4(double a, double b, double c, double e) {
   return v;
 }
 
-constexpr int kLfBranch = 14;  // per branch: T (4), inverse of S (3), 1/d, 2 wR0, 2 wI0, lo and hi of w_i, w_j
 constexpr int kLfBus = 6;      // per bus: inverse of the 2x2 matrix (3), 1/Qw, M, 2 w0
 constexpr int kLfWindow = 1024;
 
@@ -74,12 +73,7 @@ struct LfState {
   unsigned long long* res;  // [2K]: per-instance max r, s (bits of non-negative doubles)
 };
 
-// Start of the iteration (x = z = x0, lambda = 0) and the constants.  With
-// v = (w_i, w_j | wR, wI) and Yij = gij + j bij, the off-diagonal block of
-// rho F'F is rho (gii gij + bii bij, gii bij - bii gij) for w_i and
-// rho (gjj gji + bjj bji, bjj gji - gjj bji) for w_j, and the (wR, wI) block
-// d I with d = rho (|Yij|^2 + |Yji|^2) + 2; T = block / d, and S is the Schur
-// complement rho (|Yii|^2 + 1) - d T_i T_i' etc.
+// Start of the iteration (x = z = x0, lambda = 0) and the constants
 __global__ void k_lf_init(Dev d, LfState s, double rho) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   const int G = d.G, B = d.B;
@@ -112,16 +106,15 @@ __global__ void k_lf_init(Dev d, LfState s, double rho) {
     s.Y[2 * n] = d4(-rho * (gii * wi + gij * wr + bij * wim), -rho * (-bii * wi - bij * wr + gij * wim), -rho * wi, 0.0);
     s.Y[2 * n + 1] =
         d4(-rho * (gjj * wj + gji * wr - bji * wim), -rho * (-bjj * wj - bji * wr - gji * wim), -rho * wj, 0.0);
-    const double dd = rho * (gij * gij + bij * bij + gji * gji + bji * bji) + 2.0;
-    const double ir = rho / dd;
-    const double tir = ir * (gii * gij + bii * bij), tii = ir * (gii * bij - bii * gij);
-    const double tjr = ir * (gjj * gji + bjj * bji), tji = ir * (bjj * gji - gjj * bji);
-    const double s11 = rho * (gii * gii + bii * bii + 1.0) - dd * (tir * tir + tii * tii);
-    const double s22 = rho * (gjj * gjj + bjj * bjj + 1.0) - dd * (tjr * tjr + tji * tji);
-    const double s12 = -dd * (tir * tjr + tii * tji);
-    const double det = s11 * s22 - s12 * s12;
-    const double c[kLfBranch] = {tir, tii, tjr, tji, s22 / det, -s12 / det, s11 / det, 1.0 / dd, 2.0 * wr, 2.0 * wim,
-                                 d.wmin[fi], d.wmax[fi], d.wmin[ti], d.wmax[ti]};
+    double c[kLfBranch] = {};
+    const double Yn[8] = {gii, bii, gij, bij, gji, bji, gjj, bjj};
+    lf_constants(Yn, rho, c);
+    c[8] = 2.0 * wr;
+    c[9] = 2.0 * wim;
+    c[10] = d.wmin[fi];
+    c[11] = d.wmax[fi];
+    c[12] = d.wmin[ti];
+    c[13] = d.wmax[ti];
 #pragma unroll
     for (int k = 0; k < kLfBranch; ++k) s.cb[k * L + n] = c[k];
   }
@@ -153,30 +146,10 @@ __global__ void __launch_bounds__(kLfWindow) k_lf_order(Dev d, int* order) {
   if (i < d.B) order[blockIdx.x * kLfWindow + atomicAdd(&cnt[key], 1)] = i;
 }
 
-// The 2-variable box QP min 1/2 w'Sw + s'w when the unconstrained minimiser
-// lies outside the box: each edge's minimiser, the one with the least
-// objective (S from its inverse a, b, c).  Out of line: few branches need it.
-__device__ __noinline__ void lf_edges(double a, double b, double c, double si, double sj, double li, double hi,
-                                      double lj, double hj, double& wi, double& wj) {
-  const double det = 1.0 / (a * c - b * b);
-  const double s11 = c * det, s12 = -b * det, s22 = a * det;
-  double best = 0.0;
-  for (int e = 0; e < 4; ++e) {
-    double u, v;
-    if (e < 2) {
-      u = e ? hi : li;
-      v = clampv(-(sj + s12 * u) / s22, lj, hj);
-    } else {
-      v = e == 3 ? hj : lj;
-      u = clampv(-(si + s12 * v) / s11, li, hi);
-    }
-    const double o = u * (0.5 * s11 * u + s12 * v + si) + v * (0.5 * s22 * v + sj);
-    if (e == 0 || o < best) {
-      best = o;
-      wi = u;
-      wj = v;
-    }
-  }
+// Out of line: few branches need it.
+__device__ __noinline__ void lf_edges_call(double l, double i1, double i2, double si, double sj, double li, double hi,
+                                           double lj, double hj, double& wi, double& wj) {
+  lf_edges(l, i1, i2, si, sj, li, hi, lj, hj, wi, wj);
 }
 
 // generators and branches (one thread each): x from y
@@ -199,18 +172,10 @@ __global__ void __launch_bounds__(128) k_lf_components(Dev d, LfState s, double 
   double c[kLfBranch];
 #pragma unroll
   for (int k = 0; k < kLfBranch; ++k) c[k] = s.cb[k * L + l];
-  // gradient at v = 0: F' y_f + (copies, -2 wR0, -2 wI0)
-  const double ci = yi.z + gii * yi.x - bii * yi.y;
-  const double cj = yj.z + gjj * yj.x - bjj * yj.y;
-  const double cr = gij * yi.x - bij * yi.y + gji * yj.x - bji * yj.y - c[8];
-  const double cm = bij * yi.x + gij * yi.y - bji * yj.x - gji * yj.y - c[9];
-  const double si = ci - c[0] * cr - c[1] * cm;
-  const double sj = cj - c[2] * cr - c[3] * cm;
-  double wi = -(c[4] * si + c[5] * sj), wj = -(c[5] * si + c[6] * sj);
-  if (!(wi >= c[10] && wi <= c[11] && wj >= c[12] && wj <= c[13]))
-    lf_edges(c[4], c[5], c[6], si, sj, c[10], c[11], c[12], c[13], wi, wj);
-  const double wr = -(c[7] * cr + c[0] * wi + c[2] * wj);
-  const double wm = -(c[7] * cm + c[1] * wi + c[3] * wj);
+  const double Yl[8] = {gii, bii, gij, bij, gji, bji, gjj, bjj}, ei[3] = {yi.x, yi.y, yi.z}, ej[3] = {yj.x, yj.y, yj.z};
+  double v[4];
+  lf_branch(Yl, c, ei, ej, v, lf_edges_call);
+  const double wi = v[0], wj = v[1], wr = v[2], wm = v[3];
   s.X[2 * l] = d4(gii * wi + gij * wr + bij * wm, gij * wm - bii * wi - bij * wr, wi, wr);
   s.X[2 * l + 1] = d4(gjj * wj + gji * wr - bji * wm, -bjj * wj - bji * wr - gji * wm, wj, wm);
 }
