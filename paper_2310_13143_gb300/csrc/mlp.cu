@@ -39,6 +39,7 @@
 
 #include "../../include/acopf.h"
 #include "../../include/acopf_mlp.h"
+#include "line_qp.cuh"
 
 namespace acopf {
 namespace nn {
@@ -671,11 +672,11 @@ __global__ void __launch_bounds__(256) k_input(const float* X, const int* idx, i
 // One block takes 64 columns over all rows, in tiles of 64 rows transposed
 // through shared memory, each thread two neighbouring columns.  It is bound by
 // its traffic (Y, T, D and D' once: 143 MB for 256 x 46,504).  The squares are
-// accumulated in FP32 pairs (products and sums exact to 2^-48, after Dekker
-// and Knuth) and enter an FP64 sum once per 16 elements: FP64 conversions and
-// additions per element took most of the former kernel's 100 us, and the
-// column sums ran as a kernel of their own (44 us).  Now 47 us for both.  The last block to finish
-// adds the blocks' sums in a fixed order.
+// summed in FP64, over the whole range of the FP32 errors; an error is widened
+// in integer operations and takes one FP64 instruction (conversions, products
+// and additions in FP64 took most of the former kernel's 100 us, and the
+// column sums ran as a kernel of their own, 44 us).  Now 47 us for both.  The
+// last block to finish adds the blocks' sums in a fixed order.
 constexpr int kMseCols = 64, kMseRows = 64;
 __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, const int* idx, int rows, int Mb, int N,
                                              const float* mu, const float* sd, bf16* D, bf16* DT, float* gb,
@@ -695,16 +696,9 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
     s = *(const float2*)(sd + n);
   }
   const float den = (float)rows * (float)N;
-  double sq = 0.0;
-  float col = 0.0f;  // threads 0..63: the sum of column n0 + threadIdx.x
+  double sq[2][2] = {};  // of the thread's two columns, two chains of additions each
+  float col = 0.0f;      // threads 0..63: the sum of column n0 + threadIdx.x
   for (int r0 = 0; r0 < Mb; r0 += kMseRows) {
-    float hs = 0.0f, ls = 0.0f;  // the squares of this tile, as a sum of two floats
-    auto add = [&](float d) {
-      const float pr = d * d, pe = fmaf(d, d, -pr);
-      const float t = hs + pr, z = t - hs;
-      ls += ((hs - (t - z)) + (pr - z)) + pe;
-      hs = t;
-    };
 #pragma unroll
     for (int k = 0; k < kMseRows; k += 8) {
       const int r = r0 + y + k;
@@ -715,8 +709,9 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
         const float2 t = vec ? *(const float2*)tp : make_float2(tp[0], tp[1]);
         const float2 yv = *(const float2*)(Y + (size_t)r * N + n);
         const float d0 = yv.x - (t.x - m.x) / s.x, d1 = yv.y - (t.y - m.y) / s.y;
-        add(d0);
-        add(d1);
+        const double w0 = f64_widen(d0), w1 = f64_widen(d1);
+        sq[k / 8 % 2][0] = fma(w0, w0, sq[k / 8 % 2][0]);
+        sq[k / 8 % 2][1] = fma(w1, w1, sq[k / 8 % 2][1]);
         g = make_float2(2.0f * d0 / den, 2.0f * d1 / den);
       }
       const __nv_bfloat162 h = __floats2bfloat162_rn(g.x, g.y);
@@ -724,7 +719,6 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
       tile[2 * x][y + k] = h.x;
       tile[2 * x + 1][y + k] = h.y;
     }
-    sq += (double)hs + (double)ls;
     __syncthreads();
     for (int c = y; c < kMseCols && n0 + c < N; c += 8)
       *(__nv_bfloat162*)(DT + (size_t)(n0 + c) * Mb + r0 + 2 * x) = *(const __nv_bfloat162*)&tile[c][2 * x];
@@ -744,7 +738,7 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
     }
     return red[0];
   };
-  const double mine = sum(sq);
+  const double mine = sum((sq[0][0] + sq[0][1]) + (sq[1][0] + sq[1][1]));
   if (threadIdx.x == 0) {
     part[blockIdx.x] = mine;
     __threadfence();

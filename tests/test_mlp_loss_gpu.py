@@ -1,0 +1,40 @@
+"""The training loss over the range of FP32: its squares are summed in FP64, so
+errors whose squares lie outside the FP32 range still give the mean's value."""
+import numpy as np
+import pytest
+
+from paper_2310_13143_gb300 import binding
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _loss(T, rows):
+    """Loss of a zero network, whose errors are -T."""
+    net = binding.Mlp([8, T.shape[1]], max_batch=rows)
+    net.set_params(np.zeros(net.nparams, np.float32))
+    X, Td = torch.zeros(rows, 8, device="cuda"), torch.from_numpy(T).cuda()
+    out = torch.full((1,), -1.0, device="cuda")
+    net.train_step(X.data_ptr(), Td.data_ptr(), None, rows, 1e-3, out.data_ptr())
+    net.sync()
+    net.close()
+    return out.item()
+
+
+@pytest.mark.parametrize("value", [1e-21, 1e-19, 3e-5, 1.0, 1e18, 2e19, 3e20])
+@pytest.mark.parametrize("rows,width", [(128, 8), (130, 200)])
+def test_loss_of_one_large_and_many_small_errors(value, rows, width):
+    rng = np.random.default_rng(rows)
+    T = (1e-3 * value * rng.standard_normal((rows, width))).astype(np.float32)
+    T[rows // 2, width // 3] = value
+    want = np.mean(T.astype(np.float64) ** 2)
+    # the FP64 mean rounded to FP32, of which a subnormal has fewer digits
+    assert abs(_loss(T, rows) - want) <= 2.0 ** -24 * want * (1 + 1e-9) + 2.0 ** -149
+
+
+def test_loss_of_infinite_and_nan_errors():
+    T = np.zeros((128, 16), np.float32)
+    T[5, 3] = np.inf
+    assert _loss(T, 128) == np.inf
+    T[5, 3] = np.nan
+    assert np.isnan(_loss(T, 128))
