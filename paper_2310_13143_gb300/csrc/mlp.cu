@@ -34,6 +34,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -669,17 +670,22 @@ __global__ void __launch_bounds__(256) k_input(const float* X, const int* idx, i
 // N) in bfloat16, row-major and transposed, the output layer's bias gradient
 // (the column sums of dY, in row order) and the loss.
 //
-// One block takes 64 columns over all rows, in tiles of 64 rows transposed
-// through shared memory, each thread two neighbouring columns.  It is bound by
-// its traffic (Y, T, D and D' once: 143 MB for 256 x 46,504).  The squares are
-// summed in FP64, over the whole range of the FP32 errors; an error is widened
+// One block takes 64 columns over a run of rows, in tiles of 64 rows
+// transposed through shared memory, each thread two neighbouring columns.
+// Where the columns alone give every SM work (mse_run) the run is all rows and
+// the block forms the bias gradient too; a narrow output layer is split over
+// grid.y, and k_adam forms it from D' as it does for the hidden layers.  Time of
+// a training step in one run and in several: 712 outputs, 16,384 rows 3.11 and
+// 0.59 ms; 20,000 outputs, 1,024 rows 388 and 320 us; 712 outputs, 100 rows 88
+// and 84 us.  The kernel is bound by its traffic (Y, T, D and D' once: 143 MB
+// for 256 x 46,504).  The squares are summed in FP64, over the whole range of the FP32 errors; an error is widened
 // in integer operations and takes one FP64 instruction (conversions, products
 // and additions in FP64 took most of the former kernel's 100 us, and the
 // column sums ran as a kernel of their own, 44 us).  Now 47 us for both.  The
 // last block to finish adds the blocks' sums in a fixed order.
 constexpr int kMseCols = 64, kMseRows = 64;
 __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, const int* idx, int rows, int Mb, int N,
-                                             const float* mu, const float* sd, bf16* D, bf16* DT, float* gb,
+                                             const float* mu, const float* sd, int run, bf16* D, bf16* DT, float* gb,
                                              double* part, unsigned* done, float* loss, float* loss_out) {
   __shared__ __align__(4) bf16 tile[kMseCols][kMseRows + 2];  // [column][row]
   __shared__ double red[256];
@@ -698,7 +704,8 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
   const float den = (float)rows * (float)N;
   double sq[2][2] = {};  // of the thread's two columns, two chains of additions each
   float col = 0.0f;      // threads 0..63: the sum of column n0 + threadIdx.x
-  for (int r0 = 0; r0 < Mb; r0 += kMseRows) {
+  const int r1 = min(Mb, ((int)blockIdx.y + 1) * run);
+  for (int r0 = blockIdx.y * run; r0 < r1; r0 += kMseRows) {
 #pragma unroll
     for (int k = 0; k < kMseRows; k += 8) {
       const int r = r0 + y + k;
@@ -722,13 +729,13 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
     __syncthreads();
     for (int c = y; c < kMseCols && n0 + c < N; c += 8)
       *(__nv_bfloat162*)(DT + (size_t)(n0 + c) * Mb + r0 + 2 * x) = *(const __nv_bfloat162*)&tile[c][2 * x];
-    if (threadIdx.x < kMseCols) {
+    if (gb && threadIdx.x < kMseCols) {
 #pragma unroll 8
       for (int r = 0; r < kMseRows; ++r) col += __bfloat162float(tile[threadIdx.x][r]);
     }
     __syncthreads();
   }
-  if (threadIdx.x < kMseCols && n0 + (int)threadIdx.x < N) gb[n0 + threadIdx.x] = col;
+  if (gb && threadIdx.x < kMseCols && n0 + (int)threadIdx.x < N) gb[n0 + threadIdx.x] = col;
   auto sum = [&](double v) {
     red[threadIdx.x] = v;
     __syncthreads();
@@ -740,15 +747,15 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
   };
   const double mine = sum((sq[0][0] + sq[0][1]) + (sq[1][0] + sq[1][1]));
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = mine;
+    part[blockIdx.y * gridDim.x + blockIdx.x] = mine;
     __threadfence();
-    last = atomicAdd(done, 1u) == gridDim.x - 1;
+    last = atomicAdd(done, 1u) == gridDim.x * gridDim.y - 1;
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
   double t = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) t += ((volatile double*)part)[i];
+  for (int i = threadIdx.x; i < (int)(gridDim.x * gridDim.y); i += 256) t += ((volatile double*)part)[i];
   const double total = sum(t);
   if (threadIdx.x == 0) {
     const float v = (float)(total * (1.0 / ((double)rows * N)));
@@ -756,6 +763,14 @@ __global__ void __launch_bounds__(256) k_mse(const float* Y, const float* T, con
     if (loss_out) *loss_out = v;
     *done = 0u;  // for the next launch
   }
+}
+
+// rows per block of k_mse: all of them where that makes four blocks per SM, else
+// as many runs of whole tiles as make up for it
+static int mse_run(int N, int Mb, int sms) {
+  const int cols = (N + kMseCols - 1) / kMseCols, tiles = Mb / kMseRows;
+  const int runs = std::min(tiles, (4 * sms + cols - 1) / cols);
+  return (tiles + runs - 1) / runs * kMseRows;
 }
 
 // Adam (bias-corrected) on every parameter of the network in one launch: FP32
@@ -773,7 +788,7 @@ constexpr int kAdamTile = 64, kAdamBias = 64;  // tile edge; biases per block
 struct AdamLayer {
   float *W, *G, *mW, *vW, *b, *gb, *mb, *vb;
   bf16 *W16, *W16T;
-  const bf16* DT;  // hidden layers: D' [out x rows], null where gb is already formed
+  const bf16* DT;  // D' [out x rows], null where gb is already formed
   int in, out;
   int block0, bias0;  // first weight block, first bias block
 };
@@ -1090,7 +1105,7 @@ struct Net {
   float* ws = nullptr;
   size_t ws_elems = 0;
   double* part = nullptr;
-  int nparts = 0;
+  int nparts = 0, mse_run = 0;  // column blocks and rows per block of k_mse
   unsigned* done = nullptr;  // blocks of k_mse that have finished (0 between launches)
   int* err = nullptr;
   float* loss = nullptr;
@@ -1285,7 +1300,8 @@ acopf_status acopf_mlp_create(const int32_t* dims, int32_t nlayers, int32_t max_
        dalloc(n, &n->err, 1) && dalloc(n, &n->loss, 1);
   if (ok) {
     n->nparts = (dims[nlayers] + kMseCols - 1) / kMseCols;
-    ok = dalloc(n, &n->part, n->nparts) && dalloc(n, &n->done, 1);
+    n->mse_run = mse_run(dims[nlayers], Mb, n->sms);
+    ok = dalloc(n, &n->part, (size_t)n->nparts * ((Mb + n->mse_run - 1) / n->mse_run)) && dalloc(n, &n->done, 1);
   }
   if (ok) {
     // identity standardisation until fitted
@@ -1426,8 +1442,10 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
              n->sd_x, n->A[0], n->AT[0]));
   acopf_status s = forward(n, rows);
   if (s) return s;
-  NCK(launch(k_mse, n->nparts, 256, 0, n->stream, n->Y, T, idx, rows, Mb, dn, n->mu_y, n->sd_y, n->D[nl], n->DT[nl],
-             n->L[nl - 1].gb, n->part, n->done, n->loss, loss));
+  const bool whole = n->mse_run >= Mb;  // one run: k_mse forms the output layer's bias gradient
+  NCK(launch(k_mse, dim3(n->nparts, (Mb + n->mse_run - 1) / n->mse_run), 256, 0, n->stream, n->Y, T, idx, rows, Mb, dn,
+             n->mu_y, n->sd_y, n->mse_run, n->D[nl], n->DT[nl], whole ? n->L[nl - 1].gb : (float*)nullptr, n->part,
+             n->done, n->loss, loss));
   for (int l = nl - 1; l >= 0; --l) {
     const Gemm &w = n->bwd_w[l], &x = n->bwd_x[l];
     if (l >= 1 && w.small && x.small) {
@@ -1449,7 +1467,7 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
   for (int l = 0; l < nl; ++l) {
     const Layer& y = n->L[l];
     p.l[l] = AdamLayer{y.W, y.gW, y.mW, y.vW, y.b, y.gb, y.mb, y.vb, y.W16, y.W16T,
-                       l < nl - 1 ? n->DT[l + 1] : nullptr, y.in, y.out, blocks, 0};
+                       l < nl - 1 || !whole ? n->DT[l + 1] : nullptr, y.in, y.out, blocks, 0};
     blocks += tiles(y.in) * tiles(y.out);
   }
   for (int l = 0; l < nl; ++l) {

@@ -38,3 +38,26 @@ def test_loss_of_infinite_and_nan_errors():
     assert _loss(T, 128) == np.inf
     T[5, 3] = np.nan
     assert np.isnan(_loss(T, 128))
+
+
+# one run of rows and several: a wide layer, one whose last run is shorter, one
+# of a single column block with as many runs as row tiles, one row tile
+@pytest.mark.parametrize("width,rows", [(40000, 300), (2600, 1000), (8, 2000), (712, 4100), (72, 100)])
+def test_loss_and_output_bias_gradient_over_runs_of_rows(width, rows):
+    rng = np.random.default_rng(width + rows)
+    T = rng.standard_normal((rows, width)).astype(np.float32)
+    net = binding.Mlp([8, width], max_batch=rows)
+    net.set_params(np.zeros(net.nparams, np.float32))
+    X, Td = torch.zeros(rows, 8, device="cuda"), torch.from_numpy(T).cuda()
+    out = torch.zeros(1, device="cuda")
+    net.train_step(X.data_ptr(), Td.data_ptr(), None, rows, 1e-3, out.data_ptr())
+    net.sync()
+    want = np.mean(T.astype(np.float64) ** 2)
+    assert abs(out.item() - want) <= 2.0 ** -23 * want
+    # 2 (Y - T) / (rows N) rounded to bfloat16, summed in FP32 in row order: the same bits
+    g = torch.from_numpy(np.float32(2) * -T / (np.float32(rows) * np.float32(width))).bfloat16().float().numpy()
+    s = np.zeros(width, np.float32)
+    for r in range(rows):
+        s = s + g[r]
+    np.testing.assert_array_equal(net.get_grads()[8 * width:], s)
+    net.close()
