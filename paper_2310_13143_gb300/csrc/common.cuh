@@ -218,6 +218,7 @@ struct Ctx {
   int cluster_exact = -1;     // and way to solve the lines (SweepP::line_exact)
   int cluster_res = 0;        // and how many threads every branch of an instance has (0: static data not in registers)
   bool cluster_dsm = false;   // and whether the state it exchanges stays in distributed shared memory
+  unsigned smem_set = 0;      // kernels whose dynamic shared memory limit this handle has raised (allow_smem)
   std::vector<int> h_task_off, h_big_off;  // host copies of d.task_off, d.big_off
   // warm start staged by acopf_set_warm_start / acopf_set_warm_start_device
   bool warm_x = false, warm_lam = false, warm_rho = false;

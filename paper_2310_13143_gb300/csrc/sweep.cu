@@ -2088,6 +2088,21 @@ static size_t op_smem(int threads, int lanes) {
   return sizeof(T) == 8 ? (size_t)kLineOp * sizeof(double) * (threads / lanes) : 0;
 }
 
+// Lets a kernel take as much dynamic shared memory as a CTA can have.  The limit
+// belongs to the kernel on the device and not to a handle, and a launch above
+// it fails: set to one handle's own need, it would refuse the larger launches of
+// another.  bit: the kernel's place in c.smem_set, which keeps this to once per
+// handle and kernel.
+static void allow_smem(Ctx& c, int bit, const void* fn) {
+  if ((c.smem_set >> bit) & 1u) return;
+  cudaFuncAttributes a{};
+  int most = 0;
+  if (cudaFuncGetAttributes(&a, fn) == cudaSuccess &&
+      cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c.device) == cudaSuccess &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes) == cudaSuccess)
+    c.smem_set |= 1u << bit;
+}
+
 // Launch shape of k_sweep<T>.  The resident form (sweep_stages 3) is used when
 // residual balancing is off and a co-resident grid gives every generator and
 // branch threads of its own and every warp at most two bus tasks; otherwise
@@ -2117,7 +2132,7 @@ static acopf_status sweep_shape(Ctx& c, const SweepP<T>& p, SweepShape& sh) {
       void* fn = (void*)k_sweep<T, 1>;
       if constexpr (sizeof(T) == 8) if (lanes == 4) fn = (void*)k_sweep<T, 4>;
       const size_t smem = sweep_smem<T>(d.K, threads, 0) + 16 + op_smem<T>(threads, lanes);
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_smem(c, lanes == 4 ? 2 : 1, fn);
       int per_sm = 0;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
       if (c.ctas_per_sm > 0 && c.ctas_per_sm < per_sm) per_sm = c.ctas_per_sm;
@@ -2135,7 +2150,7 @@ static acopf_status sweep_shape(Ctx& c, const SweepP<T>& p, SweepShape& sh) {
     cudaGetLastError();
   }
   const size_t smem = sweep_smem<T>(d.K, threads, p.stages);
-  cudaFuncSetAttribute(k_sweep<T, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(c, 0, (const void*)k_sweep<T, 0>);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, 0>, threads, smem);
   if (per_sm < 1) {
@@ -2171,7 +2186,7 @@ static int cluster_size(Ctx& c, int threads, int exact, cudaLaunchConfig_t& cfg,
   const long wpb = threads / 32;
   auto fits = [&](long n, void* fn, size_t smem) {
     cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (smem) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem) allow_smem(c, sizeof(T) == 8 && fn == (void*)k_sweep_cluster<double, 4> ? 4 : 3, fn);
     cfg.dynamicSmemBytes = smem;
     cfg.gridDim = dim3((unsigned)n);
     attr.val.clusterDim.x = (unsigned)n;
@@ -2228,7 +2243,7 @@ static acopf_status run_sweep_cluster(Ctx& c, const SweepP<T>& p) {
     for (int k = 0; dsm && k < c.d.K; ++k) dsm = c.h_big_off[k + 1] == c.h_big_off[k];
     if constexpr (sizeof(T) == 4) if (dsm) {
       cudaFuncSetAttribute(k_sweep_cluster_dsm<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      cudaFuncSetAttribute(k_sweep_cluster_dsm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm_smem);
+      allow_smem(c, 5, (const void*)k_sweep_cluster_dsm<T>);
       cfg.gridDim = dim3(c.cluster_cs);
       attr[0].val.clusterDim.x = c.cluster_cs;
       cfg.dynamicSmemBytes = dsm_smem;
