@@ -90,6 +90,27 @@ static cudaError_t upload(Ctx* c, P* dst, const P* src, size_t count) {
   return cudaMemcpyAsync(dst, src, sizeof(P) * count, cudaMemcpyHostToDevice, c->stream);
 }
 
+// What the setters write from host memory: copies on the handle's stream, so
+// that its kernels and read-outs come after them (a copy on the default stream
+// is not ordered with a non-blocking stream, and from pageable memory it may
+// still be on its way when the call returns).  wait() before the call returns,
+// and the destructor where it returns early: the host memory is the caller's or
+// temporary.  Declared after the host memory it reads.
+struct Uploads {
+  Ctx* c;
+  bool waited = false;
+  explicit Uploads(Ctx* ctx) : c(ctx) {}
+  ~Uploads() { if (!waited) cudaStreamSynchronize(c->stream); }
+  template <typename P>
+  cudaError_t add(P* dst, const P* src, size_t count) {
+    return count ? upload(c, dst, src, count) : cudaSuccess;
+  }
+  cudaError_t wait() {
+    waited = true;
+    return cudaStreamSynchronize(c->stream);
+  }
+};
+
 // ------------------------------------------------------------- read-outs
 template <typename TT>
 static void to_double(const void* src, double* dst, size_t n) {
@@ -114,7 +135,9 @@ static acopf_status put(Ctx* c, void* dev, const std::vector<double>& in, size_t
     for (size_t k = 0; k < in.size(); ++k) ((float*)raw.data())[k] = (float)in[k];
   else
     memcpy(raw.data(), in.data(), es * in.size());
-  CK(cudaMemcpy((unsigned char*)dev + es * offset_elems, raw.data(), es * in.size(), cudaMemcpyHostToDevice));
+  Uploads up(c);
+  CK(up.add((unsigned char*)dev + es * offset_elems, raw.data(), raw.size()));
+  CK(up.wait());
   return ACOPF_OK;
 }
 
@@ -712,26 +735,26 @@ acopf_status acopf_set_iterate(acopf_handle h, int32_t inst, const double* x, co
   int b0 = c->h_bus_off[inst], nb = c->h_bus_off[inst + 1] - b0;
   int l0 = c->h_br_off[inst], nl = c->h_br_off[inst + 1] - l0;
   int g0 = c->h_gen_off[inst], ng = c->h_gen_off[inst + 1] - g0;
-  std::vector<double> pg(ng), qg(ng);
+  std::vector<double> gen(2 * (size_t)ng), rows(pi ? 4 * (size_t)nl : 0);
   for (int q = 0; q < ng; ++q) {
     int internal = c->h_gen_iperm[g0 + q] - g0;
-    pg[internal] = x[q];
-    qg[internal] = x[ng + q];
+    gen[internal] = x[q];
+    gen[ng + internal] = x[ng + q];
   }
+  if (pi)
+    for (int r = 0; r < 4; ++r)
+      for (int l = 0; l < nl; ++l) rows[(size_t)r * nl + l] = pi[4 * l + r];
   const double* w = x + 2 * ng;
-  CK(cudaMemcpy(d.pg + g0, pg.data(), sizeof(double) * ng, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.qg + g0, qg.data(), sizeof(double) * ng, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.w + b0, w, sizeof(double) * nb, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.th + b0, w + nb, sizeof(double) * nb, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.wr + l0, w + 2 * nb, sizeof(double) * nl, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.wi + l0, w + 2 * nb + nl, sizeof(double) * nl, cudaMemcpyHostToDevice));
-  if (pi) {
-    std::vector<double> col(nl);
-    for (int r = 0; r < 4; ++r) {
-      for (int l = 0; l < nl; ++l) col[l] = pi[4 * l + r];
-      CK(cudaMemcpy(d.pi + (size_t)r * d.L + l0, col.data(), sizeof(double) * nl, cudaMemcpyHostToDevice));
-    }
-  }
+  Uploads up(c);
+  CK(up.add(d.pg + g0, gen.data(), ng));
+  CK(up.add(d.qg + g0, gen.data() + ng, ng));
+  CK(up.add(d.w + b0, w, nb));
+  CK(up.add(d.th + b0, w + nb, nb));
+  CK(up.add(d.wr + l0, w + 2 * nb, nl));
+  CK(up.add(d.wi + l0, w + 2 * nb + nl, nl));
+  if (pi)
+    for (int r = 0; r < 4; ++r) CK(up.add(d.pi + (size_t)r * d.L + l0, rows.data() + (size_t)r * nl, nl));
+  CK(up.wait());
   return ACOPF_OK;
 }
 
@@ -1363,7 +1386,8 @@ acopf_status acopf_set_warm_start(acopf_handle h, int32_t inst, const double* x0
   if (x0) {
     if ((s = acopf_set_iterate(h, inst, x0, nullptr))) return s;
     int l0 = c->h_br_off[inst], nl = c->h_br_off[inst + 1] - l0;
-    for (int r = 0; r < 4; ++r) CK(cudaMemset(c->d.pi + (size_t)r * c->d.L + l0, 0, sizeof(double) * nl));
+    for (int r = 0; r < 4; ++r)
+      CK(cudaMemsetAsync(c->d.pi + (size_t)r * c->d.L + l0, 0, sizeof(double) * nl, c->stream));
     c->warm_x = true;
   }
   if (lambda0) {
@@ -1380,13 +1404,15 @@ acopf_status acopf_set_warm_start(acopf_handle h, int32_t inst, const double* x0
     int g0 = c->h_gen_off[inst], ng = c->h_gen_off[inst + 1] - g0;
     for (int l = 0; l < nl; ++l)
       if (!(rho[l] > 0)) return fail(c, ACOPF_EINVAL, "acopf_set_warm_start: rho must be positive");
-    CK(cudaMemcpy(c->d.rho_l + l0, rho, sizeof(double) * nl, cudaMemcpyHostToDevice));
     std::vector<double> rg(ng);
+    Uploads up(c);
+    CK(up.add(c->d.rho_l + l0, rho, nl));
     for (int q = 0; q < ng; ++q) {
       if (!(rho[nl + q] > 0)) return fail(c, ACOPF_EINVAL, "acopf_set_warm_start: rho must be positive");
       rg[c->h_gen_iperm[g0 + q] - g0] = rho[nl + q];
     }
-    CK(cudaMemcpy(c->d.rho_g + g0, rg.data(), sizeof(double) * ng, cudaMemcpyHostToDevice));
+    CK(up.add(c->d.rho_g + g0, rg.data(), ng));
+    CK(up.wait());
     c->warm_rho = true;
   }
   return ACOPF_OK;

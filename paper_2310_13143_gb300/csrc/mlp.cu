@@ -1309,7 +1309,8 @@ acopf_status acopf_mlp_create(const int32_t* dims, int32_t nlayers, int32_t max_
     ok = cudaMemcpy(n->sd_x, one.data(), sizeof(float) * dims[0], cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(n->sd_y, one.data(), sizeof(float) * dims[nlayers], cudaMemcpyHostToDevice) == cudaSuccess;
   }
-  if (!ok || !plan(n)) {
+  // zeros and ones were written on the default stream, which the network's need not wait for
+  if (!ok || !plan(n) || cudaStreamSynchronize(nullptr) != cudaSuccess) {
     free_net(n);
     delete n;
     cudaGetLastError();
@@ -1356,7 +1357,8 @@ static acopf_status copy_params(Net* n, float* host, int64_t count, bool to_devi
   NCK(cudaStreamSynchronize(n->stream));
   float* dev = grads ? n->grads : n->params;
   const size_t bytes = sizeof(float) * n->nparams;
-  if (to_device) NCK(cudaMemcpy(dev, host, bytes, cudaMemcpyHostToDevice));
+  // on the network's stream, before the kernels that read it; set_params waits
+  if (to_device) NCK(cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, n->stream));
   else NCK(cudaMemcpy(host, dev, bytes, cudaMemcpyDeviceToHost));
   return ACOPF_OK;
 }
