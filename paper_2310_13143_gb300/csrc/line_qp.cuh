@@ -122,6 +122,15 @@ ACOPF_HD inline float div_w(float a, float b) {
   return a / b;
 #endif
 }
+// a / b from the kept reciprocal inv = 1 / b (correctly rounded): the product
+// and one correction with its remainder, which is the correctly rounded quotient
+// (Markstein, 1990) short of underflow, in three instructions instead of some
+// ten.  An infinite or NaN product stays as it is.
+ACOPF_HD inline double quot_kept(double a, double b, double inv) {
+  const double q = a * inv;
+  const double c = fma(fma(-b, q, a), inv, q);
+  return ((unsigned)(bits_of(q) >> 32) & 0x7fffffffu) < 0x7ff00000u ? c : q;
+}
 // 1/sqrt(a) in FP64 from an estimate y0 by one third-order step: with
 // e = 1 - a y0^2 the exact value is y0 (1 - e)^(-1/2) = y0 (1 + e/2 + 3e^2/8
 // + 5e^3/16 + ...), and the step keeps the series to e^2.  A relative error d

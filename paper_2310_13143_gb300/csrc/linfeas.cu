@@ -56,7 +56,7 @@ __device__ __forceinline__ D4 d4(double a, double b, double c, double e) {
   return v;
 }
 
-constexpr int kLfBus = 6;      // per bus: inverse of the 2x2 matrix (3), 1/Qw, M, 2 w0
+constexpr int kLfBus = 7;  // per bus: inverse of the 2x2 matrix (3), 1/Qw, M, 2 w0, Qw
 constexpr int kLfWindow = 1024;
 
 struct LfState {
@@ -94,6 +94,7 @@ __global__ void k_lf_init(Dev d, LfState s, double rho) {
     c[3 * (size_t)B] = 1.0 / Qw;
     c[4 * (size_t)B] = M;
     c[5 * (size_t)B] = 2.0 * d.w[n];
+    c[6 * (size_t)B] = Qw;
     s.WB[n] = d.w[n];
     s.N[n] = make_double2(0.0, 0.0);
   }
@@ -153,14 +154,15 @@ __device__ __noinline__ void lf_edges_call(double l, double i1, double i2, doubl
 }
 
 // generators and branches (one thread each): x from y
-__global__ void __launch_bounds__(128) k_lf_components(Dev d, LfState s, double gen_scale) {
+__global__ void __launch_bounds__(128) k_lf_components(Dev d, LfState s, double gen_div,
+                                                       double gen_inv) {
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   const int G = d.G;
   const size_t L = d.L;
   if (u < G) {
     const double2 y = s.YG[u];
-    s.XG[u] = make_double2(clampv((s.g0[u] - y.x) * gen_scale, d.pmin[u], d.pmax[u]),
-                           clampv((s.g0[G + u] - y.y) * gen_scale, d.qmin[u], d.qmax[u]));
+    s.XG[u] = make_double2(clampv(quot_kept(s.g0[u] - y.x, gen_div, gen_inv), d.pmin[u], d.pmax[u]),
+                           clampv(quot_kept(s.g0[G + u] - y.y, gen_div, gen_inv), d.qmin[u], d.qmax[u]));
     return;
   }
   const int l = u - G;
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(128) k_lf_buses(Dev d, LfState s, double rho) 
     v1 -= gsh * t;
     v2 += bsh * t;
     const double n1 = c[0] * v1 + c[1 * B] * v2, n2 = c[1 * B] * v1 + c[2 * B] * v2;
-    const double w = (cw + gsh * n1 - bsh * n2) * iq, rw = rho * w;
+    const double w = quot_kept(cw + gsh * n1 - bsh * n2, c[6 * B], iq), rw = rho * w;
     // y = lambda - rho z = -+(2 nu - nu_old) - rho x
     const double a1 = no.x - 2.0 * n1, a2 = no.y - 2.0 * n2;
     if (RES) {
@@ -326,7 +328,7 @@ acopf_status project_linear(Ctx& c, double rho, double eps, int max_iter, int ch
     const int n = max_iter - it < check ? max_iter - it : check;
     cudaMemsetAsync(s.res, 0, sizeof(unsigned long long) * 2 * d.K, c.stream);
     for (int k = 0; k < n; ++k) {
-      k_lf_components<<<nblk(d.G + d.L, 128), 128, 0, c.stream>>>(d, s, 1.0 / (2.0 + rho));
+      k_lf_components<<<nblk(d.G + d.L, 128), 128, 0, c.stream>>>(d, s, 2.0 + rho, 1.0 / (2.0 + rho));
       if (k == n - 1) k_lf_buses<true><<<nblk(d.B, 128), 128, 0, c.stream>>>(d, s, rho);
       else k_lf_buses<false><<<nblk(d.B, 128), 128, 0, c.stream>>>(d, s, rho);
       c.launches += 2;

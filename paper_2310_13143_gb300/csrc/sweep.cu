@@ -191,15 +191,19 @@ __device__ __forceinline__ void gen_compute(const Dev& d, int g, const V4<T>& a,
 }
 
 // FP64 resident forms: the two divisors are constant during a sweep, so the
-// thread keeps their reciprocals (an FP64 division is some ten FP64
-// instructions, in the same warp as the first branches)
+// thread keeps their reciprocals k = (1 / (f'' + rho), 1 / rho, f'' + rho) (an
+// FP64 division is some ten FP64 instructions, in the same warp as the first
+// branches)
+__device__ __forceinline__ V4<double> gen_kept(const V4<double>& a, const V4<double>& b) {
+  return V4<double>{1.0 / (a.y + b.z), 1.0 / b.z, a.y + b.z, 0.0};
+}
 __device__ __forceinline__ void gen_compute_kept(const Dev& d, int g, const V4<double>& a, const V4<double>& b,
-                                                 double inv_p, double inv_q) {
+                                                 const V4<double>& k) {
   const double rho = b.z;
   const V2<double> z = ((const V2<double>*)d.ZG)[g], lam = ((const V2<double>*)d.LG)[g];
   V2<double> x;
-  x.x = clampv((rho * z.x - lam.x - a.x) * inv_p, a.z, a.w);
-  x.y = clampv((rho * z.y - lam.y) * inv_q, b.x, b.y);
+  x.x = clampv(quot_kept(rho * z.x - lam.x - a.x, k.z, k.x), a.z, a.w);
+  x.y = clampv(quot_kept(rho * z.y - lam.y, rho, k.y), b.x, b.y);
   ((V2<double>*)d.XG)[g] = x;
 }
 
@@ -1313,7 +1317,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
       my_k = d.gen_inst[gen];
       rr[0] = ((const V4<T>*)d.grec)[gen];
       rr[1] = ((const V4<T>*)d.grec)[d.G + gen];
-      if (sizeof(T) == 8) rr[2] = {T(1) / (rr[0].y + rr[1].z), T(1) / rr[1].z, T(0), T(0)};
+      if constexpr (sizeof(T) == 8) rr[2] = gen_kept(rr[0], rr[1]);
     } else if (is_br) {
       my_k = d.br_inst[br];
       if constexpr (RES == 4) {
@@ -1347,12 +1351,12 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
       const V4<T>* Z = (const V4<T>*)d.Z;
       const V4<T>* LM = (const V4<T>*)d.LAM;
       if constexpr (RES == 4) {
-        if (go && is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+        if (go && is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
         line_compute_quad(p, d, go && is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
       } else if (go) {
         if constexpr (sizeof(T) == 8) {
           if (is_gen)
-            gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+            gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
           else
             line_compute_kept(p, d, br, RRec<T>{rr}, Z[2 * br], Z[2 * br + 1], LM[2 * br], LM[2 * br + 1], my_rho,
                               my_wset, s_op + threadIdx.x, blockDim.x);
@@ -1673,7 +1677,7 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(const __grid_constant_
     if (is_gen) {
       rr[0] = ((const V4<T>*)d.grec)[gen];
       rr[1] = ((const V4<T>*)d.grec)[d.G + gen];
-      if (sizeof(T) == 8) rr[2] = {T(1) / (rr[0].y + rr[1].z), T(1) / rr[1].z, T(0), T(0)};
+      if constexpr (sizeof(T) == 8) rr[2] = gen_kept(rr[0], rr[1]);
     } else if (is_br) {
       if constexpr (RES == 4) {
         quad_load(d, br, lane & 3, qr);
@@ -1703,11 +1707,11 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(const __grid_constant_
       const V4<T>* Z = (const V4<T>*)d.Z;
       const V4<T>* LM = (const V4<T>*)d.LAM;
       if constexpr (RES == 4) {
-        if (is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+        if (is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
         line_compute_quad(p, d, is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
       } else if constexpr (sizeof(T) == 8) {
         if (is_gen)
-          gen_compute_kept(d, gen, rr[0], rr[1], rr[2].x, rr[2].y);
+          gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
         else if (is_br)
           line_compute_kept(p, d, br, RRec<T>{rr}, Z[2 * br], Z[2 * br + 1], LM[2 * br], LM[2 * br + 1], my_rho,
                             my_wset, s_op + threadIdx.x, blockDim.x);

@@ -16,13 +16,16 @@ DP = C.POINTER(C.c_double)
 
 
 @pytest.fixture(scope="module")
-def solve(tmp_path_factory):
+def lib(tmp_path_factory):
     if shutil.which("g++") is None:
         pytest.skip("g++ not available")
     out = str(tmp_path_factory.mktemp("host") / "linfeas_helpers.so")
     subprocess.check_call(["g++", "-O2", "-shared", "-fPIC", "-o", out, os.path.join(HERE, "host", "linfeas_helpers.cpp")])
-    lib = C.CDLL(out)
+    return C.CDLL(out)
 
+
+@pytest.fixture(scope="module")
+def solve(lib):
     def run(P):
         P = np.ascontiguousarray(P)
         v = np.zeros((len(P), 4))
@@ -122,3 +125,14 @@ def test_branch_subproblem_keeps_nan(solve):
     for k, j in enumerate((15, 16, 18, 19)):
         P[3 * k:3 * k + 3, j] = np.nan
     assert np.isnan(solve(P)).any(axis=1).all()
+
+
+def test_quotient_from_a_kept_reciprocal(lib):
+    rng = np.random.default_rng(9)
+    n = 200000
+    a = rng.standard_normal(n) * 10.0 ** rng.uniform(-12, 12, n)
+    b = 10.0 ** rng.uniform(-6, 8, n)
+    a[:6] = np.inf, -np.inf, np.nan, 0.0, 1e300, -1e300
+    out = np.zeros(n)
+    lib.host_quot_kept(n, a.ctypes.data_as(DP), b.ctypes.data_as(DP), out.ctypes.data_as(DP))
+    np.testing.assert_array_equal(out, a / b)
