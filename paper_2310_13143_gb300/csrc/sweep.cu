@@ -406,7 +406,9 @@ __device__ __forceinline__ void line_compute_to(const SweepP<T>& p, int l, const
 // FP64 resident forms: the line update with the branch's active set and the
 // set's operator kept from one iteration to the next (line_operator,
 // line_eval).  The set is corrected up to three times; a subproblem that this
-// does not settle, and line_solver = 1, take the general solves above.
+// does not settle takes the general solves above.  line_solver = 1 keeps no set
+// and solves from the record in registers (read again from memory instead, 300
+// buses took 40.3 against 34.2 us per iteration).
 //
 // What bounds it is the number of FP64 instructions on a warp's path: one takes
 // its SM partition's pipe for some 64 cycles whether the warp has one lane at
@@ -439,8 +441,8 @@ __device__ __noinline__ unsigned line_set_slow(const Dev& d, int l) {
 }
 // the whole line update of branch l by the general solves, from and to global
 // memory; returns the solution's set
-__device__ __noinline__ unsigned line_general_slow(const Dev& d, int l, int exact, double beta_scale, double tol,
-                                                   int outer, int newton) {
+__device__ __noinline__ unsigned line_general_slow(const Dev& d, int l, double beta_scale, double tol, int outer,
+                                                   int newton) {
   const V4<double>* Z = (const V4<double>*)d.Z;
   const V4<double>* LM = (const V4<double>*)d.LAM;
   const V4<double> z0 = Z[2 * l], z1 = Z[2 * l + 1], uu = ((const V4<double>*)d.U)[l];
@@ -451,8 +453,8 @@ __device__ __noinline__ unsigned line_general_slow(const Dev& d, int l, int exac
   double x[4], u[4] = {uu.x, uu.y, uu.z, uu.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = clampv(z[i], P.lo[i], P.hi[i]);
-  bool done = exact && line_pred_call(P, x, u);
-  if (exact && !done) {
+  bool done = line_pred_call(P, x, u);
+  if (!done) {
     u[0] = uu.x; u[1] = uu.y; u[2] = uu.z; u[3] = uu.w;
     done = line_exact_call(P, x, u) >= 0;
   }
@@ -476,32 +478,48 @@ template <typename Rec>
 __device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, const Dev& d, int l, const Rec& rec,
                                                   V4<double> z0, V4<double> z1, V4<double> l0, V4<double> l1,
                                                   double rho, unsigned& set, double* op, int stride) {
+  V4<double>* X = (V4<double>*)d.X;
+  V4<double>* U = (V4<double>*)d.U;
+  if (!p.line_exact) {  // no set is kept: the augmented Lagrangian on the record in registers
+    const V4<double> uu = U[l];
+    LineQP<double> A;
+    line_problem(rec, z0, z1, l0, l1, rho, A);
+    const double z[4] = {z0.z, z0.w, z1.z, z1.w};
+    double xa[4], ua[4] = {uu.x, uu.y, uu.z, uu.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) xa[i] = clampv(z[i], A.lo[i], A.hi[i]);
+    const double beta = p.beta_scale * fmax(fmax(A.q[0], A.q[4]), fmax(A.q[7], A.q[9]));
+    line_alm_call(A, xa, ua, beta, p.alm_tol, p.alm_outer, p.newton_max);
+    V4<double> o0, o1, ou;
+    line_outputs(rec, xa, ua, o0, o1, ou);
+    X[2 * l] = o0;
+    X[2 * l + 1] = o1;
+    U[l] = ou;
+    return;
+  }
   LineQP<double> P;
   line_problem(rec, z0, z1, l0, l1, rho, P);
   double x[4], u[4];
   bool ok = false;
-  if (p.line_exact) {
-    for (int attempt = 0; attempt < 4; ++attempt) {
-      if (!(set & kSetValid)) {
-        if (!line_operator_slow(d, l, set, op, stride)) break;
-        set |= kSetValid;
-      }
-      unsigned next;
-      ok = line_eval(P, set, op, stride, x, u, next);
-      if (ok || next == (set & ~kSetValid)) break;
-      set = next;
+  for (int attempt = 0; attempt < 4; ++attempt) {
+    if (!(set & kSetValid)) {
+      if (!line_operator_slow(d, l, set, op, stride)) break;
+      set |= kSetValid;
     }
+    unsigned next;
+    ok = line_eval(P, set, op, stride, x, u, next);
+    if (ok || next == (set & ~kSetValid)) break;
+    set = next;
   }
   if (!ok) {
-    set = line_general_slow(d, l, p.line_exact, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
+    set = line_general_slow(d, l, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
     return;
   }
   V4<double> o0, o1, ou;
   line_outputs(rec, x, u, o0, o1, ou);
-  V4<double>* X = (V4<double>*)p.d.X;
   X[2 * l] = o0;
   X[2 * l + 1] = o1;
-  ((V4<double>*)p.d.U)[l] = ou;
+  U[l] = ou;
 }
 
 // Four lanes per branch: what lane q of branch l holds for the sweep.
@@ -575,7 +593,7 @@ __device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const
   const double c = quad_dot(a.Fc, lf - a.rho * zf, a.c0 + lv - a.rho * zv);
   const unsigned ch = quad_max(abs_hi(c));
   double x = 0.0, mu = 0.0;
-  bool general = !p.line_exact;  // of the quad: left to the general solves
+  bool general = false;  // of the quad: left to the general solves
   // every exit from the loop is warp-uniform: all lanes take part in its shuffles
   for (int attempt = 0; attempt < 4; ++attempt) {
     // operators that are missing, by the quads' first lanes
@@ -657,7 +675,7 @@ __device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const
   if (__any_sync(FULL, is && general)) {
     unsigned s = a.set;
     if (is && general && q == 0)
-      s = line_general_slow(d, l, p.line_exact, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
+      s = line_general_slow(d, l, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
     s = __shfl_sync(FULL, s, 0, 4);
     if (general) a.set = s;
   }
