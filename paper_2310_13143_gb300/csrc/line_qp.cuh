@@ -1124,11 +1124,12 @@ ACOPF_HD inline bool line_solve_predicted(const LineQP<double>& P, double x[4], 
 // prediction, an FP64 Cholesky factorisation and triangular solves.
 //
 // Set: bits 0-3 bounds held, 4-7 at the upper bound, 8-11 rows active; bit 12
-// marks a set that holds an operator.  Operator: value e at op[e * stride]:
+// marks a set that holds an operator, bit 13 one that is left to the general
+// solves.  Operator: value e at op[e * stride]:
 //   0-9 P (packed)  10-13 p0  14-17 M of the first active row  18-21 of the
 //   second  22, 23 m0  24 max |q|  25-28 1 + |b_r| of the four rows
 constexpr int kLineOp = 29;
-constexpr unsigned kSetValid = 1u << 12;
+constexpr unsigned kSetValid = 1u << 12, kSetGeneral = 1u << 13;
 
 ACOPF_HD inline unsigned hi_of(double x) { return (unsigned)(bits_of(x) >> 32); }
 ACOPF_HD inline unsigned abs_hi(double x) { return hi_of(x) & 0x7fffffffu; }

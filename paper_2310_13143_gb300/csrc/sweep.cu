@@ -440,7 +440,9 @@ __device__ __noinline__ unsigned line_set_slow(const Dev& d, int l) {
   return line_set_of(P, x, u);
 }
 // the whole line update of branch l by the general solves, from and to global
-// memory; returns the solution's set
+// memory; returns the solution's set, with kSetGeneral where the subproblem has
+// no feasible point: the branch then comes here at once in the next iteration,
+// instead of correcting sets that cannot settle it
 __device__ __noinline__ unsigned line_general_slow(const Dev& d, int l, double beta_scale, double tol, int outer,
                                                    int newton) {
   const V4<double>* Z = (const V4<double>*)d.Z;
@@ -470,7 +472,7 @@ __device__ __noinline__ unsigned line_general_slow(const Dev& d, int l, double b
   ((V4<double>*)d.X)[2 * l] = o0;
   ((V4<double>*)d.X)[2 * l + 1] = o1;
   ((V4<double>*)d.U)[l] = ou;
-  return line_set_of(P, x, u);
+  return line_set_of(P, x, u) | (done ? 0u : kSetGeneral);
 }
 
 // one lane per branch: op in shared memory, one column per thread
@@ -501,7 +503,7 @@ __device__ __forceinline__ void line_compute_kept(const SweepP<double>& p, const
   line_problem(rec, z0, z1, l0, l1, rho, P);
   double x[4], u[4];
   bool ok = false;
-  for (int attempt = 0; attempt < 4; ++attempt) {
+  for (int attempt = 0; attempt < 4 && !(set & kSetGeneral); ++attempt) {
     if (!(set & kSetValid)) {
       if (!line_operator_slow(d, l, set, op, stride)) break;
       set |= kSetValid;
@@ -593,7 +595,7 @@ __device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const
   const double c = quad_dot(a.Fc, lf - a.rho * zf, a.c0 + lv - a.rho * zv);
   const unsigned ch = quad_max(abs_hi(c));
   double x = 0.0, mu = 0.0;
-  bool general = false;  // of the quad: left to the general solves
+  bool general = is && (a.set & kSetGeneral);  // of the quad: left to the general solves
   // every exit from the loop is warp-uniform: all lanes take part in its shuffles
   for (int attempt = 0; attempt < 4; ++attempt) {
     // operators that are missing, by the quads' first lanes
