@@ -975,7 +975,7 @@ static std::string tune_key(Ctx* c) {
     return k;
   };
   char buf[128];
-  snprintf(buf, sizeof(buf), "v4-sm%d-%s-K%d-B%d-L%d", c->num_sms, c->precision == ACOPF_MIXED ? "mixed" : "fp64",
+  snprintf(buf, sizeof(buf), "v5-sm%d-%s-K%d-B%d-L%d", c->num_sms, c->precision == ACOPF_MIXED ? "mixed" : "fp64",
            lg(c->d.K), lg(c->d.B), lg(c->d.L));
   return buf;
 }
