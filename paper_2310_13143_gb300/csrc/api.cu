@@ -151,21 +151,18 @@ static void drop_graph(Ctx* c) {
 // One instance's variables, pi (when wanted) and objective into c->h_stage;
 // synchronises the handle's stream.
 static acopf_status stage_instance(Ctx* c, int inst, const PackSrc& src) {
-  const size_t nb = c->h_bus_off[inst + 1] - c->h_bus_off[inst], nl = c->h_br_off[inst + 1] - c->h_br_off[inst],
-               ng = c->h_gen_off[inst + 1] - c->h_gen_off[inst];
-  const size_t n = 2 * ng + 2 * nb + 6 * nl + 1;
   struct OnDevice {  // a read-out works whatever device the caller has current
     int was = 0;
     explicit OnDevice(int dev) { cudaGetDevice(&was); if (was != dev) cudaSetDevice(dev); else was = -1; }
     ~OnDevice() { if (was >= 0) cudaSetDevice(was); }
   } on(c->device);
-  if (n > c->stage_values) {
-    CK(cudaStreamSynchronize(c->stream));
-    if (c->h_stage) cudaFreeHost(c->h_stage);
-    c->h_stage = nullptr;
-    c->stage_values = 0;
+  if (!c->h_stage) {
+    size_t n = 0;  // values of the largest instance
+    for (int k = 0; k < c->d.K; ++k)
+      n = std::max(n, 2 * (size_t)(c->h_gen_off[k + 1] - c->h_gen_off[k]) +
+                          2 * (size_t)(c->h_bus_off[k + 1] - c->h_bus_off[k]) +
+                          6 * (size_t)(c->h_br_off[k + 1] - c->h_br_off[k]) + 1);
     CK(cudaMallocHost(&c->h_stage, sizeof(double) * n));
-    c->stage_values = n;
   }
   launch_pack(*c, src, inst, c->h_stage);
   CK(cudaGetLastError());

@@ -232,9 +232,8 @@ struct Ctx {
   int* h_running = nullptr;        // pinned host copy of n_running
   // read-outs (acopf_get_iterate, _step, _solution): pinned host memory that
   // k_pack writes one instance's values into; as large as the largest instance
-  // read so far needs, freed with the handle
+  // needs, taken at the first read-out and freed with the handle
   double* h_stage = nullptr;
-  size_t stage_values = 0;
   cudaStream_t gstream = nullptr;  // capture stream when the handle has none
 };
 
