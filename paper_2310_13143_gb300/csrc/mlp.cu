@@ -1444,10 +1444,19 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
              n->sd_x, n->A[0], n->AT[0]));
   acopf_status s = forward(n, rows);
   if (s) return s;
+  // k_mse stores the loss where it is asked for if that is aligned memory of this
+  // device; anything else is left to a copy, which takes or refuses it
+  bool direct = loss && ((uintptr_t)loss & 3) == 0;
+  if (direct) {
+    cudaPointerAttributes at{};
+    direct = cudaPointerGetAttributes(&at, loss) == cudaSuccess &&
+             (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == n->device;
+    if (!direct) cudaGetLastError();
+  }
   const bool whole = n->mse_run >= Mb;  // one run: k_mse forms the output layer's bias gradient
   NCK(launch(k_mse, dim3(n->nparts, (Mb + n->mse_run - 1) / n->mse_run), 256, 0, n->stream, n->Y, T, idx, rows, Mb, dn,
              n->mu_y, n->sd_y, n->mse_run, n->D[nl], n->DT[nl], whole ? n->L[nl - 1].gb : (float*)nullptr, n->part,
-             n->done, n->loss, loss));
+             n->done, n->loss, direct ? loss : (float*)nullptr));
   for (int l = nl - 1; l >= 0; --l) {
     const Gemm &w = n->bwd_w[l], &x = n->bwd_x[l];
     if (l >= 1 && w.small && x.small) {
@@ -1477,6 +1486,7 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
     blocks += (n->L[l].out + kAdamBias - 1) / kAdamBias;
   }
   NCK(launch(k_adam, blocks, 256, 0, n->stream, p));
+  if (loss && !direct) NCK(cudaMemcpyAsync(loss, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, n->stream));
   return ACOPF_OK;
 }
 

@@ -61,3 +61,18 @@ def test_loss_and_output_bias_gradient_over_runs_of_rows(width, rows):
         s = s + g[r]
     np.testing.assert_array_equal(net.get_grads()[8 * width:], s)
     net.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 4])
+def test_loss_at_any_address(offset):
+    """The loss may be asked for at any byte address of device memory."""
+    rows, T = 128, torch.ones(128, 16, device="cuda")
+    net = binding.Mlp([8, 16], max_batch=rows)
+    net.set_params(np.zeros(net.nparams, np.float32))
+    X, out = torch.zeros(rows, 8, device="cuda"), torch.full((12,), 7, dtype=torch.uint8, device="cuda")
+    net.train_step(X.data_ptr(), T.data_ptr(), None, rows, 1e-3, out.data_ptr() + offset)
+    net.sync()
+    got = out.cpu().numpy()
+    assert got[offset:offset + 4].copy().view(np.float32)[0] == 1.0
+    assert (got[:offset] == 7).all() and (got[offset + 4:] == 7).all()
+    net.close()
