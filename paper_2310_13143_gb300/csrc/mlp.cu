@@ -637,13 +637,15 @@ __global__ void k_splitk(const float* ws, int splits, size_t stride, Epi e) {
 // rounded to bfloat16, stored row-major and (AT not null) transposed; rows >=
 // rows are 0.  32 x 32 tiles through shared memory, so that both stores
 // coalesce (an element-wise kernel wrote the transpose 2 bytes per sector: 12
-// us for 256 x 4000).  Grid (ceil(d0 / 32), rows of A / 32), block 32 x 8.
+// us for 256 x 4000).  Grid ceil(d0 / 32) x (rows of A / 32), in one dimension,
+// as the others end at 65,535; block 32 x 8.
 __global__ void __launch_bounds__(256) k_input(const float* X, const int* idx, int rows, int Mb, int d0,
                                                const float* mu, const float* sd, bf16* A, bf16* AT) {
   __shared__ bf16 tile[32][34];
   pdl_go();
   pdl_wait();
-  const int j = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 32;
+  const int nt = (d0 + 31) / 32, j0 = (int)(blockIdx.x % nt) * 32, r0 = (int)(blockIdx.x / nt) * 32;
+  const int j = j0 + threadIdx.x;
   const float m = j < d0 ? mu[j] : 0.0f, s = j < d0 ? sd[j] : 1.0f;
 #pragma unroll
   for (int k = threadIdx.y; k < 32; k += 8) {
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(256) k_input(const float* X, const int* idx, i
   __syncthreads();
 #pragma unroll
   for (int k = threadIdx.y; k < 32; k += 8) {
-    const int jj = blockIdx.x * 32 + k;
+    const int jj = j0 + k;
     if (jj < d0) AT[(size_t)jj * Mb + r0 + threadIdx.x] = tile[threadIdx.x][k];
   }
 }
@@ -1426,7 +1428,7 @@ acopf_status acopf_mlp_forward(acopf_mlp_handle h, const float* X, int32_t rows,
   const int d0 = n->dims[0], dn = n->dims[n->nl];
   for (int r0 = 0; r0 < rows; r0 += n->Mb) {
     int rr = rows - r0 < n->Mb ? rows - r0 : n->Mb;
-    NCK(launch(k_input, dim3((d0 + 31) / 32, (rr + BM - 1) / BM * (BM / 32)), dim3(32, 8), 0, n->stream,
+    NCK(launch(k_input, (d0 + 31) / 32 * ((rr + BM - 1) / BM * (BM / 32)), dim3(32, 8), 0, n->stream,
                X + (size_t)r0 * d0, (const int*)nullptr, rr, n->Mb, d0, n->mu_x, n->sd_x, n->A[0], (bf16*)nullptr));
     acopf_status s = forward(n, rr, Y + (size_t)r0 * dn);
     if (s) return s;
@@ -1440,7 +1442,7 @@ acopf_status acopf_mlp_train_step(acopf_mlp_handle h, const float* X, const floa
   if (!n || !X || !T || rows < 1 || rows > n->Mb || !(lr > 0)) return nfail(n, ACOPF_EINVAL, "mlp_train_step: bad arguments");
   cudaSetDevice(n->device);
   const int nl = n->nl, Mb = n->Mb, d0 = n->dims[0], dn = n->dims[nl];
-  NCK(launch(k_input, dim3((d0 + 31) / 32, Mb / 32), dim3(32, 8), 0, n->stream, X, idx, rows, Mb, d0, n->mu_x,
+  NCK(launch(k_input, (d0 + 31) / 32 * (Mb / 32), dim3(32, 8), 0, n->stream, X, idx, rows, Mb, d0, n->mu_x,
              n->sd_x, n->A[0], n->AT[0]));
   acopf_status s = forward(n, rows);
   if (s) return s;
