@@ -11,8 +11,8 @@
 //            system of the power-balance rows, per-bus sums by a segmented
 //            warp scan), fused with the multiplier update of every coupling
 //            (eq. multiplier) and the primal/dual residuals r = x - z,
-//            s = rho (z+ - z) (Sec. IV-B), reduced with warp shuffles and one
-//            64-bit atomicMax per run of lanes of one instance;
+//            s = rho (z+ - z) (Sec. IV-B), reduced by the warp's reduction
+//            instructions and one atomic maximum per task and residual;
 //   barrier
 //   every CTA reads the per-instance residual slots and decides, identically,
 //   which instances have converged; finished instances are skipped.
@@ -718,13 +718,12 @@ struct ResDst {
   unsigned long long* acc;  // shared [2][K] or null
   unsigned long long* slots;
   int K, slot;
-  int kbase;  // instance of acc[0] (a cluster's one-instance accumulator; 0 otherwise)
   // the maxima as the bit patterns of non-negative doubles (ordered as
   // integers); positive values only
   __device__ __forceinline__ void put_bits(int inst, unsigned long long r, unsigned long long s) const {
     if (acc) {
-      if (r) atomicMax(&acc[inst - kbase], r);
-      if (s) atomicMax(&acc[K + inst - kbase], s);
+      if (r) atomicMax(&acc[inst], r);
+      if (s) atomicMax(&acc[K + inst], s);
     } else {
       if (r) atomicMax(&slots[(slot * 2 + 0) * K + inst], r);
       if (s) atomicMax(&slots[(slot * 2 + 1) * K + inst], s);
@@ -742,8 +741,8 @@ struct ResDst {
   __device__ __forceinline__ void put(int inst, float rf, float sf) const {
     const double r = rf, s = sf;
     if (acc) {
-      if (r > 0.0) atomicMax(&acc[inst - kbase], (unsigned long long)__double_as_longlong(r));
-      if (s > 0.0) atomicMax(&acc[K + inst - kbase], (unsigned long long)__double_as_longlong(s));
+      if (r > 0.0) atomicMax(&acc[inst], (unsigned long long)__double_as_longlong(r));
+      if (s > 0.0) atomicMax(&acc[K + inst], (unsigned long long)__double_as_longlong(s));
     } else {
       if (r > 0.0) atomicMax(&slots[(slot * 2 + 0) * K + inst], (unsigned long long)__double_as_longlong(r));
       if (s > 0.0) atomicMax(&slots[(slot * 2 + 1) * K + inst], (unsigned long long)__double_as_longlong(s));
@@ -1472,7 +1471,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     if (prof) { tp1 = gtimer(); atomicAdd(&d.phase_ns[0], tp1 - tp0); }
     if (!grid_barrier(d.bar, epoch, d.err, p.spin_limit, solo)) { aborted = true; break; }
     if (prof) { tp0 = gtimer(); atomicAdd(&d.phase_ns[1], tp0 - tp1); }
-    const ResDst dst = {s_acc, d.res_slots, K, slot, 0};
+    const ResDst dst = {s_acc, d.res_slots, K, slot};
     // phase B: buses, in warp tasks of consecutive whole buses, two tasks at a
     // time (every entry belongs to one task, so the loads ahead never read
     // what the current tasks write); loop bounds are uniform per warp so that
@@ -2132,9 +2131,9 @@ static void allow_smem(Ctx& c, int bit, const void* fn) {
 // branch threads of its own and every warp at most two bus tasks; otherwise
 // (and for sweep_stages 0-2) the streaming form, with enough CTAs for one pass
 // over the larger of the two phases, capped at the co-resident maximum.  FP64:
-// four threads per branch where they fit, which is up to 9,600 branches (255
-// registers: two warps per SM partition, some 100 FP64 instructions on its
-// pipe per iteration), else one (one warp per partition, 150).
+// four threads per branch where these and the generators' fit, G + 4 L <= 256
+// per SM (255 registers: two warps per SM partition, some 100 FP64 instructions
+// on its pipe per iteration), else one (one warp per partition, 150).
 struct SweepShape {
   void* fn;
   int blocks;
