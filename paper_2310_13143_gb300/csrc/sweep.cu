@@ -1388,12 +1388,16 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
         }
       }
     } else if (!kTiled) {
-      // where there are several passes, warps take runs of 32 components round
+      // where there are a few passes, warps take runs of 32 components round
       // the CTAs, so that the last, partial pass is spread over all SMs (in CTA
       // order it went to the first CTAs only, and the others waited for half a
-      // pass); one pass in CTA order pairs the CTAs that share an SM with the
-      // generators' short ones (13 x 2,000 buses: 13.3 us per iteration, 13.8)
-      const int first = d.G + d.L > nthreads
+      // pass: 1 x 70,000 buses 28.2 us per iteration, 27.0 spread).  One pass in
+      // CTA order pairs the CTAs that share an SM with the generators' short
+      // ones (13 x 2,000 buses: 13.3, spread 13.8).  Many passes hide the last
+      // one, and in CTA order a CTA's warps read neighbouring components (8 x
+      // 70,000 buses, 10 passes: 118.4, spread 119.3; 16: 215.7 and 217.5; at 256
+      // x 2,000 buses, 10 passes, the two are alike)
+      const int first = d.G + d.L > nthreads && d.G + d.L <= 8 * nthreads
                             ? (((int)threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x) * 32 + lane
                             : tid;
       for (int u = first; u < d.G + d.L; u += nthreads) {
@@ -1485,13 +1489,22 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     } else {
       // a CTA takes a contiguous run of tasks, whose warps gather from
       // neighbouring branches at the same time; the runs differ by one task.
-      // With few tasks per warp a run's remainder would cost every CTA a round
-      // of its own, so there the tasks go round all warps (64 x 2,000 buses, 5
-      // tasks per warp: 29.4 -> 27.8 us per iteration in runs), as they do when
-      // only a batch's last instances take part, whose tasks lie together and
-      // would all fall to a few CTAs (256 scenarios and 64 grids of 118-10,000
-      // buses solved to the end: 1,727 ms in runs throughout, 1,597 ms so)
-      const bool runs = mostly && d.NT >= 4 * nw;
+      // 128 x 2,000 buses: 55.5 us per iteration against 56.4 with the tasks
+      // going round all warps, 8 x 70,000: 119.3 against 121.3.  They go round
+      // all warps
+      //  - with few tasks per warp, where a run's remainder would cost every CTA
+      //    a round of its own (the line at 1, 2 or 4 tasks measures alike from 16
+      //    to 128 x 2,000 buses);
+      //  - when only a batch's last instances take part, whose tasks lie together
+      //    and would all fall to a few CTAs (256 scenarios and 64 grids of
+      //    118-10,000 buses solved to the end: 1,727 ms in runs throughout, 1,597
+      //    so; 1,617 without runs; the line at 1/2 or 9/10 measures alike);
+      //  - in large batches of large grids: runs gather from all instances at
+      //    once, which together exceed L2, and going round the warps gathers from
+      //    one (24 x 70,000 buses, 65 tasks per warp: 306.9 against 315.4; 44 x
+      //    35,000: 297.9 and 301.5; 155 x 10,000, 940 tasks per instance: 293.3
+      //    and 292.6; 512 x 2,000: 197.3 and 193.9)
+      const bool runs = mostly && d.NT >= 4 * nw && (d.NT <= 32 * nw || d.NT <= 1024 * d.K);
       const int tb = runs ? (int)((long long)d.NT * blockIdx.x / gridDim.x) : 0;
       const int te = runs ? (int)((long long)d.NT * (blockIdx.x + 1) / gridDim.x) : d.NT;
       const int wpb = runs ? (int)blockDim.x >> 5 : nw, tw = runs ? tb + ((int)threadIdx.x >> 5) : wid;

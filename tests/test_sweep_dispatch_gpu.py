@@ -79,3 +79,29 @@ def test_runs_of_bus_tasks_in_a_batch_that_thins_out():
         assert (ra["sqp_iter"], ra["admm_iter"]) == (rb["sqp_iter"], rb["admm_iter"])
         for a, b in zip(ia, ib):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("case", ["large grid", "many instances"])
+def test_many_passes_and_tasks_per_warp(case):
+    """More than eight passes over the components and more than 32 tasks per
+    warp: tasks round all warps for a large grid, in runs for many instances;
+    the same bits as with many threads."""
+    sms = _sms()
+    if case == "large grid":
+        grids = [gg.geometric_grid(60000 * sms // 152, seed=3)]
+    else:
+        grids = gg.scenarios_cholesky(gg.grid_2000bus(), 32 * sms // 152, 2)
+    tasks, work = _tasks(grids), sum(g.ngen + g.nbranch for g in grids)
+    assert work > 8 * 32 * sms and tasks > 32 * sms  # one warp per SM
+    assert (tasks > 1024 * len(grids)) == (case == "large grid")
+    out = []
+    for shape in ((32, 1, 0), (256, 0, 0)):
+        s = binding.Solver(grids, precision="mixed")
+        s.tune(*shape)
+        s.build_qp(1.0, 2e4, True)
+        s.admm_iterate(6, binding.default_admm())
+        out.append([s.get_admm_state(k) for k in range(len(grids))])
+        s.close()
+    for a, b in zip(*out):
+        for k in KEYS:
+            np.testing.assert_array_equal(a[k], b[k], err_msg=k)
