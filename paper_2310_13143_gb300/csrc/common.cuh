@@ -210,7 +210,7 @@ struct Ctx {
   // reading in place (0) where the components outnumber the threads that fit.
   // Measured per ADMM iteration, in place against resident: 30 buses 10.7
   // against 4.1 us mixed (one CTA, which needs no device-wide barrier) and
-  // 21.3 against 8.4 FP64; 2,000 buses 12.2 against 9.2 and 45 against 17;
+  // 21.3 against 8.8 FP64; 2,000 buses 12.2 against 9.2 and 45 against 17;
   // 20,000 buses 13.8 against 10.5 and 51 against 41.
   int sweep_stages = 3;
   int cluster_cs = 1;         // cluster size of sweep_stages 4, chosen for

@@ -1,10 +1,11 @@
 // The ADMM sweep of Algorithm 2 fused into one persistent cooperative kernel.
 //
 // Iteration t:
-//   phase A  one thread per generator (eq. gen_kernel, closed form) and per
-//            branch (eq. line_kernel: 4-variable QP with box, line-limit and
-//            angle rows, solved by an augmented Lagrangian whose subproblems
-//            are solved by projected Newton -- Sec. IV-B);
+//   phase A  one thread per generator (eq. gen_kernel, closed form) and one
+//            or four per branch (eq. line_kernel: 4-variable QP with box,
+//            line-limit and angle rows; in FP32, and with line_solver 1, by an
+//            augmented Lagrangian whose subproblems are solved by projected
+//            Newton -- Sec. IV-B --, else exactly);
 //   barrier
 //   phase B  one lane per generator or branch end, one warp per task of
 //            consecutive buses (eq. bus_kernel, closed form from the 2x2
@@ -417,7 +418,7 @@ __device__ __forceinline__ void line_compute_to(const SweepP<T>& p, int l, const
 // flow q and row q of the constraints, the vectors pass between the lanes by
 // shuffles, and a matrix product costs four FP64 instructions instead of
 // sixteen -- about 50 on the usual path against 150.  Full FP64 solves: 2,000
-// buses 135 -> 101 ms, 30 buses 331 -> 223 ms against one lane per branch (and 244
+// buses 135 -> 103 ms, 30 buses 331 -> 217 ms against one lane per branch (and 244
 // and 638 ms with a factorisation per iteration).
 //
 // What few iterations need -- a new operator, the general solves -- is called
