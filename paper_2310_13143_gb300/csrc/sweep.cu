@@ -578,8 +578,9 @@ __device__ __forceinline__ double quad_dot(const double* a, double v, double s) 
 
 // The line update of the warp's eight branches.  All 32 lanes call it; quads
 // without a branch (is = false) go along on zeros.  op: the quad's column of
-// operators in shared memory.
-__device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const Dev& d, bool is, int l, QuadRec& a,
+// operators in shared memory.  Returns whether this lane's branch is left to
+// the general solves (quads_general).
+__device__ __forceinline__ bool line_compute_quad(const SweepP<double>& p, const Dev& d, bool is, int l, QuadRec& a,
                                                   double* op, int stride) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, q = lane & 3, qb = lane & ~3;
@@ -675,13 +676,6 @@ __device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const
     }
     if (!__any_sync(FULL, is && !general && !(a.set & kSetValid))) break;  // nothing is left to correct
   }
-  if (__any_sync(FULL, is && general)) {
-    unsigned s = a.set;
-    if (is && general && q == 0)
-      s = line_general_slow(d, l, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
-    s = __shfl_sync(FULL, s, 0, 4);
-    if (general) a.set = s;
-  }
   const double xf = quad_dot(a.Fr, x, a.f0);
   if (is && !general) {
     double* X = (double*)d.X + at;
@@ -689,6 +683,32 @@ __device__ __forceinline__ void line_compute_quad(const SweepP<double>& p, const
     X[2] = x;
     ((double*)d.U)[4 * (size_t)l + q] = ((a.set >> (8 + q)) & 1u) && pos_w(mu) ? mu : 0.0;
   }
+  return is && general;
+}
+
+// The branches that a CTA's quads leave to the general solves (general: this
+// lane's), one thread each, so that 32 of them share a warp: an instruction
+// costs a warp's FP64 pipe the same with one lane at work or 32, and eight per
+// warp, each on its quad's first lane, took a 300-bus grid whose lines are all
+// infeasible 1,439 us per iteration, this 962 (30 buses 1,110 and 925; where no
+// line is infeasible, no difference).  l0: the CTA's first branch.  All threads
+// of the CTA call it.
+struct QuadList {
+  int n;
+  unsigned quad[64], set[64];  // 256 threads
+};
+__device__ __forceinline__ void quads_general(const SweepP<double>& p, const Dev& d, bool general, int l0, QuadList& s,
+                                              unsigned& set) {
+  const int t = threadIdx.x;
+  if (general && (t & 3) == 0) s.quad[atomicAdd(&s.n, 1)] = t >> 2;
+  if (!__syncthreads_or(general)) return;
+  if (t < s.n) {
+    const unsigned k = s.quad[t];
+    s.set[k] = line_general_slow(d, l0 + (int)k, p.beta_scale, p.alm_tol, p.alm_outer, p.newton_max);
+  }
+  __syncthreads();
+  if (general) set = s.set[t >> 2];
+  if (t == 0) s.n = 0;  // written again after the next barrier
 }
 
 // line update of branch l reading its record from global memory (rs, stride L)
@@ -1307,6 +1327,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
     mbar_init(&tbar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __shared__ QuadList s_quads;  // RES 4
+  if (RES == 4 && threadIdx.x == 0) s_quads.n = 0;
   int live = 0;  // whether an instance of this thread's takes part
   for (int k = threadIdx.x; k < K; k += blockDim.x) {
     s_done[k] = d.admm_done[k];
@@ -1372,7 +1394,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && !RES) ? 2 : 1) k_sweep
       const V4<T>* LM = (const V4<T>*)d.LAM;
       if constexpr (RES == 4) {
         if (go && is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
-        line_compute_quad(p, d, go && is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
+        const bool left = line_compute_quad(p, d, go && is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
+        quads_general(p, d, left, (int)(blockIdx.x * blockDim.x >> 2), s_quads, qr.set);
       } else if (go) {
         if constexpr (sizeof(T) == 8) {
           if (is_gen)
@@ -1685,6 +1708,8 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(const __grid_constant_
   typedef ClusterRes<T> Res;
   __shared__ __align__(16) typename Res::Word s_res[2][2];  // this CTA's maxima (r, s), by iteration parity
   double last_r = 0.0, last_s = 0.0;                        // of the last iteration, over the cluster
+  __shared__ QuadList s_quads;  // RES 4
+  if (RES == 4 && threadIdx.x == 0) s_quads.n = 0;
   if (threadIdx.x < 4) (&s_res[0][0])[threadIdx.x] = 0;
   if (d.admm_done[k]) return;  // the whole cluster skips an instance that is not running
   cluster_barrier();  // every CTA has started before any distributed shared memory access
@@ -1741,7 +1766,8 @@ __global__ void __launch_bounds__(256, 1) k_sweep_cluster(const __grid_constant_
       const V4<T>* LM = (const V4<T>*)d.LAM;
       if constexpr (RES == 4) {
         if (is_gen) gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
-        line_compute_quad(p, d, is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
+        const bool left = line_compute_quad(p, d, is_br, br, qr, s_op + (threadIdx.x >> 2), blockDim.x >> 2);
+        quads_general(p, d, left, l0 + (int)(rank * blockDim.x >> 2), s_quads, qr.set);
       } else if constexpr (sizeof(T) == 8) {
         if (is_gen)
           gen_compute_kept(d, gen, rr[0], rr[1], rr[2]);
