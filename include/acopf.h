@@ -20,7 +20,8 @@
  *  - Pointers marked "host" are read (or written) during the call only; the
  *    caller keeps ownership.  Device memory is owned by the handle.
  *  - Calls are asynchronous on the handle's stream except the acopf_get_*
- *    functions, which synchronise that stream before they return.
+ *    functions and the setters of an iterate, a warm start or an ADMM state
+ *    from host arrays, which synchronise that stream before they return.
  *  - A handle is not thread-safe; calls on different handles are independent.
  *  - No CPU fallback: without a usable CUDA device acopf_create fails with
  *    ACOPF_ECUDA.

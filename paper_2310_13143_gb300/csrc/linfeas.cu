@@ -36,7 +36,7 @@
 //   - The residuals are formed only in the iterations whose residuals are read.
 //   - Each window of 1,024 buses is processed in order of degree, so that the
 //     lanes of a warp loop equally often.
-// 128 scenarios of the 2,000-bus grid (345,600 branches): 469 -> 82 us per iteration, 504 -> 101 ms per call.
+// 128 scenarios of the 2,000-bus grid (345,600 branches): 469 -> 82 us per iteration, 504 -> 92 ms per call.
 #include <math.h>
 #include <stdint.h>
 
